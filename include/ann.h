@@ -261,10 +261,14 @@ ann_status ann_shards_search(ann_shards *shards, const float *queries, uint32_t 
 /* Exact kNN lists: ids (device, n x K) gets, for every node u of X (device,
  * n x dim FP32 row-major), the K other nodes nearest to u by squared L2 in
  * FP32 (one fused multiply-add per element, index order), ordered by
- * (distance, id). Brute force: O(n^2 dim) work, for building graphs of up to
- * a few million nodes. 2 <= n < 2^32 - 1, 1 <= K < n, K <= 2 ANN_MAX_DEGREE,
+ * (distance, id). All pairs are compared (O(n^2 dim) work on the tensor
+ * cores, by distances with a proven error bound; those that could be among
+ * the K nearest are computed exactly), for building graphs of up to a few
+ * million nodes. 2 <= n < 2^32 - 1, 1 <= K < n, K <= 2 ANN_MAX_DEGREE,
  * and (96 rows x (dim + 1) + 32 K x 2) x 4 bytes of shared memory must fit a
- * block (ANN_EINVAL otherwise). Asynchronous on `stream`. */
+ * block (ANN_EINVAL otherwise). Asynchronous on `stream`; from 1,024 nodes on
+ * it takes a temporary in stream order (2 n dim bytes and at most about 20 KB
+ * per row of a chunk of 39,000 rows) and does without if it cannot have it. */
 ann_status ann_knn_exact(const float *X, uint64_t n, uint32_t dim, uint32_t K, uint32_t *ids, void *stream);
 /* Prune kNN lists (device, n x K; each row distinct ids, ANN_INVALID_ID
  * allowed) to a fixed-degree graph (device, n x degree): edge u -> v at rank

@@ -1,12 +1,7 @@
-// Graph construction on the GPU (the build the paper times in Section 5.7,
-// Fig. 16; the graph itself is an input of the search, Section 2.1):
+// Graph pruning on the GPU (the build the paper times in Section 5.7,
+// Fig. 16; the graph itself is an input of the search, Section 2.1;
+// the kNN lists are knn.cu's):
 //
-//   ann_knn_exact   the K nearest other nodes of every node, by brute force:
-//                   a block keeps 32 query rows and streams the candidates
-//                   through shared memory in tiles of 64 rows; a warp owns 4
-//                   queries and keeps each one's sorted (distance, id) list
-//                   in shared memory, inserting the few tile candidates that
-//                   beat its current K-th entry;
 //   ann_graph_prune the detour-count pruning with reverse edges: one warp per
 //                   node counts detours with a sorted (id, rank) table of its
 //                   list in shared memory and orders the list by (detours,
@@ -15,9 +10,6 @@
 //                   smallest (position, source) offers; one warp per node
 //                   assembles the row (kept, reverse, rest; repeats and the
 //                   node itself dropped).
-//
-// Distances are squared L2 in FP32, one fused multiply-add per element in
-// index order (the kNN lists rank by (distance, id)).
 #include <algorithm>
 #include <vector>
 
@@ -26,115 +18,6 @@
 using namespace ann;
 
 namespace {
-
-constexpr int KQ = 32;          // query rows per block
-constexpr int KC = 64;          // candidate rows per shared-memory tile
-constexpr int KW = 8;           // warps per block (4 queries each)
-
-__device__ __forceinline__ bool kless(float da, uint32_t ia, float db, uint32_t ib)
-{
-    return da < db || (da == db && ia < ib);
-}
-
-// Insert (d, id) into a warp's sorted list lst_d/lst_i of K entries if it
-// beats the last one (all lanes call it with the same arguments).
-__device__ __forceinline__ void list_insert(float *lst_d, uint32_t *lst_i, uint32_t K, float d, uint32_t id,
-                                            uint32_t lane)
-{
-    if (!kless(d, id, lst_d[K - 1], lst_i[K - 1])) return;
-    uint32_t pos = 0;
-    for (uint32_t j = lane; j < K; j += 32) pos += kless(lst_d[j], lst_i[j], d, id) ? 1u : 0u;
-    pos = __reduce_add_sync(0xffffffffu, pos);
-    // shift [pos, K - 1) right by one, from the top (each lane one entry
-    // per pass, read before any write of the pass)
-    for (int32_t top = (int32_t)K - 2; top >= (int32_t)pos; top -= 32) {
-        const int32_t j = top - (int32_t)lane;
-        float vd = 0.0f;
-        uint32_t vi = 0;
-        const bool mine = j >= (int32_t)pos;
-        if (mine) { vd = lst_d[j]; vi = lst_i[j]; }
-        __syncwarp();
-        if (mine) { lst_d[j + 1] = vd; lst_i[j + 1] = vi; }
-        __syncwarp();
-    }
-    if (lane == 0) { lst_d[pos] = d; lst_i[pos] = id; }
-    __syncwarp();
-}
-
-// Exact kNN: block b handles query rows [32 b, 32 b + 32); dynamic shared
-// memory holds the 32 query rows, one tile of KC candidate rows (row stride
-// d + 1 floats: lanes reading one element of 32 different rows hit 32
-// banks) and the 32 lists of K entries.
-__global__ void __launch_bounds__(KW * 32) knn_exact_kernel(const float *__restrict__ X, uint32_t n, uint32_t d,
-                                                            uint32_t K, uint32_t *__restrict__ out)
-{
-    extern __shared__ __align__(16) uint8_t sm[];
-    const uint32_t ds = d + 1;
-    float *sq = reinterpret_cast<float *>(sm);                 // KQ x ds
-    float *sc = sq + KQ * ds;                                  // KC x ds
-    float *ld = sc + KC * ds;                                  // KQ x K
-    uint32_t *li = reinterpret_cast<uint32_t *>(ld + KQ * K);  // KQ x K
-    const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const uint32_t q0 = blockIdx.x * KQ;
-    for (uint32_t i = threadIdx.x; i < KQ * d; i += blockDim.x) {
-        const uint32_t r = i / d, c = i % d;
-        sq[r * ds + c] = q0 + r < n ? X[(size_t)(q0 + r) * d + c] : 0.0f;
-    }
-    for (uint32_t i = threadIdx.x; i < KQ * K; i += blockDim.x) {
-        ld[i] = INFINITY;
-        li[i] = ANN_INVALID_ID;
-    }
-    for (uint32_t c0 = 0; c0 < n; c0 += KC) {
-        __syncthreads();
-        for (uint32_t i = threadIdx.x; i < KC * d; i += blockDim.x) {
-            const uint32_t r = i / d, c = i % d;
-            sc[r * ds + c] = c0 + r < n ? X[(size_t)(c0 + r) * d + c] : 0.0f;
-        }
-        __syncthreads();
-        // this warp's 4 queries x the tile's 64 candidates: lane owns
-        // candidates lane and lane + 32
-        float acc[4][2];
-#pragma unroll
-        for (int a = 0; a < 4; ++a) acc[a][0] = acc[a][1] = 0.0f;
-        const float *x0 = sc + lane * ds, *x1 = sc + (lane + 32) * ds;
-        const float *qw = sq + (warp * 4) * ds;
-#pragma unroll 2
-        for (uint32_t i = 0; i < d; ++i) {
-            const float xa = x0[i], xb = x1[i];
-#pragma unroll
-            for (int a = 0; a < 4; ++a) {
-                const float qv = qw[a * ds + i];
-                const float da = __fsub_rn(qv, xa), db = __fsub_rn(qv, xb);
-                acc[a][0] = __fmaf_rn(da, da, acc[a][0]);
-                acc[a][1] = __fmaf_rn(db, db, acc[a][1]);
-            }
-        }
-#pragma unroll
-        for (int a = 0; a < 4; ++a) {
-            const uint32_t qi = q0 + warp * 4 + a;
-            float *lda = ld + (warp * 4 + a) * K;
-            uint32_t *lia = li + (warp * 4 + a) * K;
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const uint32_t cid = c0 + lane + 32 * h;
-                const bool cand = qi < n && cid < n && cid != qi;
-                const float dv = acc[a][h];
-                uint32_t m = __ballot_sync(0xffffffffu, cand && kless(dv, cid, lda[K - 1], lia[K - 1]));
-                while (m) {
-                    const uint32_t src = __ffs(m) - 1;
-                    m &= m - 1;
-                    list_insert(lda, lia, K, __shfl_sync(0xffffffffu, dv, src),
-                                __shfl_sync(0xffffffffu, cid, src), lane);
-                }
-            }
-        }
-    }
-    __syncthreads();
-    for (uint32_t i = threadIdx.x; i < KQ * K; i += blockDim.x) {
-        const uint32_t r = i / K;
-        if (q0 + r < n) out[(size_t)(q0 + r) * K + (i % K)] = li[i];
-    }
-}
 
 // ------------------------------------------------------------ pruning
 // Detour counts and the (detours, rank) order of node u's list: warp per
@@ -329,28 +212,6 @@ int grid_for(uint64_t n, int threads) { return (int)std::max<uint64_t>(1, (n + t
 }  // namespace
 
 extern "C" {
-
-ann_status ann_knn_exact(const float *X, uint64_t n, uint32_t dim, uint32_t K, uint32_t *ids, void *stream)
-{
-    if (!X || !ids || n < 2 || n > 0xFFFFFFFEull || dim == 0 || dim > ANN_MAX_DIM || K == 0 || K >= n ||
-        K > 2 * ANN_MAX_DEGREE) {
-        set_error("ann_knn_exact: need 2 <= n < 2^32 - 1, 1 <= dim <= %u, 1 <= K < n, K <= %u", ANN_MAX_DIM,
-                  2 * ANN_MAX_DEGREE);
-        return ANN_EINVAL;
-    }
-    const size_t smem = (size_t)(KQ + KC) * (dim + 1) * 4 + (size_t)KQ * K * 8;
-    int dev = 0, optin = 0;
-    ANN_CUDA(cudaGetDevice(&dev));
-    ANN_CUDA(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
-    if (smem > (size_t)optin) {
-        set_error("ann_knn_exact: %zu bytes of shared memory needed (dim %u, K %u), %d available", smem, dim, K, optin);
-        return ANN_EINVAL;
-    }
-    ANN_CUDA(cudaFuncSetAttribute(knn_exact_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    knn_exact_kernel<<<grid_for(n, KQ), KW * 32, smem, (cudaStream_t)stream>>>(X, (uint32_t)n, dim, K, ids);
-    ANN_CUDA(cudaGetLastError());
-    return ANN_OK;
-}
 
 ann_status ann_graph_prune(const uint32_t *knn, uint64_t n, uint32_t K, uint32_t degree, uint32_t *graph,
                            void *stream)

@@ -16,8 +16,6 @@
 //     inference never writes the (queries x ghosts) logits.
 // Every mbarrier wait is bounded; on expiry the kernel records a timeout in
 // the error word, frees its tensor memory and returns.
-#include <cuda.h>
-#include <cudaTypedefs.h>
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -27,7 +25,7 @@
 #include <cstring>
 #include <vector>
 
-#include "ann_internal.cuh"
+#include "tcgen05.cuh"
 
 using namespace ann;
 
@@ -66,82 +64,6 @@ struct EpiArgs {
     int *err;
 };
 
-// ------------------------------------------------------------------ PTX
-__device__ __forceinline__ void tma_load_2d(void *dst, const CUtensorMap *map, int x, int y, uint64_t *bar)
-{
-    asm volatile(
-        "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], "
-        "[%4];" ::"r"(smem_addr(dst)),
-        "l"(map), "r"(x), "r"(y), "r"(smem_addr(bar))
-        : "memory");
-}
-
-__device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
-
-// Shared-memory matrix descriptor, K-major operand in the 128-byte swizzle
-// layout TMA writes: rows of 128 bytes, 8-row groups 1024 bytes apart.
-__device__ __forceinline__ uint64_t desc_sw128(uint32_t saddr)
-{
-    uint64_t d = 0;
-    d |= (uint64_t)((saddr & 0x3FFFFu) >> 4);        // start address
-    d |= (uint64_t)1 << 16;                           // leading byte offset (unused in this layout)
-    d |= (uint64_t)(1024 >> 4) << 32;                 // stride byte offset: next 8-row group
-    d |= (uint64_t)1 << 46;                           // descriptor version of this architecture
-    d |= (uint64_t)2 << 61;                           // swizzle: 128 bytes
-    return d;
-}
-
-// Instruction descriptor: BF16 x BF16 -> FP32, both K-major, M 128, N BN.
-__host__ __device__ constexpr uint32_t idesc_bf16(uint32_t m, uint32_t n)
-{
-    return (1u << 4) | (1u << 7) | (1u << 10) | ((n >> 3) << 17) | ((m >> 4) << 24);
-}
-
-__device__ __forceinline__ void mma_bf16(uint32_t tmem_d, uint64_t da, uint64_t db, uint32_t idesc, uint32_t acc)
-{
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem_d),
-        "l"(da), "l"(db), "r"(idesc), "r"(acc)
-        : "memory");
-}
-
-__device__ __forceinline__ void mma_commit(uint64_t *bar)
-{
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_addr(bar))
-                 : "memory");
-}
-
-// Two 32-column accumulator loads in flight together and one wait: the
-// second statement waits for both and names the first load's registers as
-// its operands, so no use of them can move above the wait.
-__device__ __forceinline__ void tmem_ld32x2(uint32_t taddr0, uint32_t taddr1, float (&v0)[32], float (&v1)[32])
-{
-    uint32_t r[32], s[32];
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, "
-        "%15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
-          "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
-          "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-        : "r"(taddr0));
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, "
-        "%15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%64];\n\t"
-        "tcgen05.wait::ld.sync.aligned;"
-        : "=r"(s[0]), "=r"(s[1]), "=r"(s[2]), "=r"(s[3]), "=r"(s[4]), "=r"(s[5]), "=r"(s[6]), "=r"(s[7]), "=r"(s[8]), "=r"(s[9]), "=r"(s[10]), "=r"(s[11]), "=r"(s[12]), "=r"(s[13]), "=r"(s[14]), "=r"(s[15]), "=r"(s[16]), "=r"(s[17]), "=r"(s[18]), "=r"(s[19]), "=r"(s[20]), "=r"(s[21]), "=r"(s[22]), "=r"(s[23]), "=r"(s[24]), "=r"(s[25]), "=r"(s[26]), "=r"(s[27]), "=r"(s[28]), "=r"(s[29]), "=r"(s[30]), "=r"(s[31]),
-          "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]), "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15]), "+r"(r[16]), "+r"(r[17]), "+r"(r[18]), "+r"(r[19]), "+r"(r[20]), "+r"(r[21]), "+r"(r[22]), "+r"(r[23]), "+r"(r[24]), "+r"(r[25]), "+r"(r[26]), "+r"(r[27]), "+r"(r[28]), "+r"(r[29]), "+r"(r[30]), "+r"(r[31])
-        : "r"(taddr1)
-        : "memory");
-#pragma unroll
-    for (int i = 0; i < 32; ++i) {
-        v0[i] = __uint_as_float(r[i]);
-        v1[i] = __uint_as_float(s[i]);
-    }
-}
-
 // Cluster helpers (the multicast logits kernel runs in clusters of two CTAs).
 __device__ __forceinline__ uint32_t cluster_rank()
 {
@@ -175,11 +97,6 @@ __device__ __forceinline__ void mma_commit_mc(uint64_t *bar, uint16_t mask)
             smem_addr(bar)),
         "h"(mask)
         : "memory");
-}
-
-__device__ __forceinline__ void mbar_arrive(uint64_t *bar)
-{
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(bar)) : "memory");
 }
 
 // 2^x by the hardware approximation (MUFU): the softmax sum only decides the
@@ -564,7 +481,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
                     const uint32_t a0 = smem_addr(sA + kb * TILE_A), b0 = smem_addr(sB + s * TILE_B);
 #pragma unroll
                     for (uint32_t k = 0; k < BK / 16; ++k)
-                        mma_bf16(acc, desc_sw128(a0 + k * 32), desc_sw128(b0 + k * 32), idesc, (kb | k) != 0);
+                        mma_f16kind(acc, desc_sw128(a0 + k * 32), desc_sw128(b0 + k * 32), idesc, (kb | k) != 0);
                     if (MC) mma_commit_mc(&empty[s], (uint16_t)3);   // frees the stage in both CTAs
                     else mma_commit(&empty[s]);
                 }
@@ -591,7 +508,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
                     const uint32_t a0 = smem_addr(sA + s * TILE_A), b0 = smem_addr(sB + s * TILE_B);
 #pragma unroll
                     for (uint32_t k = 0; k < BK / 16; ++k)
-                        mma_bf16(acc, desc_sw128(a0 + k * 32), desc_sw128(b0 + k * 32), idesc, (kb | k) != 0);
+                        mma_f16kind(acc, desc_sw128(a0 + k * 32), desc_sw128(b0 + k * 32), idesc, (kb | k) != 0);
                     mma_commit(&empty[s]);
                 }
                 mma_commit(&acc_full[buf]);
@@ -1022,40 +939,12 @@ struct ann_mlp {
 
 namespace {
 
-PFN_cuTensorMapEncodeTiled_v12000 g_encode = nullptr;
-
-ann_status get_encoder()
-{
-    if (g_encode) return ANN_OK;
-    void *fn = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    cudaError_t e = cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &q);
-    if (e != cudaSuccess || q != cudaDriverEntryPointSuccess || !fn) {
-        set_error("cuTensorMapEncodeTiled is not available from the driver");
-        return ANN_ECUDA;
-    }
-    g_encode = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(fn);
-    return ANN_OK;
-}
-
 // Tensor map of a row-major BF16 matrix (rows x K, row stride K elements),
 // box BK x box_rows, 128-byte swizzle; out-of-range elements read as zero.
 ann_status make_map(CUtensorMap *map, const void *ptr, uint32_t rows, uint32_t K, uint32_t box_rows = 128)
 {
-    ann_status s = get_encoder();
-    if (s != ANN_OK) return s;
-    const cuuint64_t dims[2] = {K, rows};
-    const cuuint64_t strides[1] = {(cuuint64_t)K * 2};
-    const cuuint32_t box[2] = {BK, box_rows};
-    const cuuint32_t estr[2] = {1, 1};
-    CUresult r = g_encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void *>(ptr), dims, strides, box, estr,
-                          CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                          CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    if (r != CUDA_SUCCESS) {
-        set_error("cuTensorMapEncodeTiled failed (%d) for %u x %u", (int)r, rows, K);
-        return ANN_ECUDA;
-    }
-    return ANN_OK;
+    static_assert(BK == 64, "a tensor-map box is 64 elements wide");
+    return make_map16(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, ptr, rows, K, K, box_rows);
 }
 
 // Which GEMM variant runs: the fused top-P logits with K <= RES_K keep A
