@@ -52,15 +52,12 @@
 #include <cstdlib>
 #include <vector>
 
-#include "ann_internal.cuh"
+#include "search_common.cuh"
 
 using namespace ann;
 
 namespace {
 
-constexpr uint32_t kUnexpanded = 0, kPartial = 1, kExpanded = 2;
-constexpr uint64_t kGhostTag = 0x67686F7374ull;
-constexpr uint32_t kEmpty = 0xFFFFFFFFu;
 constexpr uint32_t kMaxDegWords = ANN_MAX_DEGREE / 32;
 // Resident 4-warp blocks per SM the register allocation is sized for.
 #ifndef ANN_SEARCH_BLOCKS_PER_SM
@@ -68,34 +65,9 @@ constexpr uint32_t kMaxDegWords = ANN_MAX_DEGREE / 32;
 #endif
 constexpr int kSearchBlocksPerSm = ANN_SEARCH_BLOCKS_PER_SM;
 
-// Entries that run the ghost stage first.
-__host__ __device__ __forceinline__ bool ghost_entry(uint32_t e)
-{
-    return e == ANN_ENTRY_GHOST || e == ANN_ENTRY_GIVEN_GHOST;
-}
-// Entries that read a row of caller-given seeds.
-__host__ __device__ __forceinline__ bool given_entry(uint32_t e)
-{
-    return e == ANN_ENTRY_GIVEN_GHOST || e == ANN_ENTRY_GIVEN_BASE;
-}
-
-struct View {
-    const uint8_t *codes;
-    const float *scales;   // nullptr for FP32
-    uint32_t row_bytes;
-    const uint32_t *graph;
-    uint32_t deg, deg_pad;
-    const uint32_t *dir;   // nullptr: no DGS on this graph
-    uint32_t n;
-};
-
 struct Layout {  // byte offsets inside one warp's shared-memory region
     uint32_t q, bd, bi, bs, cd, ci, cs, adj, dir, prow, par, stage, bar, qp, total;
 };
-
-// Ghost sets up to this many nodes get an exact shared-memory bitmap as the
-// ghost stage's visited set (2 KB per warp at most).
-constexpr uint32_t kGhostBitmapMax = 16384;
 
 struct Args {
     View base, ghost;
@@ -131,64 +103,6 @@ struct Args {
 enum Phase : uint32_t { PH_SELECT = 0, PH_DGS, PH_VISIT, PH_GATHER, PH_DIST, PH_MERGE, PH_OTHER };
 enum ProfStage : uint32_t { PS_GHOST = 0, PS_BASE, PS_FINISH };
 static_assert(PH_OTHER < ANN_PROFILE_PHASES && PS_FINISH < ANN_PROFILE_STAGES, "profile table too small");
-
-__device__ __forceinline__ uint64_t splitmix64(uint64_t x)
-{
-    uint64_t z = x + 0x9E3779B97F4A7C15ull;
-    z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
-    z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
-    return z ^ (z >> 31);
-}
-
-// (da, ia) < (db, ib) in (distance, id) order. Distances are squared L2,
-// never negative nor NaN, and non-negative floats order as their bit
-// patterns do, so the key compares as one 64-bit integer (bits, id): two
-// integer compares instead of three float and integer ones.
-__device__ __forceinline__ bool key_less(float da, uint32_t ia, float db, uint32_t ib)
-{
-    return (((uint64_t)__float_as_uint(da) << 32) | ia) < (((uint64_t)__float_as_uint(db) << 32) | ib);
-}
-
-__device__ __forceinline__ uint32_t lanemask_lt()
-{
-    uint32_t m;
-    asm("mov.u32 %0, %%lanemask_lt;" : "=r"(m));
-    return m;
-}
-
-// One element: df = q - x, acc += df * df with a single rounding.
-__device__ __forceinline__ void step(float qv, float xv, float &acc)
-{
-    const float df = __fsub_rn(qv, xv);
-    acc = __fmaf_rn(df, df, acc);
-}
-
-// Stored value of element i (decoded to FP32).
-template <int ST>
-__device__ __forceinline__ float stored_elem(const uint8_t *row, uint32_t i, float scale)
-{
-    if (ST == ANN_F32) return reinterpret_cast<const float *>(row)[i];
-    if (ST == ANN_F16) return __fmul_rn(scale, __half2float(reinterpret_cast<const __half *>(row)[i]));
-    const __half_raw h = __nv_cvt_fp8_to_halfraw((__nv_fp8_storage_t)row[i], __NV_E4M3);
-    return __fmul_rn(scale, __half2float(__half(h)));
-}
-
-// One element of the distance: acc += (q - stored)^2, the difference
-// rounded once. An FP16 row's scale is a power of two, so its stored value
-// s * h is exact in FP32 (for every row whose largest |x| is at least 2^-88,
-// where s * h stays a normal number) and q - s * h is one fused multiply-add,
-// equal to the rounded difference of q and the stored value; E4M3 scales are
-// not powers of two, so that stored value is rounded first.
-template <int ST>
-__device__ __forceinline__ void elem_step(float qv, const uint8_t *row, uint32_t i, float scale, float &acc)
-{
-    if (ST == ANN_F16) {
-        const float df = __fmaf_rn(-scale, __half2float(reinterpret_cast<const __half *>(row)[i]), qv);
-        acc = __fmaf_rn(df, df, acc);
-    } else {
-        step(qv, stored_elem<ST>(row, i, scale), acc);
-    }
-}
 
 // rn(y - x) and rn(acc + df * df) for two elements at once with the packed
 // FP32 pipe: fma(x, -1, y) rounds y - x once, so both results equal the
@@ -256,21 +170,6 @@ __device__ __forceinline__ float row_dist_half(const uint8_t *row, const float *
         if (i + 2 * h + 1 < d) elem_step<ST>(q[i + 2 * h + 1], row, i + 2 * h + 1, scale, s.y);
     }
     return __fadd_rn(s.x, s.y);
-}
-
-// One of the four partial sums of the squared L2 between a staged row and
-// the query: lane j of a row's four lanes runs sum j (elements i = j, j + 4,
-// ... in index order, one fused multiply-add each), so the four lanes
-// together do the work of one row with the same operations as the
-// definition. Used for wide rows, where a round stages at most 8 rows.
-template <int ST>
-__device__ __forceinline__ float row_dist_quarter(const uint8_t *row, const float *q, float scale, uint32_t d,
-                                                  uint32_t j)
-{
-    float s = 0.0f;
-#pragma unroll 4
-    for (uint32_t i = j; i < d; i += 4) elem_step<ST>(q[i], row, i, scale, s);
-    return s;
 }
 
 template <int ST, bool PROF = false, int LPR = 2>
@@ -1394,13 +1293,29 @@ ann_status search_launch_ex(ann_index *ix, const float *queries, uint32_t nq, co
     a.counter = counter;
     a.err = err;
     a.prof = prof;
+    // one search of this index at a time: its visited tables (and work
+    // counter) are shared, so a launch on another stream waits for the last
+    if (ix->busy_set && ix->busy_stream != stream) ANN_CUDA(cudaStreamWaitEvent(stream, ix->busy, 0));
+    // a batch small enough that each query can have a block of its own goes to
+    // the teams (search_team.cu); the profile and a fixed ANN_STAGE_ROWS are
+    // the warp kernel's
+    if (!prof && env_int("ANN_STAGE_ROWS", 0) <= 0) {
+        const TeamSearch t{a.base, a.ghost, a.ghost_ids, a.x32, a.row32_bytes, a.d, a.w, std::max(q.L, ghost_entry(q.entry) ? q.Lg : 1u),
+                           a.cap_cand, a.gbm_words, q.n_keep < ix->degree || q.min_match > 0, q, queries, nq, given,
+                           ids, dists, stats, err, ix->storage, ix->num_sms, ix->smem_optin};
+        cudaError_t te = cudaSuccess;
+        if (team_search(t, stream, &te)) {
+            if (te != cudaSuccess) return cuda_fail(te, "team_kernel launch");
+            ANN_CUDA(cudaEventRecord(ix->busy, stream));
+            ix->busy_stream = stream;
+            ix->busy_set = true;
+            return ANN_OK;
+        }
+    }
     const uint64_t want = ((uint64_t)nq + warps - 1) / warps;
     // every resident warp needs its own visited table
     const uint64_t cap = std::min<uint64_t>((uint64_t)nb * ix->num_sms, ix->visited.slots / (uint32_t)warps);
     const int blocks = (int)std::min<uint64_t>(want, cap);
-    // one search of this index at a time: its visited tables (and work
-    // counter) are shared, so a launch on another stream waits for the last
-    if (ix->busy_set && ix->busy_stream != stream) ANN_CUDA(cudaStreamWaitEvent(stream, ix->busy, 0));
     ANN_CUDA(cudaMemsetAsync(counter, 0, sizeof(uint32_t), stream));
     cudaError_t e;
     if (prof) {
