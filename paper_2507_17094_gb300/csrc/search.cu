@@ -5,24 +5,27 @@
 //   - persistent CTAs of 4 warps; each warp owns one query at a time and pulls
 //     the next query index from a device counter, so long and short searches
 //     balance across the 152 SMs;
-//   - per warp, a small shared-memory region (about 9.5 KB for itopk 32 on
-//     96-d FP32) holds the query, the priority queue, the candidate list, the
-//     parents' adjacency / direction / vector rows and 16 staged rows, so 24
-//     warps share an SM and hide each other's memory latency;
+//   - per warp, a small shared-memory region (about 8 KB for itopk 32 on
+//     96-d FP32) holds the query, the priority queue, the candidate list and
+//     16 staged rows, so 24 warps share an SM and hide each other's memory
+//     latency;
 //   - the visited set of each warp is a 4,096-entry table in global memory
 //     (L2-resident, 16 KB per warp), probed with one atomicCAS per lane; the
 //     ghost stage of a small ghost set uses an exact shared-memory bitmap;
-//   - every random global read (adjacency rows, direction rows, vector rows,
-//     FP32 rerank rows) is a 1-D TMA bulk copy into shared memory completing
-//     on the warp's mbarrier: one instruction per row, all rows of a round in
-//     flight together;
+//   - the parents' lists, direction rows and own rows, a few words a lane, are
+//     read straight into registers (staged in shared memory by bulk copies they
+//     cost resident warps, copy instructions and bank conflicts: 10,000
+//     queries of FP32 96-d 1,273 -> 1,117 us, FP16 128-d with 100 results 5,134
+//     -> 3,741, 3,001 of FP16 768-d 3,430 -> 2,353);
+//   - the rows whose distances are needed (and the FP32 rerank rows) are 1-D
+//     TMA bulk copies into shared memory completing on the warp's mbarrier: one
+//     instruction per row, all rows of a round in flight together;
 //   - distances are computed by a lane pair per row from shared memory, one
 //     fused multiply-add per element into four interleaved partial sums, the
 //     same FP32 operations as the reference definition, so they agree bit
 //     for bit;
 //   - DGS needs the query's sign bits relative to each parent; they are
-//     recomputed from the parent's row, which arrives in the same bulk-copy
-//     round as its adjacency and direction rows (one ballot per 32 dims);
+//     recomputed from the parent's row (one ballot per 32 dims);
 //   - DGS keeps its top n neighbours by a ballot radix select of the score
 //     threshold, not by sorting;
 //   - the merge works in place: candidates no better than the queue's last
@@ -66,11 +69,11 @@ constexpr uint32_t kMaxDegWords = ANN_MAX_DEGREE / 32;
 constexpr int kSearchBlocksPerSm = ANN_SEARCH_BLOCKS_PER_SM;
 
 struct Layout {  // byte offsets inside one warp's shared-memory region
-    uint32_t q, bd, bi, bs, cd, ci, cs, adj, dir, prow, par, stage, bar, qp, total;
+    uint32_t q, bd, bi, bs, cd, ci, cs, gbm, stage, bar, qp, total;
 };
 
 struct Args {
-    View base, ghost;
+    View view[2];   // the ghost graph, the base graph (by stage)
     const uint32_t *ghost_ids;
     const uint8_t *x32;
     uint32_t row32_bytes;
@@ -84,7 +87,7 @@ struct Args {
     uint32_t *counter;
     int *err;
     Layout lay;
-    uint32_t cap_cand, stage_rows, stage_stride, prow_bytes;
+    uint32_t cap_buf, cap_cand, stage_rows, stage_stride;
     // the rerank's FP32 rows in the same staging area: rows per round, stride
     uint32_t rr_rows, rr_stride;
     // visited tables: slot_base + warp slot selects one table of 2^vbits
@@ -214,17 +217,13 @@ struct WarpSearch {
     __device__ __forceinline__ float *cd() const { return reinterpret_cast<float *>(base + a.lay.cd); }
     __device__ __forceinline__ uint32_t *ci() const { return reinterpret_cast<uint32_t *>(base + a.lay.ci); }
     __device__ __forceinline__ uint32_t *cs() const { return reinterpret_cast<uint32_t *>(base + a.lay.cs); }
-    __device__ __forceinline__ uint32_t *adj() const { return reinterpret_cast<uint32_t *>(base + a.lay.adj); }
-    __device__ __forceinline__ uint32_t *dirs() const { return reinterpret_cast<uint32_t *>(base + a.lay.dir); }
-    __device__ __forceinline__ uint8_t *prow() const { return base + a.lay.prow; }
-    __device__ __forceinline__ uint32_t *par() const { return reinterpret_cast<uint32_t *>(base + a.lay.par); }
     __device__ __forceinline__ uint8_t *stage() const { return base + a.lay.stage; }
     __device__ __forceinline__ uint64_t *bar() const { return reinterpret_cast<uint64_t *>(base + a.lay.bar); }
     // two words beside the mbarrier (its 16-byte slot): the ghost judge
     __device__ __forceinline__ uint32_t *judge() const { return reinterpret_cast<uint32_t *>(base + a.lay.bar + 8); }
 
     // ---------------------------------------------------------- visited set
-    __device__ __forceinline__ uint32_t *gbits() const { return reinterpret_cast<uint32_t *>(base + a.lay.dir); }
+    __device__ __forceinline__ uint32_t *gbits() const { return reinterpret_cast<uint32_t *>(base + a.lay.gbm); }
     __device__ __forceinline__ uint32_t hash_home(uint32_t v) const { return (v * 2654435761u) >> (32 - a.vbits); }
 
     // The rest of a test-and-insert of entry want (id + 1) whose first probe,
@@ -457,32 +456,24 @@ struct WarpSearch {
         __syncwarp();
     }
 
-    // Collect the kept neighbours of parent pi in slots lane + 32 (r0 + r),
-    // r < NW (bit r0 + r of km), that are new to the visited set. The first
-    // probes of a lane's NW slots are issued before any result is examined,
-    // so their latencies overlap. Returns the warp's new candidate count.
+    // Collect the ids nb[r] (those with ok[r]) that are new to the visited
+    // table. The first probes of a lane's NW ids are issued before any result
+    // is examined, so their latencies overlap. Returns the warp's new
+    // candidate count.
     template <uint32_t NW>
-    __device__ uint32_t collect_row_nw(const View &v, uint32_t pi, uint32_t km, uint32_t r0, uint32_t nc)
+    __device__ __forceinline__ uint32_t collect_ids(const uint32_t (&nb)[NW], const bool (&ok)[NW], uint32_t nc)
     {
-        uint32_t nb[NW], hs[NW], cur[NW], old[NW];
-        bool ok[NW];
-#pragma unroll
-        for (uint32_t r = 0; r < NW; ++r) {
-            const uint32_t j = lane + 32 * (r0 + r);
-            nb[r] = j < v.deg ? adj()[pi * v.deg_pad + j] : ANN_INVALID_ID;
-            ok[r] = nb[r] != ANN_INVALID_ID && ((km >> (r0 + r)) & 1u);
-        }
+        uint32_t hs[NW], old[NW];
 #pragma unroll
         for (uint32_t r = 0; r < NW; ++r) {
             if (ok[r]) {
                 hs[r] = hash_home(nb[r]);
-                cur[r] = nb[r] + 1;
-                old[r] = atomicCAS(vt + hs[r], 0u, cur[r]);
+                old[r] = atomicCAS(vt + hs[r], 0u, nb[r] + 1);
             }
         }
 #pragma unroll
         for (uint32_t r = 0; r < NW; ++r) {
-            const bool isnew = ok[r] && hash_finish(hs[r], cur[r], old[r]);
+            const bool isnew = ok[r] && hash_finish(hs[r], nb[r] + 1, old[r]);
             const uint32_t m = __ballot_sync(0xffffffffu, isnew);
             if (isnew) ci()[nc + __popc(m & lanemask_lt())] = nb[r];
             nc += __popc(m);
@@ -490,20 +481,31 @@ struct WarpSearch {
         return nc;
     }
 
-    __device__ uint32_t collect_row(const View &v, uint32_t pi, uint32_t km, uint32_t nc)
+    // Collect all neighbours of np parents (lane i holds parent i's id): the
+    // lists' slots, as one sequence, NW x 32 at a time, loaded together.
+    template <uint32_t NW>
+    __device__ uint32_t expand_all(const View &v, uint32_t np, uint32_t pid, uint32_t nc)
     {
-        if (gbm) {
-            #pragma unroll 1
-            for (uint32_t r = 0; r * 32 < v.deg; ++r) {
-                const uint32_t j = lane + 32 * r;
-                const uint32_t nb = j < v.deg ? adj()[pi * v.deg_pad + j] : ANN_INVALID_ID;
-                nc = collect(nb != ANN_INVALID_ID && ((km >> r) & 1u), nb, nc);
-            }
-            return nc;
-        }
-        if (v.deg <= 32) return collect_row_nw<1>(v, pi, km, 0, nc);
+        const uint32_t dp = v.deg_pad, slots = np * dp;
         #pragma unroll 1
-        for (uint32_t r0 = 0; r0 * 32 < v.deg; r0 += 2) nc = collect_row_nw<2>(v, pi, km, r0, nc);
+        for (uint32_t b = 0; b < slots; b += 32 * NW) {
+            uint32_t nb[NW];
+            bool ok[NW];
+#pragma unroll
+            for (uint32_t r = 0; r < NW; ++r) {
+                const uint32_t x = b + 32 * r + lane, p = __umulhi(x, v.deg_magic);
+                const uint32_t parent = __shfl_sync(0xffffffffu, pid, min(p, np - 1));
+                // past the degree a list holds no ids
+                nb[r] = x < slots ? __ldg(v.graph + (uint64_t)parent * dp + (x - p * dp)) : ANN_INVALID_ID;
+                ok[r] = nb[r] != ANN_INVALID_ID;
+            }
+            if (gbm) {
+#pragma unroll
+                for (uint32_t r = 0; r < NW; ++r) nc = collect(ok[r], nb[r], nc);
+            } else {
+                nc = collect_ids<NW>(nb, ok, nc);
+            }
+        }
         return nc;
     }
 
@@ -538,8 +540,9 @@ struct WarpSearch {
     }
 
     // ---------------------------------------------------------- iterations
-    // Parents: the first `W` eligible queue entries in queue order.
-    __device__ uint32_t select_parents(uint32_t W, bool cool)
+    // Parents: the first `W` eligible queue entries in queue order; lane i
+    // holds parent i's queue slot.
+    __device__ uint32_t select_parents(uint32_t W, bool cool, uint32_t &slot)
     {
         uint32_t np = 0;
         const uint8_t *s8 = bs();
@@ -555,11 +558,10 @@ struct WarpSearch {
             while (m && np < W) {
                 const uint32_t bit = __ffs(m) - 1;
                 m &= m - 1;
-                if (lane == 0) par()[np] = b + bit;
+                if (lane == np) slot = b + bit;
                 ++np;
             }
         }
-        __syncwarp();
         return np;
     }
 
@@ -571,93 +573,169 @@ struct WarpSearch {
         return __any_sync(0xffffffffu, p);
     }
 
-    // DGS keep-mask of parent pi (bit r of the result: slot lane + 32 r is
-    // kept). Score = matching sign bits; keep the top n_keep by (score desc,
-    // slot asc): find the threshold score t by a radix select with ballots
-    // (most significant bit first), keep scores above t and the first ties
-    // at t. With min_match > 0, keep instead every neighbour scoring at
-    // least min_match. NW = number of 32-slot words the degree spans (1, 2
-    // or 4), so no ballot is spent on slots past the degree.
-    template <uint32_t NW>
-    __device__ uint32_t dgs_keep_nw(const View &v, uint32_t pi, uint32_t n_keep, uint32_t min_match, float ps)
+    // DGS (Section 3.3.2 (b)). The parent's list, its direction words and its
+    // row are read straight into registers, four words at a time: staged in
+    // shared memory they took 1.4 KB a warp at 96 dimensions and 8 KB at 768,
+    // and direction rows of 4, 8 or 24 words fell into few banks.
+    //
+    // u = score + 2 of slots r0 + 32 r + lane, r < N: 0 past the degree (never
+    // kept), 1 for an empty slot, 2 + matching bits for a neighbour.
+    template <uint32_t N>
+    __device__ __forceinline__ void scores(const View &v, uint32_t pid, uint32_t r0, uint32_t (&nb)[N],
+                                           uint32_t (&u)[N])
     {
         const uint32_t w = a.w, deg = v.deg;
-        const uint8_t *pr = prow() + pi * a.prow_bytes;
-        // mismatching sign bits per slot, 4 words of the query's sign bits
-        // relative to the parent ([q > x_parent], one ballot per 32
-        // dimensions) at a time. Words past w have no dimension (their bits
-        // are 0) and count nothing; the loads stay in the row (clamped), so
-        // a chunk has no branch and its loads issue together.
-        int diff[NW];
-        bool live[NW];
-        const uint32_t *db[NW];
+        const uint8_t *pr = v.codes + (uint64_t)pid * v.row_bytes;
+        const uint32_t *list = v.graph + (uint64_t)pid * v.deg_pad;
+        const float ps = ST != ANN_F32 ? __ldg(v.scales + pid) : 1.0f;
+        const uint32_t *db[N];
 #pragma unroll
-        for (uint32_t r = 0; r < NW; ++r) {
-            const uint32_t j = min(lane + 32 * r, deg - 1);
-            live[r] = lane + 32 * r < deg && adj()[pi * v.deg_pad + j] != ANN_INVALID_ID;
-            db[r] = dirs() + (pi * v.deg_pad + j) * w;
-            diff[r] = 0;
+        for (uint32_t r = 0; r < N; ++r) {
+            const uint32_t j = r0 + lane + 32 * r, jc = min(j, deg - 1);
+            nb[r] = j < deg ? __ldg(list + jc) : ANN_INVALID_ID;
+            db[r] = v.dir + ((uint64_t)pid * v.deg_pad + jc) * w;
+            u[r] = 0;   // mismatching sign bits
         }
+        // 4 words of the query's sign bits relative to the parent ([q >
+        // x_parent], one ballot per 32 dimensions) at a time. Words past w
+        // have no dimension: their bits are 0 on both sides.
+        #pragma unroll 1
         for (uint32_t t0 = 0; t0 < w; t0 += 4) {
-            uint32_t qw[4];
+            uint32_t dw[N][4];
+            if (w % 4 == 0) {   // rows of whole 16-byte units
+#pragma unroll
+                for (uint32_t r = 0; r < N; ++r) {
+                    const uint4 d4 = __ldg(reinterpret_cast<const uint4 *>(db[r] + t0));
+                    dw[r][0] = d4.x; dw[r][1] = d4.y; dw[r][2] = d4.z; dw[r][3] = d4.w;
+                }
+            } else {
+#pragma unroll
+                for (uint32_t r = 0; r < N; ++r)
+#pragma unroll
+                    for (uint32_t x = 0; x < 4; ++x) dw[r][x] = t0 + x < w ? __ldg(db[r] + t0 + x) : 0u;
+            }
+            float pv[4];
+#pragma unroll
+            for (uint32_t x = 0; x < 4; ++x)
+                pv[x] = stored_elem<ST>(pr, min(32 * (t0 + x) + lane, a.d - 1), ps);
 #pragma unroll
             for (uint32_t x = 0; x < 4; ++x) {
                 const uint32_t i = 32 * (t0 + x) + lane;
-                const uint32_t ic = min(i, a.d - 1);
-                qw[x] = __ballot_sync(0xffffffffu, i < a.d && q()[ic] > stored_elem<ST>(pr, ic, ps));
+                const uint32_t qw = __ballot_sync(0xffffffffu, i < a.d && q()[min(i, a.d - 1)] > pv[x]);
+#pragma unroll
+                for (uint32_t r = 0; r < N; ++r) u[r] += __popc(qw ^ dw[r][x]);
             }
-#pragma unroll
-            for (uint32_t r = 0; r < NW; ++r)
-#pragma unroll
-                for (uint32_t x = 0; x < 4; ++x) {
-                    const uint32_t dw = db[r][min(t0 + x, w - 1)];
-                    diff[r] += t0 + x < w ? __popc(qw[x] ^ dw) : 0;
-                }
         }
-        // u = score + 2: 0 past the degree (never kept), 1 for an empty
-        // slot, 2 + matching bits for a neighbour
-        uint32_t u[NW];
 #pragma unroll
-        for (uint32_t r = 0; r < NW; ++r) {
-            const uint32_t j = lane + 32 * r;
-            u[r] = j >= deg ? 0u : (live[r] ? a.d + 2 - (uint32_t)diff[r] : 1u);
-        }
-        if (min_match > 0) {
-            uint32_t keep = 0;
-#pragma unroll
-            for (uint32_t r = 0; r < NW; ++r)
-                if (u[r] >= min_match + 2) keep |= 1u << r;
-            return keep;
-        }
-        // radix select of the n_keep-th largest u: t collects its bits from
-        // the top; `need` counts how many of the values equal to t's bits so
-        // far are still to be kept. At the end every u > t is kept and
-        // `need` of the ties at t.
-        uint32_t t = 0, need = n_keep;
+        for (uint32_t r = 0; r < N; ++r)
+            u[r] = r0 + lane + 32 * r >= deg ? 0u : (nb[r] != ANN_INVALID_ID ? a.d + 2 - u[r] : 1u);
+    }
+
+    // The n_keep-th largest u of the warp's slots (at(r): slot word r's u) and
+    // how many of the ties at it are kept: a radix select with ballots. t
+    // collects the value's bits from the top; `need` counts how many of the
+    // values equal to t's bits so far are still to be kept.
+    template <uint32_t NW, typename At>
+    __device__ __forceinline__ uint32_t threshold(uint32_t n_keep, uint32_t &need, At at)
+    {
+        uint32_t t = 0;
+        need = n_keep;
         for (int bit = 31 - __clz(a.d + 2); bit >= 0; --bit) {
             const uint32_t hi = (t >> bit) | 1u;
             uint32_t c = 0;
 #pragma unroll
-            for (uint32_t r = 0; r < NW; ++r) c += __popc(__ballot_sync(0xffffffffu, (u[r] >> bit) == hi));
+            for (uint32_t r = 0; r < NW; ++r) c += __popc(__ballot_sync(0xffffffffu, (at(r) >> bit) == hi));
             if (c >= need) t |= 1u << bit;
             else need -= c;
         }
-        uint32_t keep = 0, ties_before = 0;
-#pragma unroll
-        for (uint32_t r = 0; r < NW; ++r) {
-            const uint32_t tm = __ballot_sync(0xffffffffu, u[r] == t);
-            const bool tie_kept = u[r] == t && ties_before + __popc(tm & lanemask_lt()) < need;
-            if (u[r] > t || tie_kept) keep |= 1u << r;
-            ties_before += __popc(tm);
-        }
-        return keep;
+        return t;
     }
 
-    __device__ uint32_t dgs_keep(const View &v, uint32_t pi, uint32_t n_keep, uint32_t min_match, float ps)
+    // DGS of parent `pid` and the visited test of the neighbours it keeps
+    // (slots lane + 32 r, r < NW). Score = matching sign bits; keep the top
+    // n_keep by (score desc, slot asc): scores above the threshold and the
+    // first ties at it. With min_match > 0, keep instead every neighbour
+    // scoring at least min_match. NW = number of 32-slot words the degree
+    // spans, so no ballot is spent on slots past the degree.
+    template <uint32_t NW>
+    __device__ __forceinline__ uint32_t expand_dgs_nw(const View &v, uint32_t pid, uint32_t n_keep, uint32_t min_match,
+                                                      uint32_t nc)
     {
-        if (v.deg <= 32) return dgs_keep_nw<1>(v, pi, n_keep, min_match, ps);
-        if (v.deg <= 64) return dgs_keep_nw<2>(v, pi, n_keep, min_match, ps);
-        return dgs_keep_nw<kMaxDegWords>(v, pi, n_keep, min_match, ps);
+        uint32_t nb[NW], u[NW];
+        bool keep[NW];
+        scores<NW>(v, pid, 0, nb, u);
+        if (min_match > 0) {
+#pragma unroll
+            for (uint32_t r = 0; r < NW; ++r) keep[r] = u[r] >= min_match + 2;
+        } else {
+            uint32_t need, ties_before = 0;
+            const uint32_t t = threshold<NW>(n_keep, need, [&](uint32_t r) { return u[r]; });
+#pragma unroll
+            for (uint32_t r = 0; r < NW; ++r) {
+                const uint32_t tm = __ballot_sync(0xffffffffu, u[r] == t);
+                keep[r] = u[r] > t || (u[r] == t && ties_before + __popc(tm & lanemask_lt()) < need);
+                ties_before += __popc(tm);
+            }
+        }
+        mark(PH_DGS);
+#pragma unroll
+        for (uint32_t r = 0; r < NW; ++r) keep[r] = keep[r] && nb[r] != ANN_INVALID_ID;
+        return collect_ids<NW>(nb, keep, nc);
+    }
+
+    // The same for lists of more than 64 slots, whose scores are kept in
+    // shared memory (cs(), free until the merge): in registers they would
+    // cost every other search spills.
+    __device__ __forceinline__ uint32_t expand_dgs_long(const View &v, uint32_t pid, uint32_t n_keep,
+                                                        uint32_t min_match, uint32_t nc)
+    {
+        uint32_t *su = cs();
+        const uint32_t words = (v.deg + 31) / 32;
+        #pragma unroll 1
+        for (uint32_t r = 0; r < words; ++r) {
+            uint32_t nb[1], u[1];
+            scores<1>(v, pid, 32 * r, nb, u);
+            su[32 * r + lane] = u[0];
+        }
+        __syncwarp();
+        uint32_t need = 0, ties_before = 0, t = min_match + 1;
+        if (min_match == 0) t = threshold<kMaxDegWords>(n_keep, need, 
+                                                           [&](uint32_t r) { return r < words ? su[32 * r + lane] : 0u; });
+        mark(PH_DGS);
+        #pragma unroll 1
+        for (uint32_t r = 0; r < words; ++r) {
+            const uint32_t j = 32 * r + lane, u = su[j];
+            const uint32_t tm = __ballot_sync(0xffffffffu, u == t);
+            const uint32_t nb[1] = {j < v.deg ? __ldg(v.graph + (uint64_t)pid * v.deg_pad + j) : ANN_INVALID_ID};
+            const bool keep[1] = {nb[0] != ANN_INVALID_ID &&
+                                  (u > t || (u == t && ties_before + __popc(tm & lanemask_lt()) < need))};
+            ties_before += __popc(tm);
+            nc = collect_ids<1>(nb, keep, nc);
+        }
+        return nc;
+    }
+
+    __device__ uint32_t expand_dgs(const View &v, uint32_t pid, uint32_t n_keep, uint32_t min_match, uint32_t nc)
+    {
+        if (v.deg <= 32) return expand_dgs_nw<1>(v, pid, n_keep, min_match, nc);
+        if (v.deg <= 64) return expand_dgs_nw<2>(v, pid, n_keep, min_match, nc);
+        return expand_dgs_long(v, pid, n_keep, min_match, nc);
+    }
+
+    __device__ __forceinline__ void prefetch_parents(const View &v, uint32_t np, uint32_t pid)
+    {
+        const uint32_t list = v.deg_pad * 4, dir = v.deg_pad * a.w * 4;
+        #pragma unroll 1
+        for (uint32_t pi = 1; pi < np; ++pi) {
+            const uint64_t p = __shfl_sync(0xffffffffu, pid, pi);
+            auto lines = [&](const void *row, uint32_t bytes) {
+                for (uint32_t o = lane * 128; o < bytes; o += 32 * 128)
+                    asm volatile("prefetch.global.L2 [%0];" ::"l"(static_cast<const uint8_t *>(row) + o));
+            };
+            lines(v.graph + p * v.deg_pad, list);
+            lines(v.dir + p * v.deg_pad * a.w, dir);
+            lines(v.codes + p * v.row_bytes, v.row_bytes);
+        }
     }
 
     // Step 2 (m seeds, in chunks of the candidate capacity), then Steps 3-4
@@ -676,7 +754,6 @@ struct WarpSearch {
     {
         const uint32_t deg = v.deg;
         const bool dgs_on = v.dir != nullptr && (min_match > 0 || n_keep < deg);
-        const uint32_t w = a.w;
         bool cool = false;
         uint32_t j0 = 0, it = 0;
         for (;;) {
@@ -694,57 +771,37 @@ struct WarpSearch {
                     T = t_ext;   // judged too far: the rest of the ghost iterations
                 }
                 if (dgs_on && it >= it_cool) cool = true;
-                uint32_t np = select_parents(W, cool);
+                uint32_t slot = 0;
+                uint32_t np = select_parents(W, cool, slot);
                 if (np == 0 && dgs_on && reexpand && !cool && any_partial()) {
                     cool = true;
-                    np = select_parents(W, cool);
+                    np = select_parents(W, cool, slot);
                 }
                 if (np == 0) break;
                 ++it;
                 ++c_iters;
                 const bool dgs_now = dgs_on && !cool;
-                // mark the parents; fetch adjacency (and, under DGS, direction
-                // and vector) rows in one bulk-copy round
-                const uint32_t adj_bytes = v.deg_pad * 4;
-                const uint32_t dir_bytes = v.deg_pad * w * 4;
                 uint32_t pid = 0;
+                __syncwarp();   // every lane has read the states
                 if (lane < np) {
-                    const uint32_t b = par()[lane];
-                    pid = bi()[b];
-                    bs()[b] = (dgs_now && reexpand) ? kPartial : kExpanded;
+                    pid = bi()[slot];
+                    bs()[slot] = (dgs_now && reexpand) ? kPartial : kExpanded;
                 }
-                if (lane == 0) {
-                    fence_proxy_async();
-                    mbar_arrive_expect_tx(bar(), np * (adj_bytes + (dgs_now ? dir_bytes + v.row_bytes : 0)));
-                }
-                __syncwarp();
-                if (lane < np) {
-                    bulk_g2s(adj() + lane * v.deg_pad, v.graph + (uint64_t)pid * v.deg_pad, adj_bytes, bar());
-                    if (dgs_now) {
-                        bulk_g2s(dirs() + lane * v.deg_pad * w, v.dir + (uint64_t)pid * v.deg_pad * w, dir_bytes,
-                                 bar());
-                        bulk_g2s(prow() + lane * a.prow_bytes, v.codes + (uint64_t)pid * v.row_bytes, v.row_bytes,
-                                 bar());
-                        // the parent's scale replaces its queue slot in
-                        // par() (read by DGS after the wait)
-                        if (RST != ANN_F32) par()[lane] = __float_as_uint(__ldg(v.scales + pid));
-                    }
-                }
-                if (!wait_copies()) return false;
                 mark(PH_SELECT);
                 c_parents += np;
-                if (dgs_now) c_dgs += np;
                 hash_make_room(np * deg);
-                for (uint32_t pi = 0; pi < np; ++pi) {
-                    uint32_t km = 0xffffffffu;
-                    if (dgs_now) {
-                        km = dgs_keep(v, pi, n_keep, min_match,
-                                      RST != ANN_F32 ? __uint_as_float(par()[pi]) : 1.0f);
-                        mark(PH_DGS);
-                    }
-                    nc = collect_row(v, pi, km, nc);
-                    mark(PH_VISIT);
+                if (dgs_now) {
+                    c_dgs += np;
+                    // the further parents' lists and direction rows start on
+                    // their way to L2 while the first is expanded
+                    if (np > 1) prefetch_parents(v, np, pid);
+                    #pragma unroll 1
+                    for (uint32_t pi = 0; pi < np; ++pi)
+                        nc = expand_dgs(v, __shfl_sync(0xffffffffu, pid, pi), n_keep, min_match, nc);
+                } else {
+                    nc = expand_all<2>(v, np, pid, nc);
                 }
+                mark(PH_VISIT);
             }
             __syncwarp();
             hash_count += nc;
@@ -787,7 +844,7 @@ struct WarpSearch {
         // 1: the search on the base graph. One loop body serves both.
         bool ok = true;
         for (uint32_t stage = ghost ? 0u : 1u; stage < 2 && ok; ++stage) {
-            const View v = stage ? a.base : a.ghost;
+            const View &v = a.view[stage];
             const uint32_t lcap = stage ? qp.L : qp.Lg;
             uint32_t rows = 0, iters = 0, parents = 0, dgs_parents = 0;
             if (PROF && stage == 1 && ghost) {
@@ -974,9 +1031,8 @@ __global__ void __launch_bounds__(128, kSearchBlocksPerSm) serve_kernel(const Ar
 
 uint32_t align16(uint32_t x) { return (x + 15) & ~15u; }
 
-Layout make_layout(uint32_t d, uint32_t w, uint32_t cap_buf, uint32_t cap_cand, uint32_t W, uint32_t W_max,
-                   uint32_t adj_words, uint32_t dir_words, uint32_t prow_bytes, uint32_t stage_rows,
-                   uint32_t stage_stride, uint32_t rr_stride, uint32_t gbm_words, bool serve)
+Layout make_layout(uint32_t d, uint32_t cap_buf, uint32_t cap_cand, uint32_t stage_rows, uint32_t stage_stride,
+                   uint32_t rr_stride, uint32_t gbm_words, bool serve)
 {
     Layout L{};
     uint32_t o = 0;
@@ -989,16 +1045,10 @@ Layout make_layout(uint32_t d, uint32_t w, uint32_t cap_buf, uint32_t cap_cand, 
     L.bd = take(cap_buf * 4);
     L.bi = take(cap_buf * 4);
     L.bs = take(cap_buf);
-    L.cd = take(std::max(cap_cand, cap_buf) * 4);
+    L.cd = take(cap_cand * 4);
     L.ci = take(cap_cand * 4);
     L.cs = take(cap_cand * 4);
-    L.adj = take(adj_words * 4);
-    // the base stage's direction and parent rows share their space with the
-    // ghost stage's visited bitmap (the two stages never overlap)
-    const uint32_t dir_part = align16(dir_words * 4) + align16(dir_words ? W * prow_bytes : 0);
-    L.dir = take(std::max(dir_part, gbm_words * 4));
-    L.prow = L.dir + align16(dir_words * 4);
-    L.par = take(W_max * 4);   // parents of an iteration of either stage
+    L.gbm = take(gbm_words * 4);
     // the staged rows (at least one of the rerank's FP32 rows); the merge
     // keeps its candidates' insertion points here
     L.stage = take(std::max(std::max(stage_rows * stage_stride, rr_stride), cap_cand * 4));
@@ -1134,15 +1184,15 @@ ann_status derive_qparams(const ann_index *ix, const ann_search_params *p, uint3
 
 namespace planning {
 
-// Kernel arguments and launch shape for parameters q (the largest a launch
-// must serve): shared-memory layout per warp, warps per block, blocks per SM.
-ann_status plan_args(ann_index *ix, const QParams &q, Args &a, int &warps, size_t &smem, int &nb, bool serve)
+// Kernel arguments for parameters q (the largest a launch must serve), all but
+// the launch shape.
+ann_status plan_args(ann_index *ix, const QParams &q, Args &a)
 {
     const uint32_t deg = ix->degree;
-    a.base = View{(const uint8_t *)ix->codes, ix->scales, ix->row_bytes, ix->graph, deg, ix->deg_pad,
-                  ix->dir, (uint32_t)ix->n};
-    a.ghost = View{(const uint8_t *)ix->ghost_codes, ix->ghost_scales, ix->row_bytes, ix->ghost_graph,
-                   ix->ghost_degree, ix->gdeg_pad, nullptr, ix->n_ghost};
+    a.view[1] = View{(const uint8_t *)ix->codes, ix->scales, ix->row_bytes, ix->graph, deg, ix->deg_pad,
+                  magic32(ix->deg_pad), ix->dir, (uint32_t)ix->n};
+    a.view[0] = View{(const uint8_t *)ix->ghost_codes, ix->ghost_scales, ix->row_bytes, ix->ghost_graph,
+                   ix->ghost_degree, ix->gdeg_pad, magic32(ix->gdeg_pad), nullptr, ix->n_ghost};
     a.ghost_ids = ix->ghost_ids;
     a.x32 = (const uint8_t *)ix->x32;
     a.row32_bytes = ix->storage == ANN_F32 ? ix->row_bytes : ix->row32_bytes;
@@ -1153,11 +1203,8 @@ ann_status plan_args(ann_index *ix, const QParams &q, Args &a, int &warps, size_
     uint32_t cap_cand = std::max(q.W * deg, 32u);
     if (ghost_entry(q.entry)) cap_cand = std::max(cap_cand, q.Wg * ix->ghost_degree);
     cap_cand = round_up(cap_cand, 32);
+    a.cap_buf = cap_buf;
     a.cap_cand = cap_cand;
-    const uint32_t adj_words = std::max(q.W * ix->deg_pad, q.Wg * ix->gdeg_pad);
-    const bool dgs = q.n_keep < deg || q.min_match > 0;
-    const uint32_t dir_words = dgs ? q.W * ix->deg_pad * ix->words : 0;
-    a.prow_bytes = ix->row_bytes;
     // the search stages stored rows; the rerank stages FP32 rows in the same
     // area, fewer per round (it reads itopk rows per query, the search
     // thousands), so the area is sized by the stored rows
@@ -1179,55 +1226,77 @@ ann_status plan_args(ann_index *ix, const QParams &q, Args &a, int &warps, size_
     a.vbits = ix->visited.bits;   // 4,096 entries: measured faster than 2,048 or 1,024 (L2-resident either way)
     a.slot_base = 0;
     a.gbm_words = (ghost_entry(q.entry) && ix->n_ghost <= kGhostBitmapMax) ? (ix->n_ghost + 31) / 32 : 0;
-    // Shape for `rows` staged rows per gather round: the per-warp layout,
-    // warps per block (wide rows: fewer staged rows before fewer warps) and
-    // resident blocks per SM. False if no shape fits.
+    // one warp with a few staged rows is the least a launch can be made of
+    const uint32_t least = make_layout(a.d, cap_buf, cap_cand, 4, a.stage_stride, a.rr_stride, a.gbm_words, true).total;
+    if (least > ix->smem_optin) {
+        set_error("ann_search: per-query state (%u bytes) exceeds shared memory", least);
+        return ANN_EINVAL;
+    }
+    return ANN_OK;
+}
+
+// The launch shape for nq queries: rows staged per gather round, the per-warp
+// layout, warps per block and blocks per SM.
+ann_status plan_shape(ann_index *ix, Args &a, uint64_t nq, bool serve, int &warps, size_t &smem, int &nb)
+{
     struct Shape {
         Layout lay;
         uint32_t rows;
         int warps, nb;
         size_t smem;
     };
-    auto fit = [&](uint32_t rows, Shape &sh) -> bool {
+    auto fit = [&](uint32_t rows) {
+        Shape best{}, sh{};
         sh.rows = rows;
-        sh.warps = 4;
-        for (;;) {
-            sh.lay = make_layout(ix->dim, ix->words, cap_buf, cap_cand, q.W,
-                                 std::max(q.W, ghost_entry(q.entry) ? q.Wg : 1u), adj_words, dir_words,
-                                 a.prow_bytes, sh.rows, a.stage_stride, a.rr_stride, a.gbm_words, serve);
-            if ((size_t)sh.lay.total * sh.warps <= ix->smem_optin) break;
-            if (sh.rows > 4) { sh.rows /= 2; continue; }
-            if (sh.warps > 1) { sh.warps /= 2; continue; }
-            set_error("ann_search: per-query state (%u bytes) exceeds shared memory", sh.lay.total);
-            return false;
+        sh.lay = make_layout(a.d, a.cap_buf, a.cap_cand, rows, a.stage_stride, a.rr_stride, a.gbm_words, serve);
+        // blocks of one or two warps pack a shared memory that blocks of four
+        // leave partly unused (256-d FP32 rows, 512-entry queues: 14 resident
+        // warps an SM instead of 12)
+        for (sh.warps = 4; sh.warps >= 1; sh.warps /= 2) {
+            sh.smem = (size_t)sh.lay.total * sh.warps;
+            if (sh.smem > ix->smem_optin) continue;
+            switch (ix->storage) {
+            case ANN_F32: sh.nb = blocks_per_sm<ANN_F32>(sh.warps, sh.smem, a.lpr); break;
+            case ANN_F16: sh.nb = blocks_per_sm<ANN_F16>(sh.warps, sh.smem, a.lpr); break;
+            default: sh.nb = blocks_per_sm<ANN_E4M3>(sh.warps, sh.smem, a.lpr); break;
+            }
+            if (sh.nb * sh.warps > best.nb * best.warps) best = sh;
         }
-        sh.smem = (size_t)sh.lay.total * sh.warps;
-        switch (ix->storage) {
-        case ANN_F32: sh.nb = blocks_per_sm<ANN_F32>(sh.warps, sh.smem, a.lpr); break;
-        case ANN_F16: sh.nb = blocks_per_sm<ANN_F16>(sh.warps, sh.smem, a.lpr); break;
-        default: sh.nb = blocks_per_sm<ANN_E4M3>(sh.warps, sh.smem, a.lpr); break;
-        }
-        if (sh.nb <= 0) {
-            set_error("ann_search: kernel does not fit on an SM (%zu bytes shared)", sh.smem);
-            return false;
-        }
-        return true;
+        return best;
     };
-    // The staged rows take most of a warp's shared memory. With the full
-    // round (16 rows, 8 wide ones) shared memory can hold fewer warps than
-    // the registers allow (large queues, 1 KB rows); half a round then
-    // doubles the gather rounds but admits more resident warps, and the
-    // latency those warps hide is worth more (measured: +19% to +43% where
-    // the warps per SM rose, -18% where they did not). So half a round is
-    // taken only when it admits more warps per SM. ANN_STAGE_ROWS fixes the
-    // count instead (experiments).
+    // The staged rows take most of a warp's shared memory. Fewer of them per
+    // gather round mean more rounds, so a slower query, but can admit more
+    // resident warps. What that is worth depends on how often the resident
+    // warps have to be filled to take the batch: fewer rows are taken only
+    // where they lower that count, and a quarter round only where everything
+    // then runs at once. Measured, ms with 16 / 8 / 4 rows: 256-d FP32,
+    // itopk 256: 1,300 queries 3.27 / 3.81 / 4.96 (one filling each), 2,000
+    // queries 6.18 / 4.08 / 5.27 (2, 1, 1), 2,432 queries 6.34 / 7.43 / 5.42 (2,
+    // 2, 1), 8,000 queries 18.8 / 15.7 / 16.5 (6, 4, 4); 768-d FP16, 8 / 4
+    // rows: 1,300 queries 1.34 / 1.89 (1, 1), 3,001 queries 2.59 / 2.38 (2, 1).
+    // ANN_STAGE_ROWS fixes the count instead (experiments).
     const int env_rows = env_int("ANN_STAGE_ROWS", 0);
     const uint32_t full = 32 / a.lpr;
-    Shape best;
-    if (!fit(env_rows > 0 ? (uint32_t)std::min<int>((int)full, env_rows) : full, best)) return ANN_EINVAL;
-    if (env_rows <= 0 && best.rows == full) {
-        Shape half;
-        if (fit(full / 2, half) && half.nb * half.warps > best.nb * best.warps) best = half;
+    auto fillings = [&](const Shape &s) {
+        const uint64_t slots = (uint64_t)s.nb * s.warps * ix->num_sms;
+        return slots ? (nq + slots - 1) / slots : ~0ull;
+    };
+    Shape best{};
+    if (env_rows > 0) {
+        best = fit((uint32_t)std::min<int>((int)full, env_rows));
+    } else {
+        best = fit(full);
+        const Shape half = fit(full / 2);
+        if (fillings(half) < fillings(best)) best = half;
+        if (full / 4 >= 4 && fillings(best) > 1) {
+            const Shape quarter = fit(full / 4);
+            if (fillings(quarter) == 1) best = quarter;
+        }
+    }
+    if (best.warps == 0) best = fit(4);
+    if (best.warps == 0) {
+        set_error("ann_search: kernel does not fit on an SM");
+        return ANN_EINVAL;
     }
     a.stage_rows = best.rows;
     a.rr_rows = a.rr_stride ? std::min(full, std::max(1u, best.rows * a.stage_stride / a.rr_stride)) : 0u;
@@ -1280,9 +1349,7 @@ ann_status search_launch_ex(ann_index *ix, const float *queries, uint32_t nq, co
     }
     if (nq == 0) return ANN_OK;
     Args a{};
-    int warps = 0, nb = 0;
-    size_t smem = 0;
-    s = plan_args(ix, q, a, warps, smem, nb, false);
+    s = plan_args(ix, q, a);
     if (s != ANN_OK) return s;
     a.queries = queries;
     a.nq = nq;
@@ -1300,8 +1367,8 @@ ann_status search_launch_ex(ann_index *ix, const float *queries, uint32_t nq, co
     // the teams (search_team.cu); the profile and a fixed ANN_STAGE_ROWS are
     // the warp kernel's
     if (!prof && env_int("ANN_STAGE_ROWS", 0) <= 0) {
-        const TeamSearch t{a.base, a.ghost, a.ghost_ids, a.x32, a.row32_bytes, a.d, a.w, std::max(q.L, ghost_entry(q.entry) ? q.Lg : 1u),
-                           a.cap_cand, a.gbm_words, q.n_keep < ix->degree || q.min_match > 0, q, queries, nq, given,
+        const TeamSearch t{a.view[1], a.view[0], a.ghost_ids, a.x32, a.row32_bytes, a.d, a.w, a.cap_buf, a.cap_cand,
+                           a.gbm_words, q.n_keep < ix->degree || q.min_match > 0, q, queries, nq, given,
                            ids, dists, stats, err, ix->storage, ix->num_sms, ix->smem_optin};
         cudaError_t te = cudaSuccess;
         if (team_search(t, stream, &te)) {
@@ -1312,6 +1379,10 @@ ann_status search_launch_ex(ann_index *ix, const float *queries, uint32_t nq, co
             return ANN_OK;
         }
     }
+    int warps = 0, nb = 0;
+    size_t smem = 0;
+    s = plan_shape(ix, a, nq, false, warps, smem, nb);
+    if (s != ANN_OK) return s;
     const uint64_t want = ((uint64_t)nq + warps - 1) / warps;
     // every resident warp needs its own visited table
     const uint64_t cap = std::min<uint64_t>((uint64_t)nb * ix->num_sms, ix->visited.slots / (uint32_t)warps);
@@ -1345,7 +1416,9 @@ ann_status serve_plan(ann_index *ix, const ann_search_params *maxp, uint32_t n_g
     ann_status s = derive_qparams(ix, maxp, n_given_max, &q);
     if (s != ANN_OK) return s;
     ServePlanImpl *pl = new ServePlanImpl();
-    s = plan_args(ix, q, pl->a, pl->warps, pl->smem, pl->nb, true);
+    s = plan_args(ix, q, pl->a);
+    // a server is sized for more queries than run at once
+    if (s == ANN_OK) s = plan_shape(ix, pl->a, 1u << 20, true, pl->warps, pl->smem, pl->nb);
     if (s == ANN_OK) {
         pl->slots_per_launch = (uint32_t)(pl->nb * ix->num_sms * pl->warps);
         s = visited_pool_alloc(pl->visited, pl->slots_per_launch * std::max(1u, n_streams), kVisitedBits);

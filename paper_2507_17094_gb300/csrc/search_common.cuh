@@ -21,12 +21,15 @@ __host__ __device__ __forceinline__ bool given_entry(uint32_t e)
     return e == ANN_ENTRY_GIVEN_GHOST || e == ANN_ENTRY_GIVEN_BASE;
 }
 
+// ceil(2^32 / d): __umulhi(x, magic32(d)) = x / d for x d < 2^32 and d > 1.
+inline uint32_t magic32(uint32_t d) { return d > 1 ? (uint32_t)(((1ull << 32) + d - 1) / d) : 0u; }
+
 struct View {
     const uint8_t *codes;
     const float *scales;   // nullptr for FP32
     uint32_t row_bytes;
     const uint32_t *graph;
-    uint32_t deg, deg_pad;
+    uint32_t deg, deg_pad, deg_magic;   // deg_magic = magic32(deg_pad)
     const uint32_t *dir;   // nullptr: no DGS on this graph
     uint32_t n;
 };

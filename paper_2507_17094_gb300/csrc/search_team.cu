@@ -46,7 +46,6 @@ struct TeamArgs {
     TeamLayout lay;
     uint32_t rows, stride, rr_rows, rr_stride;   // rows per gather round and their stride: stored rows, FP32 rerank
     uint32_t row_magic, row32_magic;             // ceil(2^32 / 16-byte chunks of a row): chunk index -> row
-    uint32_t deg_magic, gdeg_magic;              // the same for the slots of a list
 };
 
 // Shared counters: the candidates found and the survivors of a loop pass,
@@ -321,7 +320,7 @@ struct Team {
         const uint32_t *dw = v.dir;
         uint32_t word[kDirWords];
         auto load = [&]() {
-            p = __umulhi(x, g.deg_magic);
+            p = __umulhi(x, v.deg_magic);
             j = x - p * dp;
             const uint64_t parent = __shfl_sync(0xffffffffu, pid, min(p, np - 1));
             if (x < slots) {
@@ -397,7 +396,7 @@ struct Team {
             const uint32_t y = b + (lane >> 2);
             uint32_t n = ANN_INVALID_ID, better = 0;
             if (y < slots) {
-                const uint32_t pp = __umulhi(y, g.deg_magic), mine = score()[y];
+                const uint32_t pp = __umulhi(y, v.deg_magic), mine = score()[y];
                 n = adj()[y];
                 const uint4 *s4 = reinterpret_cast<const uint4 *>(score() + pp * dp);
 #pragma unroll 4
@@ -416,7 +415,7 @@ struct Team {
     // Seeds, then iterations of parents, adjacency, direction-guided
     // selection, visited test, distances and merge (the warp kernel's
     // iterate, whose comments give the passages).
-    __device__ __forceinline__ void iterate(const View &v, uint32_t deg_magic, const uint32_t *seed_ids, uint32_t m,
+    __device__ __forceinline__ void iterate(const View &v, const uint32_t *seed_ids, uint32_t m,
                                             uint64_t seed_key, uint32_t lcap, uint32_t W, uint32_t T, uint32_t T_ext,
                                             float judge, uint32_t n_keep, uint32_t min_match, uint32_t it_cool,
                                             uint32_t reexpand, uint32_t &c_iters, uint32_t &c_parents,
@@ -467,7 +466,7 @@ struct Team {
                     const uint32_t dp = v.deg_pad;
                     #pragma unroll 1
                     for (uint32_t b = warp * 32; b < np * dp; b += NT) {
-                        const uint32_t x = b + lane, p = __umulhi(x, deg_magic);
+                        const uint32_t x = b + lane, p = __umulhi(x, v.deg_magic);
                         const uint64_t parent = __shfl_sync(0xffffffffu, pid, min(p, np - 1));
                         const uint32_t nb = x < np * dp ? __ldg(v.graph + parent * dp + (x - p * dp)) : ANN_INVALID_ID;
                         collect(nb != ANN_INVALID_ID, nb);   // past the degree the list holds no ids
@@ -532,7 +531,7 @@ struct Team {
             }
             const bool seeded = !(stage == 1 && ghost);
             const bool judged = stage == 0 && given && qp.judge > 0.0f && qp.Tg > qp.Tg_given;
-            iterate(v, stage ? g.deg_magic : g.gdeg_magic, given,
+            iterate(v, given,
                     seeded ? (given ? qp.n_given : (stage ? qp.m : v.deg)) : 0,
                     splitmix64(qp.seed ^ (stage ? 0 : kGhostTag)), stage ? qp.L : qp.Lg, stage ? qp.W : qp.Wg,
                     stage ? qp.T : (given ? qp.Tg_given : qp.Tg), judged ? qp.Tg : 0u, judged ? qp.judge : 0.0f,
@@ -582,8 +581,10 @@ struct Team {
     }
 };
 
+constexpr uint32_t kMostPerSm = 7;   // resident teams of 128 threads by their registers
+
 template <int ST, int NT>
-__global__ void __launch_bounds__(NT, NT == 256 ? 4 : 7) team_kernel(const __grid_constant__ TeamArgs g)
+__global__ void __launch_bounds__(NT, NT == 256 ? 4 : kMostPerSm) team_kernel(const __grid_constant__ TeamArgs g)
 {
     extern __shared__ __align__(128) uint8_t smem[];
     Team<ST, NT> t(g, smem);
@@ -593,9 +594,6 @@ __global__ void __launch_bounds__(NT, NT == 256 ? 4 : 7) team_kernel(const __gri
           (given_entry(a.qp.entry) && a.given) ? a.given + (uint64_t)qi * a.qp.n_given : nullptr,
           a.out_ids + (uint64_t)qi * a.qp.k, a.out_dists + (uint64_t)qi * a.qp.k, a.stats ? a.stats + qi : nullptr);
 }
-
-// ceil(2^32 / d): __umulhi(x, magic(d)) = x / d for x d < 2^32 and d > 1
-uint32_t magic(uint32_t d) { return d > 1 ? (uint32_t)(((1ull << 32) + d - 1) / d) : 0u; }
 
 TeamArgs plan(const TeamSearch &t, uint32_t rows, uint32_t max_rows)
 {
@@ -628,10 +626,8 @@ TeamArgs plan(const TeamSearch &t, uint32_t rows, uint32_t max_rows)
     g.rr_rows = g.rr_stride ? std::min(max_rows, bytes / g.rr_stride) : 0u;
     L.stage = take(bytes);
     L.total = o;
-    g.row_magic = magic(t.base.row_bytes / 16);
-    g.row32_magic = magic(std::max(16u, t.row32_bytes) / 16);
-    g.deg_magic = magic(t.base.deg_pad);
-    g.gdeg_magic = magic(std::max(1u, t.ghost.deg_pad));
+    g.row_magic = magic32(t.base.row_bytes / 16);
+    g.row32_magic = magic32(std::max(16u, t.row32_bytes) / 16);
     return g;
 }
 
@@ -665,6 +661,7 @@ bool try_teams(const TeamSearch &t, uint32_t least_rows, cudaStream_t stream, cu
 template <int ST>
 bool run_teams(const TeamSearch &t, cudaStream_t stream, cudaError_t *e)
 {
+    if (t.nq > kMostPerSm * (uint64_t)t.num_sms) return false;
     return try_teams<ST, 256>(t, 16, stream, e) || try_teams<ST, 128>(t, 8, stream, e);
 }
 
