@@ -404,11 +404,12 @@ ann_status ann_mlp_load(const char *path, int device, uint32_t max_batch, ann_ml
 /* ------------------------------------------------------------------------
  * Continuous-batching server (not in the paper). Requests (batches of any
  * size, each with its own ann_search_params up to the server's max_params)
- * are admitted while others run and share the GPU query by query: one device
- * ring of query slots, a FIFO that the warps of every running search kernel
- * take queries from, per-warp queue and visited state resident in shared
- * memory while a query runs. Admission is by buffer memory: submit returns
- * ANN_EBUSY when the ring or the request records are full (poll, then retry).
+ * are admitted while others run and share the GPU query by query: one ring
+ * of query slots (page-locked host memory the device reads and writes), a FIFO
+ * that the warps of every running search kernel take queries from, per-warp
+ * queue and visited state resident in shared memory while a query runs.
+ * Admission is by buffer memory: submit returns ANN_EBUSY when the ring or the
+ * request records are full (poll, then retry).
  * Results are deterministic per request (the RNG stream is qid_base + the
  * query's index within its request), so a request's answer is the same alone
  * or in any mix. One host thread drives a server.
@@ -416,13 +417,14 @@ ann_status ann_mlp_load(const char *path, int device, uint32_t max_batch, ann_ml
 typedef struct ann_server ann_server;
 
 typedef struct {
-    uint32_t capacity;            /* query slots resident on the device */
+    uint32_t capacity;            /* query slots in the ring */
     uint32_t max_requests;        /* requests in flight */
     ann_search_params max_params; /* largest k, itopk, search_width, ghost_itopk of any request, and the
                                      features allowed (DGS if dgs_discard > 0, rerank, entry != random) */
     uint32_t seeds_per_query;     /* learned entry (max_params.entry == ANN_ENTRY_GIVEN_GHOST): P, 1..8 */
     float tau;                    /* learned entry: fallback threshold on the top softmax probability */
-    uint32_t queries_per_warp;    /* queries a warp serves before its kernel may end; 0 = 4 */
+    uint32_t queries_per_warp;    /* queries a warp serves, at least, before its kernel may end; 0 = as few as
+                                     the queries in flight allow */
     uint32_t streams;             /* compute streams; 0 = 4 */
 } ann_server_config;
 

@@ -57,6 +57,9 @@ class SearchParams(C.Structure):
                 ("ghost_search_width", C.c_uint32), ("dgs_min_match", C.c_float), ("ghost_judge", C.c_float)]
 
 
+_PARAM_NAMES = frozenset(f for f, _ in SearchParams._fields_)
+
+
 class ServerConfig(C.Structure):
     _fields_ = [("capacity", C.c_uint32), ("max_requests", C.c_uint32), ("max_params", SearchParams),
                 ("seeds_per_query", C.c_uint32), ("tau", C.c_float), ("queries_per_warp", C.c_uint32),
@@ -160,9 +163,8 @@ def make_params(**kw) -> SearchParams:
     """ann_search_params from keyword arguments over the library defaults."""
     p = SearchParams()
     lib().ann_default_params(C.byref(p))
-    names = {f for f, _ in SearchParams._fields_}
     for k, v in kw.items():
-        if k not in names:
+        if k not in _PARAM_NAMES:
             raise TypeError(f"unknown search parameter {k!r}")
         setattr(p, k, v)
     return p

@@ -86,24 +86,28 @@ struct QParams {
 };
 static_assert(sizeof(QParams) <= 96, "the serve kernel keeps a request's QParams in 96 bytes of shared memory");
 
-// One request in the serving ring (device memory).
+// One request in the serving ring (host memory, mapped).
 struct ServeReq {
     QParams qp;
-    uint32_t nq, slot0, done, flag;
+    uint32_t nq, slot0, flag;
 };
 
-// The serving ring as the serve kernel sees it.
+// The serving ring as the serve kernel sees it. Queries, results, the request
+// records and the completion flags are host memory that the device reads and
+// writes directly; the counters are device memory.
 struct ServeRing {
-    const float *queries;            // cap x dim
-    const uint32_t *seeds;           // cap x P (learned entry) or NULL
+    const float *queries;            // cap x dim (host)
+    const uint32_t *seeds;           // cap x P (learned entry; device) or NULL
     uint32_t P;
-    uint32_t *ids;                   // cap x kmax
-    float *dists;                    // cap x kmax
-    const uint32_t *slot_req;        // cap: request-ring index of each slot
-    ServeReq *reqs;
-    unsigned long long *head;        // next query to take
-    const unsigned long long *tail;  // queries published
-    volatile uint32_t *flags;        // host-mapped completion flags
+    uint32_t *ids;                   // cap x kmax (host)
+    float *dists;                    // cap x kmax (host)
+    const uint32_t *slot_req;        // cap: request-ring index of each slot (host)
+    const ServeReq *reqs;            // host
+    uint32_t *done;                  // per request record: queries finished (device; zero between requests)
+    unsigned long long *counters;    // device: [0] queries taken, [1] queries made available, [2] their difference
+    unsigned long long tail;         // queries published before this launch
+    const unsigned long long *live;  // queries published so far (host), for a launch that makes later ones available; or NULL
+    volatile uint32_t *flags;        // completion flags (host)
     uint32_t cap, kmax, per_warp;
 };
 
@@ -124,9 +128,11 @@ ann_status derive_qparams(const ann_index *ix, const ann_search_params *p, uint3
 ann_status serve_plan(ann_index *ix, const ann_search_params *maxp, uint32_t n_given_max, uint32_t n_streams,
                       void **plan);
 void serve_plan_free(void *plan);
-// Launch a serve kernel with capacity for at least `queries` queries on
-// `stream`, the plan's concurrent-launch slot `stream_index`.
-ann_status serve_launch(void *plan, const ServeRing &ring, uint32_t queries, cudaStream_t stream,
+// Launch a serve kernel on `stream`, the plan's concurrent-launch slot
+// `stream_index`: `warps` of them, as far as they can be resident, each serving
+// at least ring.per_warp queries and enough that together they can serve
+// `queries`.
+ann_status serve_launch(void *plan, ServeRing ring, uint32_t warps, uint32_t queries, cudaStream_t stream,
                         uint32_t stream_index);
 
 // The search launch (search.cu) with the index's own work counter and error

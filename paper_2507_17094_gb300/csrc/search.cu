@@ -829,16 +829,16 @@ struct WarpSearch {
             pstage = ghost_entry(qp.entry) ? PS_GHOST : PS_BASE;
         }
         const uint32_t dpad = (a.d + 31) & ~31u;
-        // read through L2 only: a serving ring rewrites query slots between
-        // uses, and L1 is not kept coherent with those copies
+        // past L1: a serving ring's slots are rewritten between uses
         #pragma unroll 1
-        for (uint32_t i = lane; i < dpad; i += 32) q()[i] = i < a.d ? __ldcg(qg + i) : 0.0f;
+        for (uint32_t i = lane; i < dpad; i += 32)
+            q()[i] = i < a.d ? *reinterpret_cast<const volatile float *>(qg + i) : 0.0f;
         __syncwarp();
         const bool ghost = ghost_entry(qp.entry);
         gbm = ghost && a.gbm_words > 0;
         hash_clear();
         const uint32_t *given = nullptr;
-        if (given_entry(qp.entry) && given_row && given_row[0] != ANN_INVALID_ID)
+        if (given_entry(qp.entry) && given_row && __ldcg(given_row) != ANN_INVALID_ID)
             given = given_row;   // else: fall back to random (ghost) seeds
         // stage 0: the ghost stage (Section 3.2.2) on the ghost graph; stage
         // 1: the search on the base graph. One loop body serves both.
@@ -973,14 +973,49 @@ __global__ void __launch_bounds__(128, kSearchBlocksPerSm) search_kernel(const A
     }
 }
 
-// Continuous batching: warps of every running serve kernel pop queries, in
-// arrival order, from one device ring that the host appends to while they
-// run (head/tail are monotonic query counters; slot = counter mod capacity).
-// A warp serves at most `per_warp` queries and then leaves, so a launch's
-// capacity is blocks x warps x per_warp and SMs free up for other kernels.
-// The request's parameters are copied into the warp's shared memory; the
-// warp that finishes a request's last query raises its completion flag in
-// host-mapped memory after a system-scope fence.
+// Continuous batching: warps of every running serve kernel take queries, in
+// arrival order, from one ring (monotonic query counters; slot = counter mod
+// capacity). A launch makes available the queries published before it and, with
+// `live`, those published until its warps start; each request brings a launch,
+// so all are taken, and a warp serves at most `per_warp` queries and then
+// leaves, so SMs free up for other kernels. Queries, records and results are
+// host memory, read and written over the chip-to-chip link: a query's few
+// hundred bytes are small against the row bytes its search gathers, and no copy
+// is queued for them. The request's parameters are copied into the warp's shared
+// memory; the warp that finishes a request's last query raises its completion
+// flag after a system-scope fence.
+//
+// Taking a query is two additions: one to the count of available queries, given
+// back if there was none, and one to the count of those taken. (A compare and
+// swap of the latter fails for all but one of the warps that try together: 3,000
+// queries took 2.7 ms, 0.9 of which was searching.) A warp that gave back looks
+// again before it leaves: of several that fail together the last to give back
+// sees what the others hid, so no available query is left behind.
+
+// Make the queries up to `tail` available; lane 0 only.
+__device__ __forceinline__ void serve_publish(const ServeRing &r, unsigned long long tail)
+{
+    if (tail <= *reinterpret_cast<volatile unsigned long long *>(r.counters + 1)) return;
+    __threadfence();   // what `tail` counts, before the counts
+    const unsigned long long was = atomicMax(r.counters + 1, tail);
+    if (was < tail) atomicAdd(r.counters + 2, tail - was);
+}
+
+// Take the next query: true and its counter in *h; lane 0 only.
+__device__ __forceinline__ bool serve_take(const ServeRing &r, unsigned long long *h)
+{
+    for (uint32_t attempt = 0; attempt < (1u << 20); ++attempt) {
+        if ((long long)atomicAdd(r.counters + 2, ~0ull) > 0) {
+            *h = atomicAdd(r.counters, 1ull);
+            __threadfence();
+            return true;
+        }
+        atomicAdd(r.counters + 2, 1ull);
+        if ((long long)*reinterpret_cast<volatile unsigned long long *>(r.counters + 2) <= 0) break;
+    }
+    return false;
+}
+
 template <int ST, int LPR = 2>
 __global__ void __launch_bounds__(128, kSearchBlocksPerSm) serve_kernel(const Args a, const ServeRing r)
 {
@@ -992,37 +1027,41 @@ __global__ void __launch_bounds__(128, kSearchBlocksPerSm) serve_kernel(const Ar
     if (lane == 0) mbar_init(ws.bar(), 1);
     fence_mbar_init();
     __syncwarp();
+    if (lane == 0) {
+        unsigned long long tail = r.tail;
+        if (r.live)   // acquire: what it counts was written before it
+            asm volatile("ld.acquire.sys.global.u64 %0, [%1];" : "=l"(tail) : "l"(r.live) : "memory");
+        serve_publish(r, tail);
+    }
     for (uint32_t served = 0; served < r.per_warp; ++served) {
         unsigned long long h = 0;
         uint32_t got = 0;
-        if (lane == 0) {
-            for (uint32_t attempt = 0; attempt < (1u << 20); ++attempt) {  // lock-free: a failed CAS means another warp won
-                h = *reinterpret_cast<volatile unsigned long long *>(r.head);
-                const unsigned long long t = *reinterpret_cast<volatile const unsigned long long *>(r.tail);
-                if (h >= t) break;
-                if (atomicCAS(r.head, h, h + 1) == h) { got = 1; break; }
-            }
-        }
+        if (lane == 0) got = serve_take(r, &h);
         got = __shfl_sync(0xffffffffu, got, 0);
         if (!got) break;
         h = __shfl_sync(0xffffffffu, h, 0);
         const uint32_t slot = (uint32_t)(h % r.cap);
-        ServeReq *rq = r.reqs + __ldcg(r.slot_req + slot);
+        const uint32_t ri = *reinterpret_cast<const volatile uint32_t *>(r.slot_req + slot);
+        const ServeReq *rq = r.reqs + ri;
         if (lane < sizeof(QParams) / 4)
             reinterpret_cast<uint32_t *>(qp)[lane] = reinterpret_cast<const volatile uint32_t *>(&rq->qp)[lane];
+        const uint32_t nq = *reinterpret_cast<const volatile uint32_t *>(&rq->nq);
+        const uint32_t slot0 = *reinterpret_cast<const volatile uint32_t *>(&rq->slot0);
+        const uint32_t flag = *reinterpret_cast<const volatile uint32_t *>(&rq->flag);
         __syncwarp();
-        const uint32_t j = (slot + r.cap - *reinterpret_cast<volatile uint32_t *>(&rq->slot0)) % r.cap;
+        const uint32_t j = (slot + r.cap - slot0) % r.cap;
         const uint32_t *seeds = (qp->entry == ANN_ENTRY_GIVEN_GHOST && r.seeds) ? r.seeds + (size_t)slot * r.P : nullptr;
         ws.run(*qp, j, r.queries + (size_t)slot * a.d, seeds, r.ids + (size_t)slot * r.kmax,
                r.dists + (size_t)slot * r.kmax, nullptr);
         if (ws.failed) break;
-        __threadfence();
+        __threadfence_system();   // the results, before the count that can raise the flag
         __syncwarp();
         if (lane == 0) {
-            const uint32_t done = atomicAdd(&rq->done, 1u) + 1;
-            if (done == *reinterpret_cast<volatile uint32_t *>(&rq->nq)) {
+            const uint32_t done = atomicAdd(r.done + ri, 1u) + 1;
+            if (done == nq) {
+                r.done[ri] = 0;   // for the record's next request
                 __threadfence_system();
-                r.flags[rq->flag] = 1u;
+                r.flags[flag] = 1u;
             }
         }
         __syncwarp();
@@ -1260,7 +1299,10 @@ ann_status plan_shape(ann_index *ix, Args &a, uint64_t nq, bool serve, int &warp
             case ANN_F16: sh.nb = blocks_per_sm<ANN_F16>(sh.warps, sh.smem, a.lpr); break;
             default: sh.nb = blocks_per_sm<ANN_E4M3>(sh.warps, sh.smem, a.lpr); break;
             }
-            if (sh.nb * sh.warps > best.nb * best.warps) best = sh;
+            // A server's warps take and finish queries one by one, and a block
+            // holds its shared memory until its last warp is done: single
+            // warps where as many fit.
+            if (sh.nb * sh.warps > best.nb * best.warps || (serve && sh.nb * sh.warps == best.nb * best.warps)) best = sh;
         }
         return best;
     };
@@ -1441,14 +1483,15 @@ void serve_plan_free(void *plan)
     delete pl;
 }
 
-ann_status serve_launch(void *plan, const ServeRing &ring, uint32_t queries, cudaStream_t stream,
+ann_status serve_launch(void *plan, ServeRing ring, uint32_t warps, uint32_t queries, cudaStream_t stream,
                         uint32_t stream_index)
 {
     ServePlanImpl &pl = *static_cast<ServePlanImpl *>(plan);
     pl.a.slot_base = stream_index * pl.slots_per_launch;
-    const uint64_t per_block = (uint64_t)pl.warps * ring.per_warp;
-    const uint64_t want = ((uint64_t)queries + per_block - 1) / per_block;
+    const uint64_t want = ((uint64_t)warps + pl.warps - 1) / pl.warps;
     const int blocks = (int)std::max<uint64_t>(1, std::min<uint64_t>(want, (uint64_t)pl.nb * pl.num_sms));
+    const uint32_t resident = (uint32_t)(blocks * pl.warps);
+    ring.per_warp = std::max(std::max(1u, ring.per_warp), (queries + resident - 1) / resident);
     cudaError_t e;
     switch (pl.storage) {
     case ANN_F32: e = launch_serve<ANN_F32>(pl, ring, blocks, stream); break;
