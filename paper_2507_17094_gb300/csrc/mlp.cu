@@ -5,7 +5,7 @@
 // Dense contractions run on the 5th-generation tensor cores: one GEMM kernel
 // computes C = A * B^T with A (M x K) and B (N x K) both K-major BF16 in
 // global memory, FP32 accumulation in tensor memory:
-//   - TMA 2-D loads (128-byte swizzle) fill a 4-stage shared-memory ring,
+//   - TMA 2-D loads (128-byte swizzle) fill a shared-memory ring of 4 to 9 stages,
 //     one elected thread issues them; full/empty mbarriers link the stages;
 //   - one elected thread issues tcgen05.mma (M 128, N 128, K 16 per
 //     instruction) reading both operands from shared memory by descriptor;
@@ -19,6 +19,7 @@
 #include <cuda_bf16.h>
 
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstdio>
 #include <cstdlib>
@@ -31,16 +32,21 @@ using namespace ann;
 
 namespace {
 
-constexpr int BM = 128, BN = 128, BK = 64, STAGES = 4;
+constexpr int BM = 128, BN = 128, BK = 64;
 constexpr int TILE_A = BM * BK * 2;
 constexpr int TILE_B = BN * BK * 2;
-constexpr int GEMM_STAGE_BYTES = STAGES * (TILE_A + TILE_B);
 // top-P epilogue: each of the 8 x 32 epilogue threads parks a 32-logit chunk
 // here (stride 33 floats: conflict-free) while it inserts the chunk's
 // candidates one per step
 constexpr int XS_STRIDE = 33;
 constexpr int GEMM_XS_BYTES = 8 * 32 * XS_STRIDE * 4;
-constexpr int GEMM_SMEM = GEMM_STAGE_BYTES + 256 + GEMM_XS_BYTES + 1024;
+enum { EPI_F32 = 0, EPI_BIAS_F32 = 1, EPI_BIAS_RELU_BF16 = 2, EPI_TOPP = 3, EPI_MASK = 4 };
+// Stages of the (A, B) ring: what the epilogue leaves room for.
+constexpr int ring_stages(int epi, int nt) { return epi == EPI_TOPP ? 4 : nt == 64 ? 9 : 7; }
+constexpr int ring_smem(int epi, int nt)
+{
+    return ring_stages(epi, nt) * (TILE_A + nt * BK * 2) + 256 + (epi == EPI_TOPP ? GEMM_XS_BYTES : 0) + 1024;
+}
 // Resident-A variant (fused top-P logits, K <= RES_K): a CTA keeps its row
 // block's whole A (128 x K, as RES_K / BK swizzled 128 x BK tiles) in shared
 // memory while B streams through a ring of RES_STAGES tiles, so the L2 ->
@@ -52,12 +58,11 @@ constexpr int RES_SMEM = RES_A_BYTES + RES_STAGES * TILE_B + 256 + GEMM_XS_BYTES
 static_assert(RES_SMEM <= 232448, "resident-A GEMM exceeds the shared memory of a CTA");
 constexpr int TOPP = 8;   // top-P of the fused inference epilogue
 
-enum { EPI_F32 = 0, EPI_BIAS_F32 = 1, EPI_BIAS_RELU_BF16 = 2, EPI_TOPP = 3 };
-
 struct EpiArgs {
     float *c;                 // FP32 output, row stride ldc
     __nv_bfloat16 *cb;        // BF16 output, row stride ldc
     const float *bias;        // per output column
+    const __nv_bfloat16 *mask;   // EPI_MASK: outputs where it is not positive are 0; row stride ldc
     uint32_t ldc;
     float *part;              // top-P partials: per (row, column tile) TOPP values, TOPP ids, max, sum
     uint32_t ntiles;
@@ -152,7 +157,7 @@ struct TopP {
 template <int EPI>
 __device__ __forceinline__ void load_bias32(const EpiArgs &e, uint32_t nb, uint32_t N, float (&bias)[32])
 {
-    if (EPI == EPI_F32) return;
+    if (EPI == EPI_F32 || EPI == EPI_MASK) return;
     if (nb + 32 <= N) {
 #pragma unroll
         for (int j = 0; j < 32; j += 4) {
@@ -189,6 +194,37 @@ __device__ __forceinline__ void epilogue_chunk(const float (&v)[32], const float
 #pragma unroll
             for (int j = 0; j < 32; ++j)
                 if (nb + j < N) out[j] = v[j] + (EPI == EPI_BIAS_F32 ? bias[j] : 0.0f);
+        }
+    } else if (EPI == EPI_MASK) {
+        if (m >= M) return;
+        const size_t at = (size_t)m * e.ldc + nb;
+        if (full && (e.ldc % 8) == 0) {
+#pragma unroll
+            for (int j = 0; j < 32; j += 8) {
+                const uint4 mk = __ldg(reinterpret_cast<const uint4 *>(e.mask + at + j));
+                const uint32_t mw[4] = {mk.x, mk.y, mk.z, mk.w};
+                float o[8];
+                uint32_t b[4];
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    const __nv_bfloat162 h = *reinterpret_cast<const __nv_bfloat162 *>(&mw[k]);
+                    o[2 * k] = __bfloat162float(h.x) > 0.0f ? v[j + 2 * k] : 0.0f;
+                    o[2 * k + 1] = __bfloat162float(h.y) > 0.0f ? v[j + 2 * k + 1] : 0.0f;
+                    const __nv_bfloat162 r = __floats2bfloat162_rn(o[2 * k], o[2 * k + 1]);
+                    b[k] = *reinterpret_cast<const uint32_t *>(&r);
+                }
+                *reinterpret_cast<float4 *>(e.c + at + j) = make_float4(o[0], o[1], o[2], o[3]);
+                *reinterpret_cast<float4 *>(e.c + at + j + 4) = make_float4(o[4], o[5], o[6], o[7]);
+                *reinterpret_cast<uint4 *>(e.cb + at + j) = make_uint4(b[0], b[1], b[2], b[3]);
+            }
+        } else {
+#pragma unroll
+            for (int j = 0; j < 32; ++j)
+                if (nb + j < N) {
+                    const float o = __bfloat162float(e.mask[at + j]) > 0.0f ? v[j] : 0.0f;
+                    e.c[at + j] = o;
+                    e.cb[at + j] = __float2bfloat16_rn(o);
+                }
         }
     } else if (EPI == EPI_BIAS_RELU_BF16) {
         if (m >= M) return;
@@ -352,22 +388,26 @@ __device__ __forceinline__ void topp_flush(const EpiArgs &e, const TopP &tp, uin
 // MODE 0: the ring of (A, B) tiles; 1: resident A; 2: resident A, and the
 // CTAs run in clusters of two on the two row blocks of a pair, loading half
 // of each B tile each and multicasting it to both (B is read from L2 once
-// per pair instead of once per CTA).
-template <int EPI, int MODE = 0>
+// per pair instead of once per CTA). AMN / BMN (MODE 0): A is given as K x M, B
+// as K x N, row-major (MN-major operands), so that a product with a transposed
+// matrix reads the matrix itself.
+template <int EPI, int MODE = 0, bool AMN = false, bool BMN = false, int NT = BN>
 __global__ void __launch_bounds__(GEMM_THREADS, 1)
     gemm_kernel(const __grid_constant__ CUtensorMap tA, const __grid_constant__ CUtensorMap tB, uint32_t M,
                 uint32_t N, uint32_t K, EpiArgs e)
 {
     constexpr bool RESA = MODE >= 1, MC = MODE == 2;
+    static_assert(NT == BN || (NT == 64 && MODE == 0 && EPI != EPI_TOPP), "narrow tiles: plain ring only");
+    constexpr uint32_t TILE_N = NT * BK * 2;   // bytes of a B tile
     extern __shared__ uint8_t smem_raw[];
     const uint32_t pad = (1024u - (smem_addr(smem_raw) & 1023u)) & 1023u;
     uint8_t *smem = smem_raw + pad;
     // ring layout: STAGES x (A tile, B tile); resident-A layout: the row
     // block's A tiles, then RES_STAGES B tiles
-    constexpr int NST = RESA ? RES_STAGES : STAGES;
-    constexpr int BAR_OFF = RESA ? RES_A_BYTES + RES_STAGES * TILE_B : GEMM_STAGE_BYTES;
+    constexpr int NST = RESA ? RES_STAGES : ring_stages(EPI, NT);
+    constexpr int BAR_OFF = RESA ? RES_A_BYTES + RES_STAGES * TILE_N : NST * (TILE_A + TILE_N);
     uint8_t *sA = smem;
-    uint8_t *sB = smem + (RESA ? RES_A_BYTES : STAGES * TILE_A);
+    uint8_t *sB = smem + (RESA ? RES_A_BYTES : NST * TILE_A);
     uint64_t *full = reinterpret_cast<uint64_t *>(smem + BAR_OFF);
     uint64_t *empty = full + NST;
     uint64_t *acc_full = empty + NST;        // [2]: MMA -> epilogue
@@ -378,7 +418,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
     float *xs_all = reinterpret_cast<float *>(smem + BAR_OFF + 256);
     const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t nkb = (K + BK - 1) / BK;
-    const uint32_t n_tiles = (N + BN - 1) / BN, m_tiles = (M + BM - 1) / BM;
+    const uint32_t n_tiles = (N + NT - 1) / NT, m_tiles = (M + BM - 1) / BM;
     // work units: tiles, or with clusters (row-block pair, column tile);
     // unit t covers row block rb(t) = row unit (t / n_tiles), or with
     // clusters row block 2 (t / n_tiles) + the CTA's rank in its pair
@@ -406,7 +446,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
     if (MC) cluster_sync_all();
     if (warp == 1) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_addr(tmem_slot)),
-                     "r"((uint32_t)(2 * BN))
+                     "r"((uint32_t)(2 * NT))
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
@@ -422,7 +462,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
             uint32_t it = 0, loads = 0, cur_u = 0xFFFFFFFFu;
             bool ok = true;
             for (uint32_t t = t_begin; t < t_end && ok; ++t) {
-                const uint32_t u = t / n_tiles, n0 = (t % n_tiles) * BN;
+                const uint32_t u = t / n_tiles, n0 = (t % n_tiles) * NT;
                 if (u != cur_u) {
                     if (loads > 0 && !(ok = mbar_wait_bounded(a_empty, (loads - 1) & 1, e.err))) break;
                     mbar_arrive_expect_tx(a_full, nkb * TILE_A);
@@ -434,84 +474,84 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
                 for (uint32_t kb = 0; kb < nkb; ++kb, ++it) {
                     const uint32_t s = it % NST, ph = (it / NST) & 1;
                     if (!(ok = mbar_wait_bounded(&empty[s], ph ^ 1, e.err))) break;
-                    mbar_arrive_expect_tx(&full[s], TILE_B);
+                    mbar_arrive_expect_tx(&full[s], TILE_N);
                     if (MC)   // this CTA's half of the B tile (64 rows), to both CTAs
-                        tma_load_2d_mc(sB + s * TILE_B + crank * (TILE_B / 2), &tB, (int)(kb * BK),
-                                       (int)(n0 + crank * (BN / 2)), &full[s], (uint16_t)3);
+                        tma_load_2d_mc(sB + s * TILE_N + crank * (TILE_N / 2), &tB, (int)(kb * BK),
+                                       (int)(n0 + crank * (NT / 2)), &full[s], (uint16_t)3);
                     else
-                        tma_load_2d(sB + s * TILE_B, &tB, (int)(kb * BK), (int)n0, &full[s]);
+                        tma_load_2d(sB + s * TILE_N, &tB, (int)(kb * BK), (int)n0, &full[s]);
                 }
             }
         }
     } else if (warp == 0) {
-        if (lane == 0) {
-            uint32_t it = 0;
-            bool ok = true;
-            for (uint32_t t = t_begin; t < t_end && ok; ++t) {
-                const uint32_t m0 = (t / n_tiles) * BM, n0 = (t % n_tiles) * BN;
-                for (uint32_t kb = 0; kb < nkb; ++kb, ++it) {
-                    const uint32_t s = it % STAGES, ph = (it / STAGES) & 1;
-                    if (!(ok = mbar_wait_bounded(&empty[s], ph ^ 1, e.err))) break;
-                    mbar_arrive_expect_tx(&full[s], TILE_A + TILE_B);
-                    tma_load_2d(sA + s * TILE_A, &tA, (int)(kb * BK), (int)m0, &full[s]);
-                    tma_load_2d(sB + s * TILE_B, &tB, (int)(kb * BK), (int)n0, &full[s]);
+        uint32_t s = 0, ph = 0;
+        bool ok = true;
+        for (uint32_t t = t_begin; t < t_end && ok; ++t) {
+            const uint32_t m0 = (t / n_tiles) * BM, n0 = (t % n_tiles) * NT;
+            for (uint32_t kb = 0; kb < nkb; ++kb) {
+                if (!(ok = __all_sync(0xffffffffu, mbar_wait_bounded(&empty[s], ph ^ 1, e.err)))) break;
+                if (elect_one()) {
+                    uint8_t *a = sA + s * TILE_A, *b = sB + s * TILE_N;
+                    mbar_arrive_expect_tx(&full[s], TILE_A + TILE_N);
+                    if (AMN) {
+                        tma_load_2d(a, &tA, (int)m0, (int)(kb * BK), &full[s]);
+                        tma_load_2d(a + kBoxBytes, &tA, (int)m0 + 64, (int)(kb * BK), &full[s]);
+                    } else {
+                        tma_load_2d(a, &tA, (int)(kb * BK), (int)m0, &full[s]);
+                    }
+                    if (BMN) {
+                        tma_load_2d(b, &tB, (int)n0, (int)(kb * BK), &full[s]);
+                        if (NT == 128) tma_load_2d(b + kBoxBytes, &tB, (int)n0 + 64, (int)(kb * BK), &full[s]);
+                    } else {
+                        tma_load_2d(b, &tB, (int)(kb * BK), (int)n0, &full[s]);
+                    }
                 }
-            }
-        }
-    } else if (warp == 1 && RESA) {
-        if (lane == 0) {
-            constexpr uint32_t idesc = idesc_bf16(BM, BN);
-            uint32_t it = 0, tc = 0, loads = 0, cur_u = 0xFFFFFFFFu;
-            bool ok = true;
-            for (uint32_t t = t_begin; t < t_end && ok; ++t, ++tc) {
-                const uint32_t u = t / n_tiles;
-                if (u != cur_u) {
-                    if (!(ok = mbar_wait_bounded(a_full, loads & 1, e.err))) break;
-                    cur_u = u;
-                    ++loads;
-                }
-                const uint32_t buf = tc & 1, use = tc >> 1;
-                if (!(ok = mbar_wait_bounded(&acc_empty[buf], (use & 1) ^ 1, e.err))) break;
-                tc_fence_after();
-                const uint32_t acc = tmem + buf * BN;
-                for (uint32_t kb = 0; kb < nkb; ++kb, ++it) {
-                    const uint32_t s = it % NST, ph = (it / NST) & 1;
-                    if (!(ok = mbar_wait_bounded(&full[s], ph, e.err))) break;
-                    tc_fence_after();
-                    const uint32_t a0 = smem_addr(sA + kb * TILE_A), b0 = smem_addr(sB + s * TILE_B);
-#pragma unroll
-                    for (uint32_t k = 0; k < BK / 16; ++k)
-                        mma_f16kind(acc, desc_sw128(a0 + k * 32), desc_sw128(b0 + k * 32), idesc, (kb | k) != 0);
-                    if (MC) mma_commit_mc(&empty[s], (uint16_t)3);   // frees the stage in both CTAs
-                    else mma_commit(&empty[s]);
-                }
-                mma_commit(&acc_full[buf]);
-                // the last tile of this row block: A may be replaced once
-                // these MMAs are done
-                if (t + 1 < t_end && (t + 1) / n_tiles != u) mma_commit(a_empty);
+                __syncwarp();
+                if (++s == NST) { s = 0; ph ^= 1; }
             }
         }
     } else if (warp == 1) {
-        if (lane == 0) {
-            constexpr uint32_t idesc = idesc_bf16(BM, BN);
-            uint32_t it = 0, tc = 0;
-            bool ok = true;
-            for (uint32_t t = t_begin; t < t_end && ok; ++t, ++tc) {
-                const uint32_t buf = tc & 1, use = tc >> 1;
-                if (!(ok = mbar_wait_bounded(&acc_empty[buf], (use & 1) ^ 1, e.err))) break;
+        // all lanes run the loop, one issues (elect_one says why)
+        constexpr uint32_t idesc = idesc_bf16(BM, NT) | (AMN ? kIdescAMN : 0u) | (BMN ? kIdescBMN : 0u);
+        constexpr uint32_t a_step = AMN ? 128 : 2, b_step = BMN ? 128 : 2;   // 16 elements of K
+        const uint32_t a_lo = AMN ? desc_lo_mn(smem_addr(sA)) : desc_lo(smem_addr(sA));
+        const uint32_t b_lo = BMN ? desc_lo_mn(smem_addr(sB)) : desc_lo(smem_addr(sB));
+        auto wait = [&](uint64_t *bar, uint32_t parity) {
+            return __all_sync(0xffffffffu, mbar_wait_bounded(bar, parity, e.err));
+        };
+        uint32_t s = 0, ph = 0, tc = 0, loads = 0, cur_u = 0xFFFFFFFFu;
+        bool ok = true;
+        for (uint32_t t = t_begin; t < t_end && ok; ++t, ++tc) {
+            const uint32_t u = t / n_tiles;
+            if (RESA && u != cur_u) {
+                if (!(ok = wait(a_full, loads & 1))) break;
+                cur_u = u;
+                ++loads;
+            }
+            const uint32_t buf = tc & 1, use = tc >> 1;
+            if (!(ok = wait(&acc_empty[buf], (use & 1) ^ 1))) break;
+            const uint32_t acc = tmem + buf * NT;
+            for (uint32_t kb = 0; kb < nkb; ++kb) {
+                if (!(ok = wait(&full[s], ph))) break;
                 tc_fence_after();
-                const uint32_t acc = tmem + buf * BN;
-                for (uint32_t kb = 0; kb < nkb; ++kb, ++it) {
-                    const uint32_t s = it % STAGES, ph = (it / STAGES) & 1;
-                    if (!(ok = mbar_wait_bounded(&full[s], ph, e.err))) break;
-                    tc_fence_after();
-                    const uint32_t a0 = smem_addr(sA + s * TILE_A), b0 = smem_addr(sB + s * TILE_B);
+                const uint32_t aa = a_lo + (RESA ? kb : s) * (TILE_A >> 4), bb = b_lo + s * (TILE_N >> 4);
+                if (elect_one()) {
+                    if (kb == 0) mma_f16kind_lo<false>(acc, aa, bb, idesc);
+                    else mma_f16kind_lo<true>(acc, aa, bb, idesc);
 #pragma unroll
-                    for (uint32_t k = 0; k < BK / 16; ++k)
-                        mma_f16kind(acc, desc_sw128(a0 + k * 32), desc_sw128(b0 + k * 32), idesc, (kb | k) != 0);
-                    mma_commit(&empty[s]);
+                    for (uint32_t k = 1; k < BK / 16; ++k)
+                        mma_f16kind_lo<true>(acc, aa + a_step * k, bb + b_step * k, idesc);
+                    if (MC) mma_commit_mc(&empty[s], (uint16_t)3);   // frees the stage in both CTAs
+                    else mma_commit(&empty[s]);
+                    if (kb + 1 == nkb) {
+                        mma_commit(&acc_full[buf]);
+                        // the last tile of this row block: A may be replaced
+                        // once these MMAs are done
+                        if (RESA && t + 1 < t_end && (t + 1) / n_tiles != u) mma_commit(a_empty);
+                    }
                 }
-                mma_commit(&acc_full[buf]);
+                __syncwarp();
+                if (++s == NST) { s = 0; ph ^= 1; }
             }
         }
     } else {
@@ -526,7 +566,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
             const bool ok = __all_sync(0xffffffffu, mbar_wait_bounded(&acc_full[buf], use & 1, e.err));
             if (!ok) break;
             tc_fence_after();
-            const uint32_t u = t / n_tiles, n0 = (t % n_tiles) * BN;
+            const uint32_t u = t / n_tiles, n0 = (t % n_tiles) * NT;
             const uint32_t m = rb_of_unit(u) * BM + q * 32 + lane;
             if (EPI == EPI_TOPP && u != cur_u) {
                 // a new row block: the previous one's partial is complete
@@ -537,18 +577,18 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
                 tp.reset();
                 cur_u = u;
             }
-            // the warp's two 32-column chunks of the tile in one round of
+            // the warp's two 32-column chunks (one, narrow tiles) in one round of
             // accumulator loads; the accumulator is released to the MMA
             // warp before the epilogue arithmetic
             // (the chunks' bias loads are in flight meanwhile)
-            static_assert(BN / 2 == 64, "two 32-column chunks per epilogue warp and tile");
-            const uint32_t nb = n0 + h * (BN / 2);
+            const uint32_t nb = n0 + h * (NT / 2);
             float v0[32], v1[32], bias0[32], bias1[32];
             load_bias32<EPI>(e, nb, N, bias0);
-            load_bias32<EPI>(e, nb + 32, N, bias1);
+            if (NT == 128) load_bias32<EPI>(e, nb + 32, N, bias1);
             __syncwarp();
-            const uint32_t ta = tmem + buf * BN + ((q * 32u) << 16) + h * (BN / 2);
-            tmem_ld32x2(ta, ta + 32, v0, v1);
+            const uint32_t ta = tmem + buf * NT + ((q * 32u) << 16) + h * (NT / 2);
+            if (NT == 128) tmem_ld32x2(ta, ta + 32, v0, v1);
+            else tmem_ld32(ta, v0);
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(&acc_empty[buf]);
@@ -556,7 +596,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
                 topp_pair(v0, v1, bias0, bias1, m, M, nb, N, tp, xs_all + (threadIdx.x - 64) * XS_STRIDE);
             } else {
                 epilogue_chunk<EPI>(v0, bias0, m, M, nb, N, e);
-                epilogue_chunk<EPI>(v1, bias1, m, M, nb + 32, N, e);
+                if (NT == 128) epilogue_chunk<EPI>(v1, bias1, m, M, nb + 32, N, e);
             }
         }
         if (EPI == EPI_TOPP && cur_u != 0xFFFFFFFFu) {
@@ -570,7 +610,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
     // its barriers
     if (MC) cluster_sync_all();
     if (warp == 1) {
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"((uint32_t)(2 * BN))
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"((uint32_t)(2 * NT))
                      : "memory");
     }
 }
@@ -582,78 +622,74 @@ __global__ void to_bf16_kernel(const float *__restrict__ x, __nv_bfloat16 *__res
         y[i] = __float2bfloat16_rn(x[i]);
 }
 
-// Queries (rows x d) to the first GEMM's BF16 operand, standardised per
-// dimension on the way: (x - mean) * inv_std, each step rounded in FP32
-// (mean 0 and inv_std 1, the defaults, leave x unchanged).
-__global__ void input_bf16_kernel(const float *__restrict__ x, const float *__restrict__ mean,
-                                  const float *__restrict__ inv_std, __nv_bfloat16 *__restrict__ y, size_t rows,
-                                  uint32_t d)
+// Queries (rows x d, rows perm[r] if given) to the first GEMM's BF16 operand,
+// standardised per dimension on the way: (x - mean) * inv_std, each step
+// rounded in FP32 (mean 0 and inv_std 1, the defaults, leave x unchanged).
+__global__ void input_bf16_kernel(const float *__restrict__ x, const uint32_t *__restrict__ perm,
+                                  const float *__restrict__ mean, const float *__restrict__ inv_std,
+                                  __nv_bfloat16 *__restrict__ y, size_t rows, uint32_t d)
 {
     const size_t n = rows * d;
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-        const uint32_t c = (uint32_t)(i % d);
-        y[i] = __float2bfloat16_rn(__fmul_rn(__fsub_rn(x[i], mean[c]), inv_std[c]));
+        const size_t r = i / d;
+        const uint32_t c = (uint32_t)(i - r * d);
+        const float v = x[(perm ? (size_t)perm[r] : r) * d + c];
+        y[i] = __float2bfloat16_rn(__fmul_rn(__fsub_rn(v, mean[c]), inv_std[c]));
     }
 }
 
-// out (C x R) = in (R x C)^T, BF16, 32 x 32 tiles through shared memory
-__global__ void transpose_bf16_kernel(const __nv_bfloat16 *__restrict__ in, __nv_bfloat16 *__restrict__ out,
-                                      uint32_t R, uint32_t C)
+// Column sums of an R x C FP32 matrix, each column's rows added in order
+// (deterministic, and the bias gradients' definition). A block takes 32
+// columns: all warps stage chunks of rows by asynchronous copies, three chunks
+// ahead, and the first adds, a column per lane. Bound by the chain of R
+// additions (1,024 rows: some 4,500 clocks); a thread per column reading
+// global memory took 45 us.
+constexpr uint32_t kSumRows = 64, kSumCols = 32, kSumBufs = 4;
+__global__ void __launch_bounds__(256) colsum_kernel(const float *__restrict__ g, float *__restrict__ out, uint32_t R,
+                                                     uint32_t C)
 {
-    __shared__ __nv_bfloat16 t[32][33];
-    const uint32_t c0 = blockIdx.x * 32, r0 = blockIdx.y * 32;
-    for (uint32_t i = threadIdx.y; i < 32; i += blockDim.y) {
-        const uint32_t r = r0 + i, c = c0 + threadIdx.x;
-        if (r < R && c < C) t[i][threadIdx.x] = in[(size_t)r * C + c];
-    }
-    __syncthreads();
-    for (uint32_t i = threadIdx.y; i < 32; i += blockDim.y) {
-        const uint32_t c = c0 + i, r = r0 + threadIdx.x;
-        if (r < R && c < C) out[(size_t)c * R + r] = t[threadIdx.x][i];
-    }
-}
-
-// g' = g * [mask > 0] (mask optional), as BF16 (optional) and BF16^T (optional)
-__global__ void post_grad_kernel(const float *__restrict__ g, const __nv_bfloat16 *__restrict__ mask,
-                                 float *__restrict__ gm, __nv_bfloat16 *__restrict__ gb,
-                                 __nv_bfloat16 *__restrict__ gT, uint32_t R, uint32_t C)
-{
-    __shared__ __nv_bfloat16 t[32][33];
-    const uint32_t c0 = blockIdx.x * 32, r0 = blockIdx.y * 32;
-    for (uint32_t i = threadIdx.y; i < 32; i += blockDim.y) {
-        const uint32_t r = r0 + i, c = c0 + threadIdx.x;
-        if (r < R && c < C) {
-            const size_t at = (size_t)r * C + c;
-            float v = g[at];
-            if (mask && !(__bfloat162float(mask[at]) > 0.0f)) v = 0.0f;
-            if (gm) gm[at] = v;
-            const __nv_bfloat16 b = __float2bfloat16_rn(v);
-            if (gb) gb[at] = b;
-            t[i][threadIdx.x] = b;
-        }
-    }
-    if (!gT) return;
-    __syncthreads();
-    for (uint32_t i = threadIdx.y; i < 32; i += blockDim.y) {
-        const uint32_t c = c0 + i, r = r0 + threadIdx.x;
-        if (r < R && c < C) gT[(size_t)c * R + r] = t[threadIdx.x][i];
-    }
-}
-
-// Column sums of an R x C FP32 matrix, rows in order (deterministic).
-__global__ void colsum_kernel(const float *__restrict__ g, float *__restrict__ out, uint32_t R, uint32_t C)
-{
-    const uint32_t c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= C) return;
+    __shared__ __align__(16) float buf[kSumBufs][kSumRows][kSumCols];
+    const uint32_t c0 = blockIdx.x * kSumCols, chunks = (R + kSumRows - 1) / kSumRows;
+    auto load = [&](uint32_t k) {
+        // 8 16-byte pieces a row; C is a multiple of 8, so a piece is all in or all out
+        if (k < chunks)
+            for (uint32_t i = threadIdx.x; i < kSumRows * (kSumCols / 4); i += blockDim.x) {
+                const uint32_t r = i / (kSumCols / 4), c = i % (kSumCols / 4) * 4, row = k * kSumRows + r;
+                if (row < R && c0 + c < C)
+                    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_addr(&buf[k % kSumBufs][r][c])),
+                                 "l"(g + (size_t)row * C + c0 + c)
+                                 : "memory");
+            }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
     float s = 0.0f;
-    for (uint32_t r = 0; r < R; ++r) s += g[(size_t)r * C + c];
-    out[c] = s;
+    for (uint32_t k = 0; k + 1 < kSumBufs; ++k) load(k);
+    for (uint32_t k = 0; k < chunks; ++k) {
+        load(k + kSumBufs - 1);   // into the buffer read in the last pass
+        asm volatile("cp.async.wait_group %0;" ::"n"(kSumBufs - 1) : "memory");
+        __syncthreads();
+        if (threadIdx.x < 32) {
+            const float *col = &buf[k % kSumBufs][0][threadIdx.x];
+            const uint32_t rows = min(kSumRows, R - k * kSumRows);
+            if (rows == kSumRows) {   // unrolled, so that the reads run ahead of the additions
+#pragma unroll
+                for (uint32_t r = 0; r < kSumRows; ++r) s += col[r * kSumCols];
+            } else {
+                for (uint32_t r = 0; r < rows; ++r) s += col[r * kSumCols];
+            }
+        }
+        __syncthreads();
+    }
+    if (threadIdx.x < 32 && c0 + threadIdx.x < C) out[c0 + threadIdx.x] = s;
 }
 
 // Row-wise softmax cross-entropy over z (B x N): z <- (softmax(z) - onehot(y)) / B,
-// loss += mean_i(logsumexp(z_i) - z_i[y_i]). One warp per row.
-__global__ void softmax_ce_kernel(float *__restrict__ z, const uint32_t *__restrict__ y, uint32_t B, uint32_t N,
-                                  float *__restrict__ loss)
+// loss += mean_i(logsumexp(z_i) - z_i[y_i]); zb <- z in BF16. The labels are
+// y[perm[r]] if perm is given. One warp per row: rows too long for the
+// block's kernel below.
+__global__ void softmax_ce_kernel(float *__restrict__ z, __nv_bfloat16 *__restrict__ zb,
+                                  const uint32_t *__restrict__ y, const uint32_t *__restrict__ perm, uint32_t B,
+                                  uint32_t N, float *__restrict__ loss)
 {
     const uint32_t lane = threadIdx.x & 31;
     const uint32_t r = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
@@ -666,11 +702,81 @@ __global__ void softmax_ce_kernel(float *__restrict__ z, const uint32_t *__restr
     for (uint32_t c = lane; c < N; c += 32) s += expf(zr[c] - mx);
     for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     const float lse = mx + logf(s);
-    const uint32_t yr = y[r];
+    const uint32_t yr = y[perm ? perm[r] : r];
     const float zy = zr[yr];
     const float inv = 1.0f / (float)B;
-    for (uint32_t c = lane; c < N; c += 32) zr[c] = (expf(zr[c] - lse) - (c == yr ? 1.0f : 0.0f)) * inv;
+    for (uint32_t c = lane; c < N; c += 32) {
+        const float v = (expf(zr[c] - lse) - (c == yr ? 1.0f : 0.0f)) * inv;
+        zr[c] = v;
+        zb[(size_t)r * N + c] = __float2bfloat16_rn(v);
+    }
     if (lane == 0) atomicAdd(loss, (lse - zy) * inv);
+}
+
+// The same with a block per row and the row's exponentials in shared memory:
+// they are formed by all threads, and the first warp adds them as above (lane
+// l the columns l, l + 32, ... in order, then the lanes by halves), so the sum
+// is the same. 1,024 rows of 10,000: a warp per row 53 us, most of it the chain
+// of loads, exponentials and additions.
+__global__ void __launch_bounds__(256) softmax_ce_block_kernel(float *__restrict__ z, __nv_bfloat16 *__restrict__ zb,
+                                                               const uint32_t *__restrict__ y,
+                                                               const uint32_t *__restrict__ perm, uint32_t B,
+                                                               uint32_t N, float *__restrict__ loss)
+{
+    extern __shared__ __align__(16) float ex[];
+    __shared__ float red[8], stat;
+    const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5, r = blockIdx.x;
+    float *zr = z + (size_t)r * N;
+    float mx = -INFINITY;
+    for (uint32_t c = threadIdx.x * 4; c < N; c += 1024) {   // N is a multiple of 8
+        const float4 v = *reinterpret_cast<const float4 *>(zr + c);
+        *reinterpret_cast<float4 *>(ex + c) = v;
+        mx = fmaxf(mx, fmaxf(fmaxf(v.x, v.y), fmaxf(v.z, v.w)));
+    }
+    for (int o = 16; o; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    if (lane == 0) red[warp] = mx;
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < 8; ++k) mx = fmaxf(mx, red[k]);
+    const uint32_t yr = y[perm ? perm[r] : r];
+    const float zy = ex[yr];
+    __syncthreads();
+    for (uint32_t c = threadIdx.x * 4; c < N; c += 1024) {
+        float4 v = *reinterpret_cast<const float4 *>(ex + c);
+        v.x = expf(v.x - mx);
+        v.y = expf(v.y - mx);
+        v.z = expf(v.z - mx);
+        v.w = expf(v.w - mx);
+        *reinterpret_cast<float4 *>(ex + c) = v;
+    }
+    __syncthreads();
+    const float inv = 1.0f / (float)B;
+    if (warp == 0) {
+        float s = 0.0f;
+#pragma unroll 8
+        for (uint32_t c = lane; c < N; c += 32) s += ex[c];
+        for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        const float lse = mx + logf(s);
+        if (lane == 0) {
+            stat = lse;
+            atomicAdd(loss, (lse - zy) * inv);
+        }
+    }
+    __syncthreads();
+    const float lse = stat;
+    for (uint32_t c = threadIdx.x * 4; c < N; c += 1024) {
+        float4 v = *reinterpret_cast<const float4 *>(zr + c);
+        v.x = (expf(v.x - lse) - (c == yr ? 1.0f : 0.0f)) * inv;
+        v.y = (expf(v.y - lse) - (c + 1 == yr ? 1.0f : 0.0f)) * inv;
+        v.z = (expf(v.z - lse) - (c + 2 == yr ? 1.0f : 0.0f)) * inv;
+        v.w = (expf(v.w - lse) - (c + 3 == yr ? 1.0f : 0.0f)) * inv;
+        *reinterpret_cast<float4 *>(zr + c) = v;
+        const __nv_bfloat162 lo = __floats2bfloat162_rn(v.x, v.y), hi = __floats2bfloat162_rn(v.z, v.w);
+        uint2 o;
+        o.x = *reinterpret_cast<const uint32_t *>(&lo);
+        o.y = *reinterpret_cast<const uint32_t *>(&hi);
+        *reinterpret_cast<uint2 *>(zb + (size_t)r * N + c) = o;
+    }
 }
 
 struct AdamHP {
@@ -678,18 +784,52 @@ struct AdamHP {
 };
 
 // AdamW (decoupled weight decay) on FP32 masters; refreshes the BF16 copy.
-__global__ void adamw_kernel(float *__restrict__ w, const float *__restrict__ g, float *__restrict__ m,
-                             float *__restrict__ v, __nv_bfloat16 *__restrict__ wb, size_t n, AdamHP h)
+// All six parameter arrays in one launch, four elements a thread (every array's
+// size is a multiple of 8): one pass over 30 bytes a parameter.
+struct AdamArray {
+    float *w, *m, *v;
+    const float *g;
+    __nv_bfloat16 *wb;   // or NULL
+};
+struct AdamArrays {
+    AdamArray a[6];
+    size_t end[6];       // running element counts
+};
+
+__global__ void __launch_bounds__(256) adamw_kernel(const AdamArrays p, AdamHP h)
 {
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-        const float gi = g[i];
-        const float mi = h.b1 * m[i] + (1.0f - h.b1) * gi;
-        const float vi = h.b2 * v[i] + (1.0f - h.b2) * gi * gi;
-        m[i] = mi;
-        v[i] = vi;
-        const float wi = w[i] - h.lr * ((mi / h.c1) / (sqrtf(vi / h.c2) + h.eps) + h.wd * w[i]);
-        w[i] = wi;
-        if (wb) wb[i] = __float2bfloat16_rn(wi);
+    const size_t n = p.end[5];
+    for (size_t i = (blockIdx.x * (size_t)blockDim.x + threadIdx.x) * 4; i < n;
+         i += (size_t)gridDim.x * blockDim.x * 4) {
+        int k = 0;
+#pragma unroll
+        for (int j = 0; j < 5; ++j) k += i >= p.end[j] ? 1 : 0;
+        const AdamArray &a = p.a[k];
+        const size_t at = i - (k ? p.end[k - 1] : 0);
+        const float4 g4 = *reinterpret_cast<const float4 *>(a.g + at);
+        float4 w4 = *reinterpret_cast<const float4 *>(a.w + at), m4 = *reinterpret_cast<const float4 *>(a.m + at);
+        float4 v4 = *reinterpret_cast<const float4 *>(a.v + at);
+        auto one = [&](float &w, float &m, float &v, float gi) {
+            const float mi = h.b1 * m + (1.0f - h.b1) * gi;
+            const float vi = h.b2 * v + (1.0f - h.b2) * gi * gi;
+            m = mi;
+            v = vi;
+            w = w - h.lr * ((mi / h.c1) / (sqrtf(vi / h.c2) + h.eps) + h.wd * w);
+        };
+        one(w4.x, m4.x, v4.x, g4.x);
+        one(w4.y, m4.y, v4.y, g4.y);
+        one(w4.z, m4.z, v4.z, g4.z);
+        one(w4.w, m4.w, v4.w, g4.w);
+        *reinterpret_cast<float4 *>(a.w + at) = w4;
+        *reinterpret_cast<float4 *>(a.m + at) = m4;
+        *reinterpret_cast<float4 *>(a.v + at) = v4;
+        if (a.wb) {
+            const __nv_bfloat162 lo = __floats2bfloat162_rn(w4.x, w4.y), hi = __floats2bfloat162_rn(w4.z, w4.w);
+            uint2 o;
+            o.x = *reinterpret_cast<const uint32_t *>(&lo);
+            o.y = *reinterpret_cast<const uint32_t *>(&hi);
+            *reinterpret_cast<uint2 *>(a.wb + at) = o;
+        }
     }
 }
 
@@ -780,18 +920,6 @@ __global__ void topp_merge_kernel(const float *__restrict__ part, uint32_t M, ui
         if (pmax) pmax[r] = pm;
         if (pm < tau) seeds[(size_t)r * P] = ANN_INVALID_ID;
     }
-}
-
-// Rows perm[0, n) of x (and their labels) into contiguous batch buffers.
-__global__ void gather_batch_kernel(const float *__restrict__ x, const uint32_t *__restrict__ y,
-                                    const uint32_t *__restrict__ perm, uint32_t n, uint32_t d,
-                                    float *__restrict__ xb, uint32_t *__restrict__ yb)
-{
-    const uint32_t r = blockIdx.x;
-    if (r >= n) return;
-    const uint32_t src = perm[r];
-    for (uint32_t c = threadIdx.x; c < d; c += blockDim.x) xb[(size_t)r * d + c] = x[(size_t)src * d + c];
-    if (threadIdx.x == 0) yb[r] = y[src];
 }
 
 __global__ void accumulate_kernel(float *__restrict__ acc, const float *__restrict__ v, float w)
@@ -922,13 +1050,13 @@ struct ann_mlp {
     int device = 0;
     uint32_t d = 0, h1 = 0, h2 = 0, out = 0, maxb = 0;
     float *W[3] = {}, *b[3] = {}, *mW[3] = {}, *vW[3] = {}, *mb[3] = {}, *vb[3] = {}, *gW[3] = {}, *gb[3] = {};
-    __nv_bfloat16 *Wb[3] = {}, *WT[3] = {};
-    __nv_bfloat16 *xb = nullptr, *xT = nullptr, *h1b = nullptr, *h1T = nullptr, *h2b = nullptr, *h2T = nullptr;
-    __nv_bfloat16 *dzb = nullptr, *dzT = nullptr, *da2b = nullptr, *da2T = nullptr, *da1T = nullptr;
-    float *z = nullptr, *dh = nullptr, *dm = nullptr, *loss = nullptr, *part = nullptr;
-    float *xbat = nullptr, *epoch_loss = nullptr;
+    __nv_bfloat16 *Wb[3] = {};
+    __nv_bfloat16 *xb = nullptr, *h1b = nullptr, *h2b = nullptr;
+    __nv_bfloat16 *dzb = nullptr, *dab = nullptr;   // logit and hidden gradients
+    float *z = nullptr, *da = nullptr, *loss = nullptr, *part = nullptr;
+    float *epoch_loss = nullptr;
     float *mean = nullptr, *inv_std = nullptr;   // input standardisation (in_dim each)
-    uint32_t *ybat = nullptr, *perm = nullptr;
+    uint32_t *perm = nullptr;
     size_t perm_cap = 0;
     uint32_t train_cap = 0;
     size_t part_cap = 0;
@@ -1019,7 +1147,8 @@ uint32_t pair_slots(uint32_t sms)
     return cached;
 }
 
-template <int EPI>
+// C = A * B^T; AMN / BMN: A is given as K x M, B as K x N.
+template <int EPI, bool AMN = false, bool BMN = false>
 ann_status gemm(const __nv_bfloat16 *A, const __nv_bfloat16 *B, uint32_t M, uint32_t N, uint32_t K, EpiArgs e,
                 cudaStream_t st)
 {
@@ -1030,41 +1159,56 @@ ann_status gemm(const __nv_bfloat16 *A, const __nv_bfloat16 *B, uint32_t M, uint
     }
     const int mode = gemm_mode(EPI, K);
     CUtensorMap ta, tb;
-    ann_status s = make_map(&ta, A, M, K);
-    if (s == ANN_OK) s = make_map(&tb, B, N, K, mode == 2 ? BN / 2 : 128);
-    if (s != ANN_OK) return s;
-    static bool attr[3] = {false, false, false};
-    if (!attr[mode]) {
-        if (mode == 0)
-            ANN_CUDA(cudaFuncSetAttribute(gemm_kernel<EPI, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, GEMM_SMEM));
-        else if (mode == 1)
-            ANN_CUDA(cudaFuncSetAttribute(gemm_kernel<EPI, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, RES_SMEM));
-        else
-            ANN_CUDA(cudaFuncSetAttribute(gemm_kernel<EPI, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, RES_SMEM));
-        attr[mode] = true;
-    }
+    ann_status s = AMN ? make_map(&ta, A, K, M, 64) : make_map(&ta, A, M, K);
+    // Tiles of 64 columns where tiles of 128 would leave more than half of the
+    // SMs idle: the products of a training batch have 4 to 32 tiles (the hidden
+    // gradient 1,024 x 512 x 10,000 is a chain of 157 K blocks per tile).
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const bool narrow = EPI != EPI_TOPP && 2 * gemm_units(M, N, 0) <= (uint32_t)sms;
+    if (s == ANN_OK)
+        s = BMN ? make_map(&tb, B, K, N, 64) : make_map(&tb, B, N, K, mode == 2 ? BN / 2 : narrow ? 64 : 128);
+    if (s != ANN_OK) return s;
     const uint32_t grid = gemm_grid(M, N, (uint32_t)sms, mode);
-    if (mode == 0) {
-        gemm_kernel<EPI, 0><<<grid, GEMM_THREADS, GEMM_SMEM, st>>>(ta, tb, M, N, K, e);
-    } else if (mode == 1) {
-        gemm_kernel<EPI, 1><<<grid, GEMM_THREADS, RES_SMEM, st>>>(ta, tb, M, N, K, e);
-    } else {
-        cudaLaunchConfig_t cfg{};
-        cfg.gridDim = dim3(grid);
-        cfg.blockDim = dim3(GEMM_THREADS);
-        cfg.dynamicSmemBytes = RES_SMEM;
-        cfg.stream = st;
-        cudaLaunchAttribute at[1];
-        at[0].id = cudaLaunchAttributeClusterDimension;
-        at[0].val.clusterDim.x = 2;
-        at[0].val.clusterDim.y = 1;
-        at[0].val.clusterDim.z = 1;
-        cfg.attrs = at;
-        cfg.numAttrs = 1;
-        ANN_CUDA(cudaLaunchKernelEx(&cfg, gemm_kernel<EPI, 2>, ta, tb, M, N, K, e));
+    static std::atomic<bool> attr[4];
+    const auto prepare = [&](const void *kernel, int smem, int which) {
+        if (attr[which].load(std::memory_order_relaxed)) return cudaSuccess;
+        const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        if (e == cudaSuccess) attr[which].store(true, std::memory_order_relaxed);
+        return e;
+    };
+    if (narrow) {
+        if constexpr (EPI != EPI_TOPP) {
+            constexpr int smem = ring_smem(EPI, 64);
+            ANN_CUDA(prepare((const void *)gemm_kernel<EPI, 0, AMN, BMN, 64>, smem, 3));
+            const uint32_t tiles = (N + 63) / 64 * ((M + BM - 1) / BM);
+            gemm_kernel<EPI, 0, AMN, BMN, 64><<<std::min(tiles, (uint32_t)sms), GEMM_THREADS, smem, st>>>(ta, tb, M, N, K, e);
+        }
+    } else if (mode == 0) {
+        constexpr int smem = ring_smem(EPI, BN);
+        ANN_CUDA(prepare((const void *)gemm_kernel<EPI, 0, AMN, BMN>, smem, 0));
+        gemm_kernel<EPI, 0, AMN, BMN><<<grid, GEMM_THREADS, smem, st>>>(ta, tb, M, N, K, e);
+    } else if constexpr (EPI == EPI_TOPP) {
+        if (mode == 1) {
+            ANN_CUDA(prepare((const void *)gemm_kernel<EPI, 1>, RES_SMEM, 1));
+            gemm_kernel<EPI, 1><<<grid, GEMM_THREADS, RES_SMEM, st>>>(ta, tb, M, N, K, e);
+        } else {
+            ANN_CUDA(prepare((const void *)gemm_kernel<EPI, 2>, RES_SMEM, 2));
+            cudaLaunchConfig_t cfg{};
+            cfg.gridDim = dim3(grid);
+            cfg.blockDim = dim3(GEMM_THREADS);
+            cfg.dynamicSmemBytes = RES_SMEM;
+            cfg.stream = st;
+            cudaLaunchAttribute at[1];
+            at[0].id = cudaLaunchAttributeClusterDimension;
+            at[0].val.clusterDim.x = 2;
+            at[0].val.clusterDim.y = 1;
+            at[0].val.clusterDim.z = 1;
+            cfg.attrs = at;
+            cfg.numAttrs = 1;
+            ANN_CUDA(cudaLaunchKernelEx(&cfg, gemm_kernel<EPI, 2>, ta, tb, M, N, K, e));
+        }
     }
     ANN_CUDA(cudaGetLastError());
     return ANN_OK;
@@ -1072,49 +1216,29 @@ ann_status gemm(const __nv_bfloat16 *A, const __nv_bfloat16 *B, uint32_t M, uint
 
 int grid1d(size_t n, int num_sms) { return (int)std::min<size_t>((n + 255) / 256, (size_t)num_sms * 8); }
 
-ann_status transpose(const __nv_bfloat16 *in, __nv_bfloat16 *out, uint32_t R, uint32_t C, cudaStream_t st)
-{
-    dim3 grid((C + 31) / 32, (R + 31) / 32), block(32, 8);
-    transpose_bf16_kernel<<<grid, block, 0, st>>>(in, out, R, C);
-    ANN_CUDA(cudaGetLastError());
-    return ANN_OK;
-}
-
 // Training-only buffers for batches of up to train_cap rows (grown once).
 ann_status ensure_train_buffers(ann_mlp *m, uint32_t n)
 {
     if (n <= m->train_cap) return ANN_OK;
-    __nv_bfloat16 **bf[] = {&m->xT, &m->h1T, &m->h2T, &m->dzb, &m->dzT, &m->da2b, &m->da2T, &m->da1T};
-    float **fp[] = {&m->z, &m->dh, &m->dm, &m->xbat};
-    for (auto p : bf) if (*p) { cudaFree(*p); *p = nullptr; }
-    for (auto p : fp) if (*p) { cudaFree(*p); *p = nullptr; }
-    if (m->ybat) { cudaFree(m->ybat); m->ybat = nullptr; }
+    for (void **p : {(void **)&m->dzb, (void **)&m->dab, (void **)&m->z, (void **)&m->da})
+        if (*p) { cudaFree(*p); *p = nullptr; }
     m->train_cap = 0;
-    const size_t B = n;
+    const size_t B = n, h = std::max(m->h1, m->h2);
     cudaError_t e = cudaSuccess;
     auto al = [&](void **p, size_t bytes) { if (e == cudaSuccess) e = cudaMalloc(p, bytes); };
-    al((void **)&m->xT, B * m->d * 2);
-    al((void **)&m->h1T, B * m->h1 * 2);
-    al((void **)&m->h2T, B * m->h2 * 2);
     al((void **)&m->dzb, B * m->out * 2);
-    al((void **)&m->dzT, B * m->out * 2);
-    al((void **)&m->da2b, B * m->h2 * 2);
-    al((void **)&m->da2T, B * m->h2 * 2);
-    al((void **)&m->da1T, B * m->h1 * 2);
+    al((void **)&m->dab, B * (m->h1 + m->h2) * 2);
     al((void **)&m->z, B * m->out * 4);
-    al((void **)&m->dh, B * std::max(m->h1, m->h2) * 4);
-    al((void **)&m->dm, B * std::max(m->h1, m->h2) * 4);
-    al((void **)&m->xbat, B * m->d * 4);
-    al((void **)&m->ybat, B * 4);
+    al((void **)&m->da, B * h * 4);
     if (e != cudaSuccess) return cuda_fail(e, "MLP training buffers");
     m->train_cap = n;
     return ANN_OK;
 }
 
-ann_status forward(ann_mlp *m, const float *x, uint32_t n, cudaStream_t st, int logits_epi, float *logits,
-                   float *part, uint32_t ntiles)
+ann_status forward(ann_mlp *m, const float *x, const uint32_t *perm, uint32_t n, cudaStream_t st, int logits_epi,
+                   float *logits, float *part, uint32_t ntiles)
 {
-    input_bf16_kernel<<<grid1d((size_t)n * m->d, m->num_sms), 256, 0, st>>>(x, m->mean, m->inv_std, m->xb, n, m->d);
+    input_bf16_kernel<<<grid1d((size_t)n * m->d, m->num_sms), 256, 0, st>>>(x, perm, m->mean, m->inv_std, m->xb, n, m->d);
     ANN_CUDA(cudaGetLastError());
     EpiArgs e{};
     e.err = m->d_error;
@@ -1133,15 +1257,76 @@ ann_status forward(ann_mlp *m, const float *x, uint32_t n, cudaStream_t st, int 
     return gemm<EPI_TOPP>(m->h2b, m->Wb[2], n, m->out, m->h2, e, st);
 }
 
+// One AdamW step on the minibatch of rows perm[0, n) (or 0 .. n - 1) of x and
+// their labels; the mean loss goes to m->loss. Gradient products read the
+// forward pass's matrices as they lie (MN-major operands where the product is
+// with a transpose), and the hidden gradients are masked, and rounded to BF16
+// for the next product, as they leave the accumulator.
+ann_status train_step(ann_mlp *m, const float *x, const uint32_t *labels, const uint32_t *perm, uint32_t n, float lr,
+                      float beta1, float beta2, float eps, float weight_decay, cudaStream_t st)
+{
+    ann_status s = ensure_train_buffers(m, n);
+    if (s != ANN_OK) return s;
+    ANN_CUDA(cudaMemsetAsync(m->loss, 0, 4, st));
+    s = forward(m, x, perm, n, st, EPI_BIAS_F32, m->z, nullptr, 0);
+    if (s != ANN_OK) return s;
+    // logits' gradient, FP32 in z and BF16
+    constexpr size_t kRowMax = 200 * 1024;
+    const size_t row = (size_t)m->out * 4;
+    if (row <= kRowMax) {
+        ANN_CUDA(cudaFuncSetAttribute(softmax_ce_block_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)row));
+        softmax_ce_block_kernel<<<n, 256, row, st>>>(m->z, m->dzb, labels, perm, n, m->out, m->loss);
+    } else {
+        softmax_ce_kernel<<<(n + 7) / 8, 256, 0, st>>>(m->z, m->dzb, labels, perm, n, m->out, m->loss);
+    }
+    ANN_CUDA(cudaGetLastError());
+    auto colsum = [&](const float *g, float *out, uint32_t C) {
+        colsum_kernel<<<(C + kSumCols - 1) / kSumCols, 256, 0, st>>>(g, out, n, C);
+    };
+    __nv_bfloat16 *da2 = m->dab, *da1 = m->dab + (size_t)n * m->h2;
+    EpiArgs e{};
+    e.err = m->d_error;
+    colsum(m->z, m->gb[2], m->out);
+    e.c = m->gW[2]; e.ldc = m->h2;
+    s = gemm<EPI_F32, true, true>(m->dzb, m->h2b, m->out, m->h2, n, e, st);
+    e.c = m->da; e.cb = da2; e.mask = m->h2b;
+    if (s == ANN_OK) s = gemm<EPI_MASK, false, true>(m->dzb, m->Wb[2], n, m->h2, m->out, e, st);
+    if (s != ANN_OK) return s;
+    colsum(m->da, m->gb[1], m->h2);
+    e.c = m->gW[1]; e.ldc = m->h1;
+    s = gemm<EPI_F32, true, true>(da2, m->h1b, m->h2, m->h1, n, e, st);
+    e.c = m->da; e.cb = da1; e.mask = m->h1b;
+    if (s == ANN_OK) s = gemm<EPI_MASK, false, true>(da2, m->Wb[1], n, m->h1, m->h2, e, st);
+    if (s != ANN_OK) return s;
+    colsum(m->da, m->gb[0], m->h1);
+    e.c = m->gW[0]; e.ldc = m->d;
+    s = gemm<EPI_F32, true, true>(da1, m->xb, m->h1, m->d, n, e, st);
+    if (s != ANN_OK) return s;
+    m->step++;
+    const AdamHP h{lr, beta1, beta2, eps, weight_decay, (float)(1.0 - std::pow((double)beta1, (double)m->step)),
+                   (float)(1.0 - std::pow((double)beta2, (double)m->step))};
+    const uint32_t rows[3] = {m->h1, m->h2, m->out}, cols[3] = {m->d, m->h1, m->h2};
+    AdamArrays p{};
+    size_t at = 0;
+    for (int l = 0; l < 3; ++l) {
+        p.a[2 * l] = AdamArray{m->W[l], m->mW[l], m->vW[l], m->gW[l], m->Wb[l]};
+        p.end[2 * l] = at += (size_t)rows[l] * cols[l];
+        p.a[2 * l + 1] = AdamArray{m->b[l], m->mb[l], m->vb[l], m->gb[l], nullptr};
+        p.end[2 * l + 1] = at += rows[l];
+    }
+    adamw_kernel<<<grid1d((at + 3) / 4, m->num_sms), 256, 0, st>>>(p, h);
+    ANN_CUDA(cudaGetLastError());
+    return ANN_OK;
+}
+
 void mlp_free_all(ann_mlp *m)
 {
     for (int l = 0; l < 3; ++l) {
-        void *p[] = {m->W[l], m->b[l], m->mW[l], m->vW[l], m->mb[l], m->vb[l], m->gW[l], m->gb[l], m->Wb[l], m->WT[l]};
+        void *p[] = {m->W[l], m->b[l], m->mW[l], m->vW[l], m->mb[l], m->vb[l], m->gW[l], m->gb[l], m->Wb[l]};
         for (void *x : p) if (x) cudaFree(x);
     }
-    void *q[] = {m->xb, m->xT, m->h1b, m->h1T, m->h2b, m->h2T, m->dzb, m->dzT, m->da2b, m->da2T, m->da1T,
-                 m->z, m->dh, m->dm, m->loss, m->part, m->d_error, m->xbat, m->ybat, m->perm, m->epoch_loss,
-                 m->mean, m->inv_std};
+    void *q[] = {m->xb, m->h1b, m->h2b, m->dzb, m->dab, m->z, m->da, m->loss, m->part, m->d_error, m->perm,
+                 m->epoch_loss, m->mean, m->inv_std};
     for (void *x : q) if (x) cudaFree(x);
 }
 
@@ -1179,7 +1364,7 @@ ann_status ann_mlp_create(int device, uint32_t in_dim, uint32_t hidden1, uint32_
     for (int l = 0; l < 3; ++l) {
         const size_t nw = (size_t)rows[l] * cols[l];
         al((void **)&m->W[l], nw * 4); al((void **)&m->mW[l], nw * 4); al((void **)&m->vW[l], nw * 4);
-        al((void **)&m->gW[l], nw * 4); al((void **)&m->Wb[l], nw * 2); al((void **)&m->WT[l], nw * 2);
+        al((void **)&m->gW[l], nw * 4); al((void **)&m->Wb[l], nw * 2);
         al((void **)&m->b[l], rows[l] * 4); al((void **)&m->mb[l], rows[l] * 4); al((void **)&m->vb[l], rows[l] * 4);
         al((void **)&m->gb[l], rows[l] * 4);
     }
@@ -1242,7 +1427,6 @@ ann_status ann_mlp_set_params(ann_mlp *m, const float *W1, const float *b1, cons
         if (e == cudaSuccess) e = cudaMemset(m->vb[l], 0, rows[l] * 4);
         if (e != cudaSuccess) { s = cuda_fail(e, "ann_mlp_set_params"); break; }
         to_bf16_kernel<<<grid1d(nw, m->num_sms), 256>>>(m->W[l], m->Wb[l], nw);
-        if (l > 0) s = transpose(m->Wb[l], m->WT[l], rows[l], cols[l], 0);
     }
     m->step = 0;
     cudaError_t e = cudaDeviceSynchronize();
@@ -1395,7 +1579,7 @@ ann_status ann_mlp_forward(ann_mlp *m, const float *x, uint32_t n, float *logits
         const ann_status ds = enter_device(m->device, &prev, "ann_mlp_forward");
         if (ds != ANN_OK) return ds;
     }
-    ann_status s = forward(m, x, n, (cudaStream_t)stream, EPI_BIAS_F32, logits, nullptr, 0);
+    ann_status s = forward(m, x, nullptr, n, (cudaStream_t)stream, EPI_BIAS_F32, logits, nullptr, 0);
     leave_device(m->device, prev);
     return s;
 }
@@ -1417,59 +1601,7 @@ ann_status ann_mlp_train_step(ann_mlp *m, const float *x, const uint32_t *labels
         if (ds != ANN_OK) return ds;
     }
     cudaStream_t st = (cudaStream_t)stream;
-    ann_status s = ensure_train_buffers(m, n);
-    auto chk = [&]() { cudaError_t e = cudaGetLastError(); if (e != cudaSuccess && s == ANN_OK) s = cuda_fail(e, "ann_mlp_train_step"); };
-    if (s == ANN_OK && cudaMemsetAsync(m->loss, 0, 4, st) != cudaSuccess) s = ANN_ECUDA;
-    if (s == ANN_OK) s = forward(m, x, n, st, EPI_BIAS_F32, m->z, nullptr, 0);
-    const dim3 tb(32, 8);
-    EpiArgs e{};
-    e.err = m->d_error;
-    if (s == ANN_OK) {
-        softmax_ce_kernel<<<(n + 7) / 8, 256, 0, st>>>(m->z, labels, n, m->out, m->loss);
-        chk();
-        post_grad_kernel<<<dim3((m->out + 31) / 32, (n + 31) / 32), tb, 0, st>>>(m->z, nullptr, nullptr, m->dzb, m->dzT, n, m->out);
-        chk();
-        colsum_kernel<<<(m->out + 255) / 256, 256, 0, st>>>(m->z, m->gb[2], n, m->out);
-        chk();
-    }
-    if (s == ANN_OK) s = transpose(m->h2b, m->h2T, n, m->h2, st);
-    e.c = m->gW[2]; e.ldc = m->h2;
-    if (s == ANN_OK) s = gemm<EPI_F32>(m->dzT, m->h2T, m->out, m->h2, n, e, st);
-    e.c = m->dh; e.ldc = m->h2;
-    if (s == ANN_OK) s = gemm<EPI_F32>(m->dzb, m->WT[2], n, m->h2, m->out, e, st);
-    if (s == ANN_OK) {
-        post_grad_kernel<<<dim3((m->h2 + 31) / 32, (n + 31) / 32), tb, 0, st>>>(m->dh, m->h2b, m->dm, m->da2b, m->da2T, n, m->h2);
-        chk();
-        colsum_kernel<<<(m->h2 + 255) / 256, 256, 0, st>>>(m->dm, m->gb[1], n, m->h2);
-        chk();
-    }
-    if (s == ANN_OK) s = transpose(m->h1b, m->h1T, n, m->h1, st);
-    e.c = m->gW[1]; e.ldc = m->h1;
-    if (s == ANN_OK) s = gemm<EPI_F32>(m->da2T, m->h1T, m->h2, m->h1, n, e, st);
-    e.c = m->dh; e.ldc = m->h1;
-    if (s == ANN_OK) s = gemm<EPI_F32>(m->da2b, m->WT[1], n, m->h1, m->h2, e, st);
-    if (s == ANN_OK) {
-        post_grad_kernel<<<dim3((m->h1 + 31) / 32, (n + 31) / 32), tb, 0, st>>>(m->dh, m->h1b, m->dm, nullptr, m->da1T, n, m->h1);
-        chk();
-        colsum_kernel<<<(m->h1 + 255) / 256, 256, 0, st>>>(m->dm, m->gb[0], n, m->h1);
-        chk();
-    }
-    if (s == ANN_OK) s = transpose(m->xb, m->xT, n, m->d, st);
-    e.c = m->gW[0]; e.ldc = m->d;
-    if (s == ANN_OK) s = gemm<EPI_F32>(m->da1T, m->xT, m->h1, m->d, n, e, st);
-    if (s == ANN_OK) {
-        m->step++;
-        AdamHP h{lr, beta1, beta2, eps, weight_decay, (float)(1.0 - std::pow((double)beta1, (double)m->step)),
-                 (float)(1.0 - std::pow((double)beta2, (double)m->step))};
-        const uint32_t rows[3] = {m->h1, m->h2, m->out}, cols[3] = {m->d, m->h1, m->h2};
-        for (int l = 0; l < 3; ++l) {
-            const size_t nw = (size_t)rows[l] * cols[l];
-            adamw_kernel<<<grid1d(nw, m->num_sms), 256, 0, st>>>(m->W[l], m->gW[l], m->mW[l], m->vW[l], m->Wb[l], nw, h);
-            adamw_kernel<<<grid1d(rows[l], m->num_sms), 256, 0, st>>>(m->b[l], m->gb[l], m->mb[l], m->vb[l], nullptr, rows[l], h);
-            chk();
-            if (l > 0 && s == ANN_OK) s = transpose(m->Wb[l], m->WT[l], rows[l], cols[l], st);
-        }
-    }
+    ann_status s = train_step(m, x, labels, nullptr, n, lr, beta1, beta2, eps, weight_decay, st);
     if (s == ANN_OK && loss_out) {
         cudaError_t ce = cudaMemcpyAsync(loss_out, m->loss, 4, cudaMemcpyDeviceToDevice, st);
         if (ce != cudaSuccess) s = cuda_fail(ce, "ann_mlp_train_step loss");
@@ -1512,7 +1644,7 @@ ann_status ann_mlp_predict(ann_mlp *m, const float *x, uint32_t n, uint32_t P, f
         // slots no CTA writes read as empty (ids 0xFFFFFFFF, exp-sum NaN)
         if (cudaError_t me = cudaMemsetAsync(m->part, 0xFF, need, st); me != cudaSuccess)
             s = cuda_fail(me, "ann_mlp_predict");
-        if (s == ANN_OK) s = forward(m, x + (size_t)r0 * m->d, rows, st, EPI_TOPP, nullptr, m->part, ntiles);
+        if (s == ANN_OK) s = forward(m, x + (size_t)r0 * m->d, nullptr, rows, st, EPI_TOPP, nullptr, m->part, ntiles);
         if (s == ANN_OK) {
             topp_merge_kernel<<<(rows + 3) / 4, 128, 0, st>>>(m->part, rows, ntiles, P, tau, seeds + (size_t)r0 * P,
                                                                pmax ? pmax + r0 : nullptr);
@@ -1569,10 +1701,7 @@ ann_status ann_mlp_train_epochs(ann_mlp *m, const float *x, const uint32_t *labe
         for (uint32_t b0 = 0; b0 + 8 <= n; b0 += batch) ++steps;
         for (uint32_t b0 = 0; b0 + 8 <= n && s == ANN_OK; b0 += batch) {
             uint32_t rows = std::min(batch, n - b0) & ~7u;
-            gather_batch_kernel<<<rows, 128, 0, st>>>(x, labels, m->perm + b0, rows, m->d, m->xbat, m->ybat);
-            e = cudaGetLastError();
-            if (e != cudaSuccess) { s = cuda_fail(e, "gather_batch_kernel"); break; }
-            s = ann_mlp_train_step(m, m->xbat, m->ybat, rows, lr, beta1, beta2, eps, weight_decay, nullptr, stream);
+            s = train_step(m, x, labels, m->perm + b0, rows, lr, beta1, beta2, eps, weight_decay, st);
             if (s == ANN_OK) accumulate_kernel<<<1, 32, 0, st>>>(m->epoch_loss + ep, m->loss, 1.0f / (float)steps);
         }
     }

@@ -57,6 +57,21 @@ __device__ __forceinline__ void mma_f16kind(uint32_t tmem_d, uint64_t da, uint64
         : "memory");
 }
 
+// desc_sw128's high word (both majors: 1,024 bytes between 8-row groups)
+constexpr uint32_t kDescHi = (1024u >> 4) | (1u << 14) | (2u << 29);
+
+// MN-major operands (the K index is the row of a row-major matrix): TMA boxes of
+// 64 elements x 64 rows in the 128-byte swizzle, 1,024 bytes per 8 rows (the
+// stride offset), the next 64 elements in the next box (the leading offset).
+// Stepping K by 16 rows adds 128 to the low word.
+constexpr uint32_t kBoxBytes = 64 * 64 * 2;
+__device__ __forceinline__ uint32_t desc_lo_mn(uint32_t saddr)
+{
+    return ((saddr & 0x3FFFFu) >> 4) | ((kBoxBytes >> 4) << 16);
+}
+// instruction-descriptor bits of an MN-major A or B
+constexpr uint32_t kIdescAMN = 1u << 15, kIdescBMN = 1u << 16;
+
 // True in one lane of a converged warp. The MMA warp's loop is run by all its
 // lanes and only the MMAs and commits are guarded by this: descriptors and
 // loop state then are warp-uniform, which the instructions' uniform-register
@@ -77,12 +92,11 @@ __device__ __forceinline__ uint32_t desc_lo(uint32_t saddr) { return ((saddr & 0
 template <bool ACC>
 __device__ __forceinline__ void mma_f16kind_lo(uint32_t tmem_d, uint32_t da, uint32_t db, uint32_t idesc)
 {
-    constexpr uint32_t hi = (1024u >> 4) | (1u << 14) | (2u << 29);   // desc_sw128's high word
     asm volatile(
         "{\n\t.reg .pred p;\n\t.reg .b64 a, b;\n\tsetp.ne.b32 p, %5, 0;\n\t"
         "mov.b64 a, {%1, %3};\n\tmov.b64 b, {%2, %3};\n\t"
         "tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %4, p;\n\t}" ::"r"(tmem_d),
-        "r"(da), "r"(db), "r"(hi), "r"(idesc), "n"(ACC ? 1 : 0)
+        "r"(da), "r"(db), "r"(kDescHi), "r"(idesc), "n"(ACC ? 1 : 0)
         : "memory");
 }
 
