@@ -158,8 +158,8 @@ ann_status ann_index_export(const ann_index *index, int which, void *host_dst, u
  *   stats        device, nq ann_query_stats, or NULL
  *   stream       cudaStream_t (NULL = legacy default stream)
  * Asynchronous on `stream`; returns after the launch. The launch shape is
- * chosen per call from the parameters (rows gathered per round: 16, or 8 of
- * rows over 1 KB, halved when that admits more resident warps per SM); the
+ * chosen per call from the parameters and nq (rows gathered per round: 16, or 8
+ * or 4 where the resident warps that this admits take the batch in fewer fillings); the
  * environment variable ANN_STAGE_ROWS fixes the rows per round instead (for
  * experiments). Results do not depend on the shape. */
 ann_status ann_search(ann_index *index, const float *queries, uint32_t nq, const ann_search_params *params,

@@ -20,10 +20,12 @@
 //   - the rows whose distances are needed (and the FP32 rerank rows) are 1-D
 //     TMA bulk copies into shared memory completing on the warp's mbarrier: one
 //     instruction per row, all rows of a round in flight together;
-//   - distances are computed by a lane pair per row from shared memory, one
-//     fused multiply-add per element into four interleaved partial sums, the
-//     same FP32 operations as the reference definition, so they agree bit
-//     for bit;
+//   - distances are computed by two or four lanes per row from shared memory,
+//     the query laid out so that a lane reads four of its elements at once (10,000
+//     queries, in index order / so: FP32 96-d 1,104 / 1,024 us, FP16 128-d with
+//     100 results 3,740 / 3,652), one fused multiply-add per element into four
+//     interleaved partial sums, the same FP32 operations as the reference
+//     definition, so they agree bit for bit;
 //   - DGS needs the query's sign bits relative to each parent; they are
 //     recomputed from the parent's row (one ballot per 32 dims);
 //   - DGS keeps its top n neighbours by a ballot radix select of the score
@@ -95,7 +97,8 @@ struct Args {
     uint32_t *vtab;
     uint32_t vbits, vstride_bits, slot_base;
     uint32_t gbm_words;   // > 0: the ghost stage's visited set is a bitmap of this many words
-    uint32_t lpr;         // lanes per staged row in the distance step: 2, or 4 for wide rows
+    uint32_t lpr;         // lanes per staged row in the distance step, 2 or 4 (plan_shape)
+    uint32_t q_part;      // floats between the parts of the query (query_part)
     // profile build only: per warp slot, ANN_PROFILE_STAGES x ANN_PROFILE_PHASES
     // cycle counters (slot_base + warp slot selects a row)
     unsigned long long *prof;
@@ -117,12 +120,12 @@ __device__ __forceinline__ void step2(float2 y, float2 x, float2 &acc)
 }
 
 // Half of the squared L2 between a staged row and the query (both in
-// shared memory). The distance keeps four partial sums, element i (in index
-// order) fused into sum i mod 4, and is (s0 + s1) + (s2 + s3); half h of the
-// lane pair of a row computes s_{2h} + s_{2h+1}, so one more add of the two
-// halves gives the distance and each lane does half the elements. The two
-// sums of a lane are one float2, updated with packed FP32 instructions. The
-// loops unroll by two only: with 24 warps per SM spread over the whole
+// shared memory; q: part h). The distance keeps four partial sums, element i
+// (in index order) fused into sum i mod 4, and is (s0 + s1) + (s2 + s3); half
+// h of the lane pair of a row computes s_{2h} + s_{2h+1}, so one more add of
+// the two halves gives the distance and each lane does half the elements. The
+// two sums of a lane are one float2, updated with packed FP32 instructions.
+// The loops unroll little: with 24 warps per SM spread over the whole
 // iteration, the kernel is bound by instruction fetch, and the compiler's
 // deeper unrolling cost 6% of throughput (measured on the 1M x 96 workload).
 template <int ST>
@@ -131,46 +134,53 @@ __device__ __forceinline__ float row_dist_half(const uint8_t *row, const float *
 {
     float2 s = make_float2(0.0f, 0.0f);  // s_{2h}, s_{2h+1}
     const float2 sc = make_float2(scale, scale), nsc = make_float2(-scale, -scale);
-    uint32_t i = 0;
+    const float4 *yp = reinterpret_cast<const float4 *>(q);
+    const uint32_t units = d / (ST == ANN_E4M3 ? 16 : 8);
     if (ST == ANN_F32) {
-#pragma unroll 2
-        for (; i + 4 <= d; i += 4) {
-            const float2 x = *reinterpret_cast<const float2 *>(row + (size_t)(i + 2 * h) * 4);
-            const float2 y = *reinterpret_cast<const float2 *>(q + i + 2 * h);
-            step2(y, x, s);
+        const float2 *xp = reinterpret_cast<const float2 *>(row) + h;
+#pragma unroll 4
+        for (uint32_t u = 0; u < units; ++u) {
+            const float4 y = yp[u];
+            const float2 x0 = xp[4 * u], x1 = xp[4 * u + 2];
+            step2(make_float2(y.x, y.y), x0, s);
+            step2(make_float2(y.z, y.w), x1, s);
         }
     } else if (ST == ANN_F16) {
+        const __half2 *xp = reinterpret_cast<const __half2 *>(row) + h;
 #pragma unroll 2
-        for (; i + 8 <= d; i += 8) {
-#pragma unroll
-            for (uint32_t g = 0; g < 2; ++g) {
-                const uint32_t e = i + 4 * g + 2 * h;
-                const __half2 hv = *reinterpret_cast<const __half2 *>(row + (size_t)e * 2);
-                const float2 y = *reinterpret_cast<const float2 *>(q + e);
-                // y - s h in one rounding (s h is exact: s is a power of two)
-                const float2 df = __ffma2_rn(nsc, __half22float2(hv), y);
-                s = __ffma2_rn(df, df, s);
-            }
+        for (uint32_t u = 0; u < units; ++u) {
+            const float4 y = yp[u];
+            const __half2 x0 = xp[4 * u], x1 = xp[4 * u + 2];
+            // y - s h in one rounding (s h is exact: s is a power of two)
+            float2 df = __ffma2_rn(nsc, __half22float2(x0), make_float2(y.x, y.y));
+            s = __ffma2_rn(df, df, s);
+            df = __ffma2_rn(nsc, __half22float2(x1), make_float2(y.z, y.w));
+            s = __ffma2_rn(df, df, s);
         }
     } else {
+        const uint4 *xp = reinterpret_cast<const uint4 *>(row);
 #pragma unroll 2
-        for (; i + 16 <= d; i += 16) {
-            const uint4 raw = *reinterpret_cast<const uint4 *>(row + i);
+        for (uint32_t u = 0; u < units; ++u) {
+            const uint4 raw = xp[u];
             const uint32_t wds[4] = {raw.x, raw.y, raw.z, raw.w};
 #pragma unroll
-            for (uint32_t g = 0; g < 4; ++g) {
-                const __half2_raw pr =
+            for (uint32_t g = 0; g < 4; g += 2) {
+                const float4 y = yp[2 * u + g / 2];
+                const __half2_raw p0 =
                     __nv_cvt_fp8x2_to_halfraw2((__nv_fp8x2_storage_t)((wds[g] >> (16 * h)) & 0xffffu), __NV_E4M3);
-                const float2 y = *reinterpret_cast<const float2 *>(q + i + 4 * g + 2 * h);
-                step2(y, __fmul2_rn(sc, __half22float2(__half2(pr))), s);
+                const __half2_raw p1 =
+                    __nv_cvt_fp8x2_to_halfraw2((__nv_fp8x2_storage_t)((wds[g + 1] >> (16 * h)) & 0xffffu), __NV_E4M3);
+                step2(make_float2(y.x, y.y), __fmul2_rn(sc, __half22float2(__half2(p0))), s);
+                step2(make_float2(y.z, y.w), __fmul2_rn(sc, __half22float2(__half2(p1))), s);
             }
         }
     }
+    uint32_t i = units * (ST == ANN_E4M3 ? 16 : 8);
     // tail (d not a multiple of the vector width); i is a multiple of 4 here
     #pragma unroll 1
     for (; i < d; i += 4) {
-        if (i + 2 * h < d) elem_step<ST>(q[i + 2 * h], row, i + 2 * h, scale, s.x);
-        if (i + 2 * h + 1 < d) elem_step<ST>(q[i + 2 * h + 1], row, i + 2 * h + 1, scale, s.y);
+        if (i + 2 * h < d) elem_step<ST>(q[i / 2], row, i + 2 * h, scale, s.x);
+        if (i + 2 * h + 1 < d) elem_step<ST>(q[i / 2 + 1], row, i + 2 * h + 1, scale, s.y);
     }
     return __fadd_rn(s.x, s.y);
 }
@@ -210,7 +220,9 @@ struct WarpSearch {
     }
 
     // shared-memory arrays of this warp
+    // the query, in the layout of query_pos
     __device__ __forceinline__ float *q() const { return reinterpret_cast<float *>(base + a.lay.q); }
+    __device__ __forceinline__ const float *qpart(uint32_t p) const { return q() + p * a.q_part; }
     __device__ __forceinline__ float *bd() const { return reinterpret_cast<float *>(base + a.lay.bd); }
     __device__ __forceinline__ uint32_t *bi() const { return reinterpret_cast<uint32_t *>(base + a.lay.bi); }
     __device__ __forceinline__ uint8_t *bs() const { return base + a.lay.bs; }
@@ -306,7 +318,7 @@ struct WarpSearch {
     // ----------------------------------------------------- evaluate rows
     // Distances of rows ids[0, n) of `codes` into out[0, n), R (<= 32 / LPR)
     // rows of `stride` bytes per bulk-copy round; lanes LPR r .. LPR r + LPR
-    // - 1 compute row r (a lane pair, or four lanes for wide rows).
+    // - 1 compute row r.
     template <int RST>
     __device__ bool evaluate(const uint8_t *codes, const float *scales, uint32_t row_bytes, const uint32_t *ids,
                              uint32_t n, float *out, uint32_t R, uint32_t stride)
@@ -331,10 +343,10 @@ struct WarpSearch {
             const float rs = __shfl_sync(0xffffffffu, scale, r);
             float part = 0.0f;
             if (LPR == 2) {
-                if (r < rows) part = row_dist_half<RST>(stage() + r * stride, q(), rs, a.d, lane & 1);
+                if (r < rows) part = row_dist_half<RST>(stage() + r * stride, qpart(lane & 1), rs, a.d, lane & 1);
             } else {
                 // sum j of the row, then (s0 + s1) and (s2 + s3) on lane pairs
-                if (r < rows) part = row_dist_quarter<RST>(stage() + r * stride, q(), rs, a.d, lane & 3);
+                if (r < rows) part = row_dist_quarter<RST>(stage() + r * stride, qpart(lane & 3), rs, a.d, lane & 3);
                 part = __fadd_rn(part, __shfl_xor_sync(0xffffffffu, part, 1));
             }
             const float other = __shfl_xor_sync(0xffffffffu, part, LPR / 2);
@@ -599,6 +611,7 @@ struct WarpSearch {
         // 4 words of the query's sign bits relative to the parent ([q >
         // x_parent], one ballot per 32 dimensions) at a time. Words past w
         // have no dimension: their bits are 0 on both sides.
+        const float *ql = q() + query_pos<LPR>(lane, a.q_part);   // + 32 / LPR each 32 dimensions
         #pragma unroll 1
         for (uint32_t t0 = 0; t0 < w; t0 += 4) {
             uint32_t dw[N][4];
@@ -621,7 +634,7 @@ struct WarpSearch {
 #pragma unroll
             for (uint32_t x = 0; x < 4; ++x) {
                 const uint32_t i = 32 * (t0 + x) + lane;
-                const uint32_t qw = __ballot_sync(0xffffffffu, i < a.d && q()[min(i, a.d - 1)] > pv[x]);
+                const uint32_t qw = __ballot_sync(0xffffffffu, i < a.d && ql[min(t0 + x, w - 1) * (32 / LPR)] > pv[x]);
 #pragma unroll
                 for (uint32_t r = 0; r < N; ++r) u[r] += __popc(qw ^ dw[r][x]);
             }
@@ -832,7 +845,7 @@ struct WarpSearch {
         // past L1: a serving ring's slots are rewritten between uses
         #pragma unroll 1
         for (uint32_t i = lane; i < dpad; i += 32)
-            q()[i] = i < a.d ? *reinterpret_cast<const volatile float *>(qg + i) : 0.0f;
+            q()[query_pos<LPR>(i, a.q_part)] = i < a.d ? *reinterpret_cast<const volatile float *>(qg + i) : 0.0f;
         __syncwarp();
         const bool ghost = ghost_entry(qp.entry);
         gbm = ghost && a.gbm_words > 0;
@@ -1070,7 +1083,7 @@ __global__ void __launch_bounds__(128, kSearchBlocksPerSm) serve_kernel(const Ar
 
 uint32_t align16(uint32_t x) { return (x + 15) & ~15u; }
 
-Layout make_layout(uint32_t d, uint32_t cap_buf, uint32_t cap_cand, uint32_t stage_rows, uint32_t stage_stride,
+Layout make_layout(uint32_t q_floats, uint32_t cap_buf, uint32_t cap_cand, uint32_t stage_rows, uint32_t stage_stride,
                    uint32_t rr_stride, uint32_t gbm_words, bool serve)
 {
     Layout L{};
@@ -1080,7 +1093,7 @@ Layout make_layout(uint32_t d, uint32_t cap_buf, uint32_t cap_cand, uint32_t sta
         o = align16(o + bytes);
         return at;
     };
-    L.q = take(((d + 31) & ~31u) * 4);
+    L.q = take(q_floats * 4);
     L.bd = take(cap_buf * 4);
     L.bi = take(cap_buf * 4);
     L.bs = take(cap_buf);
@@ -1247,13 +1260,8 @@ ann_status plan_args(ann_index *ix, const QParams &q, Args &a)
     // the search stages stored rows; the rerank stages FP32 rows in the same
     // area, fewer per round (it reads itopk rows per query, the search
     // thousands), so the area is sized by the stored rows
-    const uint32_t stage_bytes = std::max(ix->row_bytes, q.rerank ? a.row32_bytes : 0u);
     a.stage_stride = smem_row_stride(ix->row_bytes);
     a.rr_stride = q.rerank ? smem_row_stride(a.row32_bytes) : 0u;
-    // rows of more than 1 KB (wide FP32 vectors, 512 and up to ANN_MAX_DIM
-    // dimensions) are computed by four lanes each, at most 8 per round;
-    // narrower ones by lane pairs, 16 per round
-    a.lpr = stage_bytes > 1024 ? 4 : 2;
     // visited tables: the queue plus one iteration's candidates must fit in
     // half a table (the reset threshold)
     if (cap_buf + cap_cand > (1u << (kVisitedBits - 1))) {
@@ -1266,7 +1274,8 @@ ann_status plan_args(ann_index *ix, const QParams &q, Args &a)
     a.slot_base = 0;
     a.gbm_words = (ghost_entry(q.entry) && ix->n_ghost <= kGhostBitmapMax) ? (ix->n_ghost + 31) / 32 : 0;
     // one warp with a few staged rows is the least a launch can be made of
-    const uint32_t least = make_layout(a.d, cap_buf, cap_cand, 4, a.stage_stride, a.rr_stride, a.gbm_words, true).total;
+    const uint32_t least = 
+        make_layout(query_part(a.d, 4) * 4, cap_buf, cap_cand, 4, a.stage_stride, a.rr_stride, a.gbm_words, true).total;
     if (least > ix->smem_optin) {
         set_error("ann_search: per-query state (%u bytes) exceeds shared memory", least);
         return ANN_EINVAL;
@@ -1274,20 +1283,22 @@ ann_status plan_args(ann_index *ix, const QParams &q, Args &a)
     return ANN_OK;
 }
 
-// The launch shape for nq queries: rows staged per gather round, the per-warp
-// layout, warps per block and blocks per SM.
+// The launch shape for nq queries: lanes per row, rows staged per gather
+// round, the per-warp layout, warps per block and blocks per SM.
 ann_status plan_shape(ann_index *ix, Args &a, uint64_t nq, bool serve, int &warps, size_t &smem, int &nb)
 {
     struct Shape {
         Layout lay;
-        uint32_t rows;
+        uint32_t lpr, rows;
         int warps, nb;
         size_t smem;
     };
-    auto fit = [&](uint32_t rows) {
+    auto fit = [&](uint32_t lpr, uint32_t rows) {
         Shape best{}, sh{};
+        sh.lpr = lpr;
         sh.rows = rows;
-        sh.lay = make_layout(a.d, a.cap_buf, a.cap_cand, rows, a.stage_stride, a.rr_stride, a.gbm_words, serve);
+        sh.lay = make_layout(query_part(a.d, lpr) * lpr, a.cap_buf, a.cap_cand, rows, a.stage_stride, a.rr_stride,
+                             a.gbm_words, serve);
         // blocks of one or two warps pack a shared memory that blocks of four
         // leave partly unused (256-d FP32 rows, 512-entry queues: 14 resident
         // warps an SM instead of 12)
@@ -1295,9 +1306,9 @@ ann_status plan_shape(ann_index *ix, Args &a, uint64_t nq, bool serve, int &warp
             sh.smem = (size_t)sh.lay.total * sh.warps;
             if (sh.smem > ix->smem_optin) continue;
             switch (ix->storage) {
-            case ANN_F32: sh.nb = blocks_per_sm<ANN_F32>(sh.warps, sh.smem, a.lpr); break;
-            case ANN_F16: sh.nb = blocks_per_sm<ANN_F16>(sh.warps, sh.smem, a.lpr); break;
-            default: sh.nb = blocks_per_sm<ANN_E4M3>(sh.warps, sh.smem, a.lpr); break;
+            case ANN_F32: sh.nb = blocks_per_sm<ANN_F32>(sh.warps, sh.smem, lpr); break;
+            case ANN_F16: sh.nb = blocks_per_sm<ANN_F16>(sh.warps, sh.smem, lpr); break;
+            default: sh.nb = blocks_per_sm<ANN_E4M3>(sh.warps, sh.smem, lpr); break;
             }
             // A server's warps take and finish queries one by one, and a block
             // holds its shared memory until its last warp is done: single
@@ -1308,40 +1319,48 @@ ann_status plan_shape(ann_index *ix, Args &a, uint64_t nq, bool serve, int &warp
     };
     // The staged rows take most of a warp's shared memory. Fewer of them per
     // gather round mean more rounds, so a slower query, but can admit more
-    // resident warps. What that is worth depends on how often the resident
-    // warps have to be filled to take the batch: fewer rows are taken only
-    // where they lower that count, and a quarter round only where everything
-    // then runs at once. Measured, ms with 16 / 8 / 4 rows: 256-d FP32,
-    // itopk 256: 1,300 queries 3.27 / 3.81 / 4.96 (one filling each), 2,000
-    // queries 6.18 / 4.08 / 5.27 (2, 1, 1), 2,432 queries 6.34 / 7.43 / 5.42 (2,
-    // 2, 1), 8,000 queries 18.8 / 15.7 / 16.5 (6, 4, 4); 768-d FP16, 8 / 4
-    // rows: 1,300 queries 1.34 / 1.89 (1, 1), 3,001 queries 2.59 / 2.38 (2, 1).
+    // resident warps: 16 rows on lane pairs, 8 or 4 on four lanes each. What
+    // that is worth depends on how often the resident warps have to be filled
+    // to take the batch. 8 rows are taken where that count falls by an eighth.
+    // 4 rows want more than a third, or an eighth with queues of 128 and more,
+    // where the distances are a smaller part of the work and all queries take
+    // about as long, so that every filling counts in full. Measured, us with 16
+    // / 8 / 4 rows (fillings), FP32 256-d, itopk 64: 1,500 queries 738 / 794 /
+    // 1,011 (1, 1, 1), 3,000 queries 1,245 / 876 / 1,116 (2, 1, 1), 6,500
+    // queries 2,396 / 1,764 / 2,120 (4, 3, 2), 10,000 queries 3,281 / 2,380 /
+    // 2,493 (6, 4, 3); itopk 256: 3,000 queries 4,072 / 3,950 / 2,894 (2, 2,
+    // 1), 6,500 queries 9,290 / 6,566 / 5,769 (5, 3, 2); FP32 512-d, itopk 64,
+    // 10,000 queries 7,824 / 5,338 / 4,785 (11, 7, 4). FP32 96-d, itopk 64: 24
+    // resident warps an SM by their registers either way, 10,000 queries 1,450
+    // / 1,484 with 16 / 8.
     // ANN_STAGE_ROWS fixes the count instead (experiments).
     const int env_rows = env_int("ANN_STAGE_ROWS", 0);
-    const uint32_t full = 32 / a.lpr;
     auto fillings = [&](const Shape &s) {
         const uint64_t slots = (uint64_t)s.nb * s.warps * ix->num_sms;
-        return slots ? (nq + slots - 1) / slots : ~0ull;
+        return slots ? (nq + slots - 1) / slots : 1ull << 32;
     };
     Shape best{};
     if (env_rows > 0) {
-        best = fit((uint32_t)std::min<int>((int)full, env_rows));
+        best = env_rows > 8 ? fit(2, (uint32_t)std::min(16, env_rows)) : fit(4, (uint32_t)env_rows);
     } else {
-        best = fit(full);
-        const Shape half = fit(full / 2);
-        if (fillings(half) < fillings(best)) best = half;
-        if (full / 4 >= 4 && fillings(best) > 1) {
-            const Shape quarter = fit(full / 4);
-            if (fillings(quarter) == 1) best = quarter;
+        best = fit(2, 16);
+        if (fillings(best) > 1) {
+            const Shape eight = fit(4, 8);
+            if (fillings(eight) * 8 <= fillings(best) * 7) best = eight;
+            const Shape four = fit(4, 4);
+            if (a.qp.L >= 128 ? fillings(four) * 8 <= fillings(best) * 7 : fillings(four) * 3 < fillings(best) * 2)
+                best = four;
         }
     }
-    if (best.warps == 0) best = fit(4);
+    if (best.warps == 0) best = fit(4, 4);
     if (best.warps == 0) {
         set_error("ann_search: kernel does not fit on an SM");
         return ANN_EINVAL;
     }
+    a.lpr = best.lpr;
+    a.q_part = query_part(a.d, a.lpr);
     a.stage_rows = best.rows;
-    a.rr_rows = a.rr_stride ? std::min(full, std::max(1u, best.rows * a.stage_stride / a.rr_stride)) : 0u;
+    a.rr_rows = a.rr_stride ? std::min(32 / a.lpr, std::max(1u, best.rows * a.stage_stride / a.rr_stride)) : 0u;
     a.lay = best.lay;
     warps = best.warps;
     smem = best.smem;

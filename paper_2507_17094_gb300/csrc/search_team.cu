@@ -24,8 +24,9 @@
 // termination and the counters are those of the warp kernel, so results and
 // counters are the same. Measured, us a call, warps / teams: one query of FP16
 // 96-d rows with rerank, itopk 64: 477 / 228; 61 queries of E4M3 128-d rows:
-// 586 / 341; 152 queries of FP32 256-d rows, itopk 256: 3,294 / 1,386. Nothing here waits on a barrier that a copy completes,
-// so there is no time-out to report.
+// 586 / 304; 152 queries of FP32 256-d rows, itopk 256: 3,294 / 1,239. Nothing
+// here waits on a barrier that a copy completes, so there is no time-out to
+// report.
 #include <algorithm>
 
 #include "search_common.cuh"
@@ -45,6 +46,7 @@ struct TeamArgs {
     TeamSearch t;
     TeamLayout lay;
     uint32_t rows, stride, rr_rows, rr_stride;   // rows per gather round and their stride: stored rows, FP32 rerank
+    uint32_t q_part;                             // floats between the parts of the query
     uint32_t row_magic, row32_magic;             // ceil(2^32 / 16-byte chunks of a row): chunk index -> row
 };
 
@@ -81,6 +83,7 @@ struct Team {
     {
     }
 
+    // the query, in the layout of query_pos for four lanes per row
     __device__ __forceinline__ float *q() const { return reinterpret_cast<float *>(base + g.lay.q); }
     __device__ __forceinline__ uint64_t *qk() const { return reinterpret_cast<uint64_t *>(base + g.lay.qk); }
     __device__ __forceinline__ uint8_t *bs() const { return base + g.lay.bs; }
@@ -171,6 +174,7 @@ struct Team {
                                              uint32_t magic, uint32_t n, uint32_t R, uint32_t stride, Id id, Out out)
     {
         const uint32_t quad = tid >> 2, chunks = row_bytes >> 4;
+        const float *qj = q() + (lane & 3) * g.q_part;
         #pragma unroll 1
         for (uint32_t b0 = 0; b0 < n; b0 += R) {
             const uint32_t rows = min(R, n - b0);
@@ -190,7 +194,7 @@ struct Team {
             #pragma unroll 1
             for (uint32_t r = quad; r - quad < rows; r += kQuads, s0 = s1) {
                 float part = 0.0f;
-                if (r < rows) part = row_dist_quarter<RST, 8>(stage() + r * stride, q(), s0, a.d, lane & 3);
+                if (r < rows) part = row_dist_quarter<RST>(stage() + r * stride, qj, s0, a.d, lane & 3);
                 part = __fadd_rn(part, __shfl_xor_sync(0xffffffffu, part, 1));
                 part = __fadd_rn(part, __shfl_xor_sync(0xffffffffu, part, 2));
                 if (r < rows && (lane & 3) == 0) out(b0 + r, part);
@@ -349,7 +353,8 @@ struct Team {
             const uint32_t parent = __shfl_sync(0xffffffffu, pid, pp);
             const float ps = ST != ANN_F32 ? __ldg(v.scales + parent) : 1.0f;
             bool b = false;
-            if (i < a.d) b = q()[i] > stored_elem<ST>(v.codes + (uint64_t)parent * v.row_bytes, i, ps);
+            if (i < a.d)
+                b = q()[query_pos<4>(i, g.q_part)] > stored_elem<ST>(v.codes + (uint64_t)parent * v.row_bytes, i, ps);
             const uint32_t bits = __ballot_sync(0xffffffffu, b);
             if (lane == 0) sign()[y] = bits;
         }
@@ -503,7 +508,8 @@ struct Team {
         st = ann_query_stats{};
         cnt = 0;
         const uint32_t dpad = (a.d + 31) & ~31u;
-        for (uint32_t i = tid; i < dpad; i += NT) q()[i] = i < a.d ? __ldcg(qg + i) : 0.0f;
+        for (uint32_t i = tid; i < dpad; i += NT)
+            q()[query_pos<4>(i, g.q_part)] = i < a.d ? __ldcg(qg + i) : 0.0f;
         const bool ghost = ghost_entry(qp.entry);
         gbm = ghost && a.gbm_words > 0;
         hash_clear();
@@ -607,7 +613,8 @@ TeamArgs plan(const TeamSearch &t, uint32_t rows, uint32_t max_rows)
         return at;
     };
     TeamLayout &L = g.lay;
-    L.q = take(round_up(t.d, 32) * 4);
+    g.q_part = query_part(t.d, 4);
+    L.q = take(g.q_part * 16);
     L.qk = take(t.cap_buf * 8);
     L.bs = take(t.cap_buf);
     L.ck = take(t.cap_cand * 8);
