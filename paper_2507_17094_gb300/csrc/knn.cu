@@ -187,11 +187,11 @@ constexpr uint32_t kTileBytes = kTileRows * kBK * 2;
 constexpr uint32_t kMinStages = 4, kMaxStages = 12;   // column tiles (64 elements deep) in flight
 constexpr uint32_t kSample = 4096;       // rows the centre is estimated from
 constexpr uint32_t kCarry = 512;         // columns a row carries from range to range
-constexpr uint32_t kEntries = 768;       // carried and new columns one selection can hold
+constexpr uint32_t kEntries = 768, kFewEntries = 576;   // carried and new columns one selection can hold
 constexpr uint32_t kFirstTiles = 4;      // column tiles of the first range: kept whole
 constexpr uint32_t kMaxS = kFirstTiles;  // column segments of a range (one CTA each)
 constexpr uint32_t kParts = 4;           // parts of the columns: one half of every second tile, an epilogue warp each
-constexpr uint32_t kSelectWarps = 8, kRescoreWarps = 8;
+constexpr uint32_t kSelectWarps = 4, kRescoreWarps = 8;
 constexpr uint32_t kChunk = 64;          // elements of a row staged at a time by the rescoring
 constexpr uint32_t kChunkStride = kChunk + 4;   // floats: 8 lanes' 16-byte reads hit 8 bank groups
 static_assert(2 * ANN_MAX_DEGREE <= kCarry && 2 * ANN_MAX_DEGREE < kFirstTiles * kTileRows, "K entries are carried");
@@ -326,6 +326,7 @@ struct KnnWork {
     uint32_t S, cap;         // column segments; entries per row, segment and part
     uint32_t stages;         // slots of the column-tile ring
     uint32_t low_slots;      // slots of lower[] in shared memory (a power of two)
+    uint32_t entries;        // columns that a selection can hold
 };
 
 // One CTA: NSUB x 128 operand rows against the column tiles of one segment
@@ -349,6 +350,15 @@ __device__ __forceinline__ float fmin3(float a, float b, float c)
     return r;
 }
 
+// Entries of columns nb .. nb + 3 at p (32-byte aligned).
+__device__ __forceinline__ void store_four(uint2 *p, float2 x, float2 y, uint32_t nb)
+{
+    asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "r"(__float_as_uint(x.x)),
+                 "r"(nb), "r"(__float_as_uint(x.y)), "r"(nb + 1), "r"(__float_as_uint(y.x)), "r"(nb + 2),
+                 "r"(__float_as_uint(y.y)), "r"(nb + 3)
+                 : "memory");
+}
+
 // Append (v, col) to a list at p if v <= T, without a branch: the lanes that
 // append differ from value to value.
 __device__ __forceinline__ void append_if(uint2 *&p, float v, float T, uint32_t col)
@@ -367,10 +377,10 @@ constexpr int kFilterThreads = 64 + 32 * kFilterEpiWarps;
 constexpr uint32_t kLowSlots = 8;        // column tiles whose lower[] is in shared memory, at most
 constexpr uint32_t kFilterBars = 384;    // bytes for the barriers
 
-template <int NSUB>
+template <int NSUB, bool FIRST>
 __global__ void __launch_bounds__(kFilterThreads, 1)
     knn_filter_kernel(const __grid_constant__ CUtensorMap map, uint32_t n, uint32_t nkb, uint32_t row0, uint32_t t0,
-                      uint32_t t1, uint32_t first, KnnWork w)
+                      uint32_t t1, KnnWork w)
 {
     extern __shared__ uint8_t smem_raw[];
     if (w.st->all) return;
@@ -498,7 +508,7 @@ __global__ void __launch_bounds__(kFilterThreads, 1)
 #pragma unroll
         for (int sub = 0; sub < NSUB; ++sub) {
             const uint32_t lr = rb * NSUB * kTileRows + sub * kTileRows + q * 32 + lane;
-            T[sub] = row0 + lr >= n ? -FLT_MAX : first ? FLT_MAX : w.T[lr];
+            T[sub] = row0 + lr >= n ? -FLT_MAX : FIRST ? FLT_MAX : w.T[lr];
             list[sub] = next[sub] = w.kept + ((size_t)lr * lists + seg * kParts + h) * cap;
         }
         for (uint32_t t = b0 + buf; t < b1; t += 2) {
@@ -528,21 +538,44 @@ __global__ void __launch_bounds__(kFilterThreads, 1)
                 }
                 const float *low = sLow + ls * kTileRows + c;
                 const uint32_t nb = t * kTileRows + c;
+                auto values = [&](int sub, int g, const float4 &l, float2 &x, float2 &y) {
+                    x = __ffma2_rn(make_float2(v[sub][g], v[sub][g + 1]), make_float2(-2.0f, -2.0f),
+                                   make_float2(l.x, l.y));
+                    y = __ffma2_rn(make_float2(v[sub][g + 2], v[sub][g + 3]), make_float2(-2.0f, -2.0f),
+                                   make_float2(l.z, l.w));
+                };
+                if (FIRST) {
+                    // every column of every row is kept (none lies past n): four
+                    // entries to a store (one by one, the lanes' lists being
+                    // apart: 190 us instead of 38 for 38,912 rows)
 #pragma unroll
-                for (int g = 0; g < 32; g += 4) {
-                    const float4 l = *reinterpret_cast<const float4 *>(low + g);
+                    for (int g = 0; g < 32; g += 4) {
+                        const float4 l = *reinterpret_cast<const float4 *>(low + g);
 #pragma unroll
-                    for (int sub = 0; sub < NSUB; ++sub) {
-                        const float2 x = __ffma2_rn(make_float2(v[sub][g], v[sub][g + 1]), make_float2(-2.0f, -2.0f),
-                                                    make_float2(l.x, l.y));
-                        const float2 y = __ffma2_rn(make_float2(v[sub][g + 2], v[sub][g + 3]),
-                                                    make_float2(-2.0f, -2.0f), make_float2(l.z, l.w));
-                        // the row itself is dropped by the selection
-                        if (fmin3(fminf(x.x, x.y), y.x, y.y) <= T[sub]) {
-                            append_if(next[sub], x.x, T[sub], nb + g);
-                            append_if(next[sub], x.y, T[sub], nb + g + 1);
-                            append_if(next[sub], y.x, T[sub], nb + g + 2);
-                            append_if(next[sub], y.y, T[sub], nb + g + 3);
+                        for (int sub = 0; sub < NSUB; ++sub) {
+                            float2 x, y;
+                            values(sub, g, l, x, y);
+                            if (T[sub] > 0.0f) {
+                                store_four(next[sub], x, y, nb + g);
+                                next[sub] += 4;
+                            }
+                        }
+                    }
+                } else {
+#pragma unroll
+                    for (int g = 0; g < 32; g += 4) {
+                        const float4 l = *reinterpret_cast<const float4 *>(low + g);
+#pragma unroll
+                        for (int sub = 0; sub < NSUB; ++sub) {
+                            float2 x, y;
+                            values(sub, g, l, x, y);
+                            // the row itself is dropped by the selection
+                            if (fmin3(fminf(x.x, x.y), y.x, y.y) <= T[sub]) {
+                                append_if(next[sub], x.x, T[sub], nb + g);
+                                append_if(next[sub], x.y, T[sub], nb + g + 1);
+                                append_if(next[sub], y.x, T[sub], nb + g + 2);
+                                append_if(next[sub], y.y, T[sub], nb + g + 3);
+                            }
                         }
                     }
                 }
@@ -579,16 +612,30 @@ __global__ void __launch_bounds__(kSelectWarps * 32)
     const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t lr = blockIdx.x * kSelectWarps + warp;
     if (lr >= rows) return;
-    uint2 *e = reinterpret_cast<uint2 *>(sm) + warp * kEntries;   // (upper value bits, column)
-    uint32_t *hist = reinterpret_cast<uint32_t *>(sm + kSelectWarps * kEntries * 8) + warp * 256;
+    uint2 *e = reinterpret_cast<uint2 *>(sm) + warp * w.entries;   // (upper value bits, column)
+    uint32_t *hist = reinterpret_cast<uint32_t *>(sm + kSelectWarps * w.entries * 8) + warp * 256;
     const float c = bound_c(w.st, d), up = 2.0f * c / (1.0f - c);   // upper - lower value = 2 c N = up * lower[]
     const uint32_t lists = kParts * w.S;   // at most 16
     uint2 *carry = w.carry + (size_t)lr * kCarry;
     uint32_t m = 0;
     bool over = !first && w.T[lr] == -FLT_MAX;
+    float lo = INFINITY, hi = -INFINITY;
+    // four entries a lane at a time, so that their loads are in flight together
     if (!first && !over) {
         m = w.n_carry[lr];
-        for (uint32_t i = lane; i < m; i += 32) e[i] = carry[i];
+        for (uint32_t b = 0; b < m; b += 128) {
+            uint2 x[4];
+#pragma unroll
+            for (uint32_t u = 0; u < 4; ++u)
+                if (b + 32 * u + lane < m) x[u] = carry[b + 32 * u + lane];
+#pragma unroll
+            for (uint32_t u = 0; u < 4; ++u)
+                if (b + 32 * u + lane < m) {
+                    lo = fminf(lo, __uint_as_float(x[u].x));
+                    hi = fmaxf(hi, __uint_as_float(x[u].x));
+                    e[b + 32 * u + lane] = x[u];
+                }
+        }
     }
     const uint32_t counts = lane < lists ? w.n_kept[(size_t)lr * lists + lane] : 0u;
     uint32_t ends = counts;   // of this lane's list among the new entries
@@ -597,37 +644,44 @@ __global__ void __launch_bounds__(kSelectWarps * 32)
         if (lane >= (uint32_t)o) ends += y;
     }
     const uint32_t fresh = __shfl_sync(0xffffffffu, ends, 15);
-    over = over || __any_sync(0xffffffffu, counts > w.cap) || m + fresh > kEntries;
-    float lo = INFINITY, hi = -INFINITY;
+    over = over || __any_sync(0xffffffffu, counts > w.cap) || m + fresh > w.entries;
     bool self = false;
     if (!over) {
-        // the lists as one sequence, so that several loads are in flight
+        // the lists as one sequence
         const uint2 *src = w.kept + (size_t)lr * lists * w.cap;
-#pragma unroll 4
-        for (uint32_t b = 0; b < fresh; b += 32) {
-            const uint32_t i = b + lane;
-            uint32_t s = 0;   // the list that holds entry i
+        for (uint32_t b = 0; b < fresh; b += 128) {
+            uint2 x[4];
+            float nv[4];
 #pragma unroll
-            for (uint32_t step = 8; step; step >>= 1)
-                if (__shfl_sync(0xffffffffu, ends, s + step - 1) <= i) s += step;
-            const uint32_t begin = __shfl_sync(0xffffffffu, ends, s ? s - 1 : 0);
-            if (i < fresh) {
-                const uint2 x = src[s * w.cap + i - (s ? begin : 0u)];
-                float v = fmaf(up, __ldg(w.lower + x.y), __uint_as_float(x.x));
-                if (x.y == row0 + lr) { v = INFINITY; self = true; }   // the row itself
-                e[m + i] = make_uint2(__float_as_uint(v), x.y);
+            for (uint32_t u = 0; u < 4; ++u) {
+                const uint32_t i = b + 32 * u + lane;
+                uint32_t s = 0;   // the list that holds entry i
+#pragma unroll
+                for (uint32_t step = 8; step; step >>= 1)
+                    if (__shfl_sync(0xffffffffu, ends, s + step - 1) <= i) s += step;
+                const uint32_t begin = __shfl_sync(0xffffffffu, ends, s ? s - 1 : 0);
+                if (i < fresh) x[u] = src[s * w.cap + i - (s ? begin : 0u)];
+            }
+#pragma unroll
+            for (uint32_t u = 0; u < 4; ++u)
+                if (b + 32 * u + lane < fresh) nv[u] = __ldg(w.lower + x[u].y);
+#pragma unroll
+            for (uint32_t u = 0; u < 4; ++u) {
+                const uint32_t i = b + 32 * u + lane;
+                if (i >= fresh) continue;
+                float v = fmaf(up, nv[u], __uint_as_float(x[u].x));
+                if (x[u].y == row0 + lr) { v = INFINITY; self = true; }   // the row itself
+                lo = fminf(lo, v);
+                if (v < INFINITY) hi = fmaxf(hi, v);
+                e[m + i] = make_uint2(__float_as_uint(v), x[u].y);
             }
         }
         m += fresh;
         __syncwarp();
-        for (uint32_t i = lane; i < m; i += 32) {
-            const float v = __uint_as_float(e[i].x);
-            lo = fminf(lo, v);
-            if (v < INFINITY) hi = fmaxf(hi, v);
-        }
         self = __any_sync(0xffffffffu, self);
     }
     if (!over && m - (self ? 1u : 0u) >= K) {
+        const uint32_t slack = 4 + K / 16;
         uint32_t need = K;
         float tau = INFINITY;
         for (int o = 16; o; o >>= 1) {
@@ -658,19 +712,20 @@ __global__ void __launch_bounds__(kSelectWarps * 32)
             }
             const uint32_t before = incl - sum;
             const bool here = before < need && need <= incl;
-            uint32_t at = 0, left = need - before;
+            uint32_t at = 0, left = need - before, in_bin = 0;
             if (here) {
                 bool found = false;
 #pragma unroll
                 for (int b = 0; b < 8; ++b)
                     if (!found) {
-                        if (left <= mine[b]) { at = lane * 8 + b; found = true; }
+                        if (left <= mine[b]) { at = lane * 8 + b; in_bin = mine[b]; found = true; }
                         else left -= mine[b];
                     }
             }
             const uint32_t src = __ffs(__ballot_sync(0xffffffffu, here)) - 1;
             at = __shfl_sync(0xffffffffu, at, src);
             need = __shfl_sync(0xffffffffu, left, src);
+            in_bin = __shfl_sync(0xffffffffu, in_bin, src);
             float blo = INFINITY, bhi = -INFINITY;   // the values of that bin
             for (uint32_t i = lane; i < m; i += 32) {
                 const float v = __uint_as_float(e[i].x);
@@ -687,24 +742,33 @@ __global__ void __launch_bounds__(kSelectWarps * 32)
             hi = bhi;
             tau = bhi;
             __syncwarp();
+            if (in_bin - need <= slack) break;   // so few more than K: not worth a second round
         }
         const float nu = __ldg(w.lower + row0 + lr) / (1.0f - c);
         // the row's own share of both bounds, and the rounding of the few
         // operations on these values
         const float T = tau + 2.0f * c * nu + 2.0f * bound_kappa(d) + (fabsf(tau) + nu) * 3.8146973e-6f;
         uint32_t kept = 0;
-        for (uint32_t b = 0; b < m; b += 32) {
-            uint2 x = make_uint2(0, 0);
-            bool keep = false;
-            if (b + lane < m) {
-                x = e[b + lane];
-                const float v = __uint_as_float(x.x);
-                keep = v < INFINITY && fmaf(-up, __ldg(w.lower + x.y), v) <= T;
+        for (uint32_t b = 0; b < m; b += 128) {
+            uint2 x[4];
+            float low[4];
+#pragma unroll
+            for (uint32_t u = 0; u < 4; ++u) {
+                const uint32_t i = b + 32 * u + lane;
+                x[u] = i < m ? e[i] : make_uint2(__float_as_uint(INFINITY), 0u);
+                // the lower value is no larger than the upper one: needed only
+                // of what that alone does not keep
+                low[u] = __uint_as_float(x[u].x);
+                if (low[u] > T && low[u] < INFINITY) low[u] = fmaf(-up, __ldg(w.lower + x[u].y), low[u]);
             }
-            const uint32_t mask = __ballot_sync(0xffffffffu, keep);
-            const uint32_t at = kept + __popc(mask & ((1u << lane) - 1u));
-            if (keep && at < kCarry) carry[at] = x;
-            kept += __popc(mask);
+#pragma unroll
+            for (uint32_t u = 0; u < 4; ++u) {
+                const bool keep = low[u] <= T && low[u] < INFINITY;
+                const uint32_t mask = __ballot_sync(0xffffffffu, keep);
+                const uint32_t at = kept + __popc(mask & ((1u << lane) - 1u));
+                if (keep && at < kCarry) carry[at] = x[u];
+                kept += __popc(mask);
+            }
         }
         over = kept > kCarry;
         if (!over && lane == 0) {
@@ -826,14 +890,14 @@ uint32_t gcd(uint32_t a, uint32_t b)
     return a;
 }
 
-template <int NSUB>
+template <int NSUB, bool FIRST>
 cudaError_t launch_filter(const CUtensorMap &map, uint32_t blocks, size_t smem, uint32_t n, uint32_t nkb, uint32_t row0,
-                          uint32_t t0, uint32_t t1, uint32_t first, const KnnWork &w, cudaStream_t st)
+                          uint32_t t0, uint32_t t1, const KnnWork &w, cudaStream_t st)
 {
     cudaError_t e =
-        cudaFuncSetAttribute(knn_filter_kernel<NSUB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaFuncSetAttribute(knn_filter_kernel<NSUB, FIRST>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    knn_filter_kernel<NSUB><<<blocks, kFilterThreads, smem, st>>>(map, n, nkb, row0, t0, t1, first, w);
+    knn_filter_kernel<NSUB, FIRST><<<blocks, kFilterThreads, smem, st>>>(map, n, nkb, row0, t0, t1, w);
     return cudaGetLastError();
 }
 
@@ -865,6 +929,11 @@ ann_status knn_filtered(const float *X, uint32_t n, uint32_t d, uint32_t K, uint
     // and eight standard deviations (and its share of the first range), and
     // the 64 columns of a tile that have to fit before it is tested.
     const uint32_t growth = K <= 32 ? 6 : K <= 128 ? 4 : 2;
+    // A selection's entries, carried (about K) and new: the first range's 512,
+    // and with K up to 64 at most 260 expected, eight standard deviations below
+    // 576; their shared memory decides how many warps are resident (36 an SM
+    // against 28).
+    const uint32_t entries = K <= 64 ? kFewEntries : kEntries;
     auto segments = [&](uint32_t blocks) {   // a power of two: the first range divides evenly
         uint32_t S = 1;
         while (2 * S <= kMaxS && blocks * 2 * S <= (uint32_t)sms) S *= 2;
@@ -911,7 +980,7 @@ ann_status knn_filtered(const float *X, uint32_t n, uint32_t d, uint32_t K, uint
                     reinterpret_cast<uint32_t *>(ws + o_nc),
                     reinterpret_cast<uint2 *>(ws + o_kept),
                     reinterpret_cast<uint32_t *>(ws + o_nk),
-                    state, 1, 0, stages, slots};
+                    state, 1, 0, stages, slots, entries};
     uint32_t stride = std::max(1u, (uint32_t)(0.6180339887 * n));
     while (gcd(stride, n) != 1) ++stride;
     CUtensorMap map;
@@ -928,7 +997,7 @@ ann_status knn_filtered(const float *X, uint32_t n, uint32_t d, uint32_t K, uint
                                                                                 norm, state);
         knn_bound_kernel<<<std::min(grid_for(n_pad, 256), sms * 8), 256, 0, st>>>(norm, n, n_pad, d, lower, state);
         run(cudaGetLastError());
-        const size_t sel_smem = kSelectWarps * (kEntries * 8 + 1024);
+        const size_t sel_smem = kSelectWarps * (w.entries * 8 + 1024);
         const size_t res_smem =
             kRescoreWarps * (32 * kChunkStride * 4 + (kCarry + 1) * 8 + (size_t)((d + 3) & ~3u) * 4);
         // bulk copies move whole 16-byte units from 16-byte boundaries
@@ -943,8 +1012,9 @@ ann_status knn_filtered(const float *X, uint32_t n, uint32_t d, uint32_t K, uint
             uint32_t t0 = 0, t1 = std::min(kFirstTiles, n_tiles);
             while (t0 < n_tiles && e == cudaSuccess) {
                 const uint32_t first = t0 == 0;
-                run(nsub == 2 ? launch_filter<2>(map, blocks * w.S, filter_smem, n, nkb, row0, t0, t1, first, w, st)
-                              : launch_filter<1>(map, blocks * w.S, filter_smem, n, nkb, row0, t0, t1, first, w, st));
+                const auto launch = nsub == 2 ? (first ? launch_filter<2, true> : launch_filter<2, false>)
+                                              : (first ? launch_filter<1, true> : launch_filter<1, false>);
+                run(launch(map, blocks * w.S, filter_smem, n, nkb, row0, t0, t1, w, st));
                 knn_select_kernel<<<grid_for(rows, kSelectWarps), kSelectWarps * 32, sel_smem, st>>>(
                     n, d, K, row0, rows, first, w);
                 t0 = t1;
