@@ -21,9 +21,9 @@
 //   4. knn_rescore_kernel computes the exact distances of the few columns left
 //      (K and those too close to call) and writes the K first.
 //
-// Measured: 120,000 x 128, K 64: 265 -> 8.1 ms (filter 5.0, selection 2.1,
-// rescoring 0.9; the product alone at the measured BF16 rate would take 1.9);
-// 10,000 x 96, K 32: 2,504 -> 335 us.
+// Measured: 120,000 x 128, K 64: 265 -> 7.1 ms (filter 4.5, selection 1.8,
+// rescoring 0.8; the product alone at the measured BF16 rate would take 1.9);
+// 10,000 x 96, K 32: 2,504 -> 269 us.
 //
 // Steps 2 and 3 repeat over growing column ranges (4 tiles, then 2 to 6 times
 // more each time), so a row sees about K (growth - 1) survivors per range
@@ -192,7 +192,7 @@ constexpr uint32_t kFirstTiles = 4;      // column tiles of the first range: kep
 constexpr uint32_t kMaxS = kFirstTiles;  // column segments of a range (one CTA each)
 constexpr uint32_t kParts = 4;           // parts of the columns: one half of every second tile, an epilogue warp each
 constexpr uint32_t kSelectWarps = 4, kRescoreWarps = 8;
-constexpr uint32_t kChunk = 64;          // elements of a row staged at a time by the rescoring
+constexpr uint32_t kChunk = 32;          // elements of a row staged at a time by the rescoring
 constexpr uint32_t kChunkStride = kChunk + 4;   // floats: 8 lanes' 16-byte reads hit 8 bank groups
 static_assert(2 * ANN_MAX_DEGREE <= kCarry && 2 * ANN_MAX_DEGREE < kFirstTiles * kTileRows, "K entries are carried");
 
@@ -603,7 +603,8 @@ __global__ void __launch_bounds__(kFilterThreads, 1)
 // exponent, into a few), then the columns it does not exclude are carried.
 // A row that overflowed a buffer gets the threshold -FLT_MAX: it keeps
 // nothing any more and is left to the plain kernel. Bound by the latency of
-// its short dependent steps; 28 warps per SM hide it.
+// its short dependent steps and of its gathers, which 36 warps per SM and four
+// loads a lane in flight hide.
 __global__ void __launch_bounds__(kSelectWarps * 32)
     knn_select_kernel(uint32_t n, uint32_t d, uint32_t K, uint32_t row0, uint32_t rows, uint32_t first, KnnWork w)
 {
@@ -784,15 +785,26 @@ __global__ void __launch_bounds__(kSelectWarps * 32)
     }
 }
 
+template <int N>
+__device__ __forceinline__ void copy_async(void *dst, const void *src)
+{
+    if (N == 16)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_addr(dst)), "l"(src) : "memory");
+    else
+        asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(smem_addr(dst)), "l"(src), "n"(N) : "memory");
+}
+
 // One warp per row of the chunk: the exact distances of the carried columns
 // (a lane each, one fused multiply-add per element in index order), ranked by
 // (distance, id); rows without a valid carried list are listed for the plain
-// kernel. The candidates' rows are staged 64 elements at a time, one bulk
-// copy per lane: read by the lanes directly, every load would touch 32 lines
-// (120,000 x 128, K 64: 544 us per 38,912 rows).
+// kernel. Bound by the gathers: a column's row is read in pieces of kChunk
+// elements by asynchronous copies, neighbouring lanes copying neighbouring
+// units, one piece ahead of the arithmetic (120,000 x 128, K 64, us per 38,912
+// rows: 268; one bulk copy per lane and no overlap 295; read by the lanes
+// directly, every load touching 32 lines, 544).
 __global__ void __launch_bounds__(kRescoreWarps * 32)
     knn_rescore_kernel(const float *__restrict__ X, uint32_t n, uint32_t d, uint32_t K, uint32_t stride, uint32_t row0,
-                       uint32_t rows, uint32_t bulk, KnnWork w, uint32_t *__restrict__ list,
+                       uint32_t rows, bool wide, KnnWork w, uint32_t *__restrict__ list,
                        uint32_t *__restrict__ out)
 {
     extern __shared__ __align__(16) uint8_t sm[];
@@ -800,10 +812,9 @@ __global__ void __launch_bounds__(kRescoreWarps * 32)
     const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t lr = blockIdx.x * kRescoreWarps + warp;
     if (lr >= rows) return;
-    float *stage = reinterpret_cast<float *>(sm) + warp * 32 * kChunkStride;
-    uint64_t *keys = reinterpret_cast<uint64_t *>(sm + kRescoreWarps * 32 * kChunkStride * 4) + warp * (kCarry + 1);
-    uint64_t *bar = keys + kCarry;
-    float *q = reinterpret_cast<float *>(sm + kRescoreWarps * (32 * kChunkStride * 4 + (kCarry + 1) * 8)) +
+    float *stage = reinterpret_cast<float *>(sm) + warp * 2 * 32 * kChunkStride;
+    uint64_t *keys = reinterpret_cast<uint64_t *>(sm + kRescoreWarps * 2 * 32 * kChunkStride * 4) + warp * kCarry;
+    float *q = reinterpret_cast<float *>(sm + kRescoreWarps * (2 * 32 * kChunkStride * 4 + kCarry * 8)) +
                warp * ((d + 3) & ~3u);
     const uint32_t u = source_row(row0 + lr, stride, n);
     const uint32_t m = w.n_carry[lr];
@@ -811,58 +822,69 @@ __global__ void __launch_bounds__(kRescoreWarps * 32)
         if (lane == 0) list[atomicAdd(&w.st->listed, 1u)] = u;
         return;
     }
-    if (lane == 0) mbar_init(bar, 1);
-    fence_mbar_init();
     for (uint32_t i = lane; i < d; i += 32) q[i] = X[(size_t)u * d + i];
-    __syncwarp();
     const uint2 *carry = w.carry + (size_t)lr * kCarry;
-    uint32_t phase = 0;
-    bool ok = true;
-    for (uint32_t b = 0; b < m && ok; b += 32) {
-        const bool mine = b + lane < m;
-        const uint32_t v = mine ? source_row(carry[b + lane].y, stride, n) : 0u;
-        const float *x = X + (size_t)v * d;
-        float acc = 0.0f;
-        for (uint32_t c0 = 0; c0 < d && ok; c0 += kChunk) {
-            const uint32_t len = min(kChunk, d - c0);
-            __syncwarp();   // the last chunk has been read
-            if (bulk) {
-                if (lane == 0) {
-                    fence_proxy_async();
-                    mbar_arrive_expect_tx(bar, min(32u, m - b) * len * 4);
-                }
-                __syncwarp();
-                if (mine) bulk_g2s(stage + lane * kChunkStride, x + c0, len * 4, bar);
-                ok = __all_sync(0xffffffffu, mbar_wait_bounded(bar, phase, &w.st->err));
-                phase ^= 1;
-            } else {
-                for (uint32_t r = 0; r < min(32u, m - b); ++r) {
-                    const float *xr = X + (size_t)__shfl_sync(0xffffffffu, v, r) * d + c0;
-                    for (uint32_t c = lane; c < len; c += 32) stage[r * kChunkStride + c] = __ldg(xr + c);
-                }
-                __syncwarp();
+    // steps of 32 columns by kChunk elements, the next one's copies in flight
+    // while one is computed
+    const uint32_t steps = (m + 31) / 32 * ((d + kChunk - 1) / kChunk);
+    uint32_t ib = 0, ic = 0, iv = 0;   // the step being copied: first column, first element, this lane's row
+    auto issue = [&](uint32_t buf) {
+        if (ic == 0) iv = source_row(carry[min(ib + lane, m - 1)].y, stride, n);
+        const uint32_t rows = min(32u, m - ib), len = min(kChunk, d - ic);
+        float *dst = stage + buf * 32 * kChunkStride;
+        if (wide) {   // 16-byte units: 8 lanes a row
+#pragma unroll
+            for (uint32_t r0 = 0; r0 < 32; r0 += 4) {
+                const uint32_t r = r0 + (lane >> 3), c = (lane & 7) * 4;
+                const uint32_t v = __shfl_sync(0xffffffffu, iv, r);
+                if (r < rows && c < len) copy_async<16>(dst + r * kChunkStride + c, X + (size_t)v * d + ic + c);
             }
-            const float *row = stage + lane * kChunkStride;
-            auto step = [&](float a, float y) {
-                const float df = __fsub_rn(a, y);
-                acc = __fmaf_rn(df, df, acc);
-            };
-            uint32_t c = 0;
+        } else {
 #pragma unroll 4
-            for (; c + 4 <= len; c += 4) {
-                const float4 xv = *reinterpret_cast<const float4 *>(row + c);
-                const float4 qv = *reinterpret_cast<const float4 *>(q + c0 + c);
-                step(qv.x, xv.x);
-                step(qv.y, xv.y);
-                step(qv.z, xv.z);
-                step(qv.w, xv.w);
+            for (uint32_t r = 0; r < rows; ++r) {
+                const uint32_t v = __shfl_sync(0xffffffffu, iv, r);
+                if (lane < len) copy_async<4>(dst + r * kChunkStride + lane, X + (size_t)v * d + ic + lane);
             }
-            for (; c < len; ++c) step(q[c0 + c], row[c]);
         }
-        if (mine) keys[b + lane] = ((uint64_t)__float_as_uint(acc) << 32) | v;   // non-negative: the bits order as the values
+        ic += kChunk;
+        if (ic >= d) { ic = 0; ib += 32; }
+    };
+    issue(0);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    float acc = 0.0f;
+    uint32_t b = 0, c0 = 0;   // the step being computed
+    for (uint32_t t = 0; t < steps; ++t) {
+        const uint32_t mine = iv;   // (the next batch's after the issue)
+        if (t + 1 < steps) issue((t + 1) & 1);
+        asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 1;" ::: "memory");
+        __syncwarp();
+        const float *row = stage + ((t & 1) * 32 + lane) * kChunkStride;
+        const uint32_t len = min(kChunk, d - c0);
+        auto step = [&](float a, float y) {
+            const float df = __fsub_rn(a, y);
+            acc = __fmaf_rn(df, df, acc);
+        };
+        uint32_t c = 0;
+#pragma unroll 4
+        for (; c + 4 <= len; c += 4) {
+            const float4 xv = *reinterpret_cast<const float4 *>(row + c);
+            const float4 qv = *reinterpret_cast<const float4 *>(q + c0 + c);
+            step(qv.x, xv.x);
+            step(qv.y, xv.y);
+            step(qv.z, xv.z);
+            step(qv.w, xv.w);
+        }
+        for (; c < len; ++c) step(q[c0 + c], row[c]);
+        c0 += kChunk;
+        if (c0 >= d) {
+            if (b + lane < m)   // non-negative: the bits order as the values
+                keys[b + lane] = ((uint64_t)__float_as_uint(acc) << 32) | mine;
+            acc = 0.0f;
+            c0 = 0;
+            b += 32;
+        }
+        __syncwarp();   // the step's buffer has been read
     }
-    if (!ok) return;   // the error word has every row done by the plain kernel
-    __syncwarp();
     for (uint32_t i = lane; i < m; i += 32) {
         const uint64_t k = keys[i];
         uint32_t r = 0;
@@ -999,9 +1021,9 @@ ann_status knn_filtered(const float *X, uint32_t n, uint32_t d, uint32_t K, uint
         run(cudaGetLastError());
         const size_t sel_smem = kSelectWarps * (w.entries * 8 + 1024);
         const size_t res_smem =
-            kRescoreWarps * (32 * kChunkStride * 4 + (kCarry + 1) * 8 + (size_t)((d + 3) & ~3u) * 4);
-        // bulk copies move whole 16-byte units from 16-byte boundaries
-        const uint32_t bulk = d % 4 == 0 && (reinterpret_cast<uintptr_t>(X) & 15u) == 0;
+            kRescoreWarps * (2 * 32 * kChunkStride * 4 + kCarry * 8 + (size_t)((d + 3) & ~3u) * 4);
+        // rows of whole 16-byte units
+        const bool wide = d % 4 == 0 && (reinterpret_cast<uintptr_t>(X) & 15u) == 0;
         run(cudaFuncSetAttribute(knn_select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sel_smem));
         run(cudaFuncSetAttribute(knn_rescore_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)res_smem));
         for (uint32_t row0 = 0; row0 < n && e == cudaSuccess; row0 += chunk_rows) {
@@ -1021,7 +1043,7 @@ ann_status knn_filtered(const float *X, uint32_t n, uint32_t d, uint32_t K, uint
                 t1 = (uint32_t)std::min<uint64_t>(n_tiles, (uint64_t)t1 * growth);
             }
             knn_rescore_kernel<<<grid_for(rows, kRescoreWarps), kRescoreWarps * 32, res_smem, st>>>(
-                X, n, d, K, stride, row0, rows, bulk, w, list, ids);
+                X, n, d, K, stride, row0, rows, wide, w, list, ids);
             run(cudaGetLastError());
         }
         knn_exact_kernel<<<std::min(grid_for(n, KQ), sms * 8), KW * 32, plain_smem, st>>>(X, n, d, K, ids, state, list);
