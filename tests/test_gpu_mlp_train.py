@@ -83,3 +83,42 @@ def test_an_epoch_equals_its_steps(n, batch):
         assert np.array_equal(p, q)
     a.close()
     b.close()
+
+
+@pytest.mark.parametrize("d,h1,h2,out,n", [(24, 200, 264, 1000, 264), (96, 512, 512, 4096, 1024), (8, 8, 8, 8, 8)])
+def test_overlapped_steps_are_ordered(d, h1, h2, out, n):
+    """A step uses a second stream: steps one after another without a wait, on
+    the default stream, on another one and as a captured graph, give the bits
+    that steps with a wait after each give, and the caller's stream waits for
+    all of a step's work."""
+    rng = np.random.default_rng(n)
+    X = torch.from_numpy(rng.standard_normal((n, d)).astype(np.float32)).cuda()
+    y = torch.from_numpy(rng.integers(0, out, n).astype(np.int32)).cuda()
+    steps, results = 6, []
+    for mode in ("wait", "default", "stream", "graph"):
+        _, g = make(d, h1, h2, out, 7)
+        go = lambda: g.train_step(X, y, lr=1e-3, weight_decay=0.01)
+        go()
+        torch.cuda.synchronize()
+        if mode == "stream":
+            with torch.cuda.stream(torch.cuda.Stream()):
+                for _ in range(steps):
+                    go()
+        elif mode == "graph":
+            graph = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(graph):
+                for _ in range(steps):
+                    go()
+            graph.replay()
+        else:
+            for _ in range(steps):
+                go()
+                if mode == "wait":
+                    torch.cuda.synchronize()
+        if mode == "stream":
+            torch.cuda.synchronize()
+        g.sync()
+        results.append([np.copy(a) for a in g.get(0)])
+    for other in results[1:]:
+        for a, b in zip(results[0], other):
+            assert np.array_equal(a, b)
