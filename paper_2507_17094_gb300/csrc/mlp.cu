@@ -1080,10 +1080,11 @@ struct ann_mlp {
     uint32_t step = 0;
     int *d_error = nullptr;
     int num_sms = 0;
-    // a training step's second stream and the events that tie it to the
-    // caller's (made with the training buffers)
-    cudaStream_t side = nullptr;
-    cudaEvent_t ev[3] = {};
+    // a training step's other streams and the events that tie them to the
+    // caller's (made with the training buffers; none of them, or all)
+    cudaStream_t side[2] = {};
+    cudaEvent_t ev[5] = {};
+    bool overlap = false;
 };
 
 namespace {
@@ -1256,11 +1257,10 @@ ann_status ensure_train_buffers(ann_mlp *m, uint32_t n)
     m->train_cap = n;
     for (cudaEvent_t &ev : m->ev)
         if (!ev && e == cudaSuccess) e = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming);
-    if (!m->side && e == cudaSuccess) e = cudaStreamCreateWithFlags(&m->side, cudaStreamNonBlocking);
-    if (e != cudaSuccess) {   // the step then runs on the caller's stream alone
-        m->side = nullptr;
-        cudaGetLastError();
-    }
+    for (cudaStream_t &side : m->side)
+        if (!side && e == cudaSuccess) e = cudaStreamCreateWithFlags(&side, cudaStreamNonBlocking);
+    m->overlap = e == cudaSuccess;   // else the step runs on the caller's stream alone
+    if (!m->overlap) cudaGetLastError();
     return ANN_OK;
 }
 
@@ -1294,12 +1294,14 @@ ann_status forward(ann_mlp *m, const float *x, const uint32_t *perm, uint32_t n,
 //
 // The hidden layers' gradients are a chain of products of few tiles (1,024 x
 // 512 x 10,000: 64 CTAs for 44 us), and nothing but the update waits for the
-// gradients of weights and biases: those run on a second stream, forked and
-// joined by events within the step, and the largest leaves the chain its SMs.
-// Measured, us a step on one stream / so: 96-512-512-10,000, batch 1,024: 236 /
-// 183, batch 256: 174 / 146; 96-64-64-512, batch 64: 77 / 60; 768-512-512-
-// 20,000, batch 4,096: 911 / 826. With the bias sums on a third stream they take
-// SMs that the chain's CTAs then wait for: 192.
+// gradients of weights and biases: those run on other streams, forked and
+// joined by events within the step, and the largest leaves the chain its SMs
+// (where the chain takes at most half of them; else it waits for free ones).
+// Measured, us a step on one stream / with a second: 96-512-512-10,000, batch
+// 1,024: 236 / 183, batch 256: 174 / 146; 96-64-64-512, batch 64: 77 / 60;
+// 768-512-512-20,000, batch 4,096: 911 / 826. The first layer's bias sum, after
+// the chain, on a third: 174 / 166. With the other bias sums there too, they
+// take SMs that the chain's CTAs then wait for: 183 -> 192.
 ann_status train_step(ann_mlp *m, const float *x, const uint32_t *labels, const uint32_t *perm, uint32_t n, float lr,
                       float beta1, float beta2, float eps, float weight_decay, cudaStream_t st)
 {
@@ -1318,11 +1320,12 @@ ann_status train_step(ann_mlp *m, const float *x, const uint32_t *labels, const 
         softmax_ce_kernel<<<(n + 7) / 8, 256, 0, st>>>(m->z, m->dzb, labels, perm, n, m->out, m->loss);
     }
     ANN_CUDA(cudaGetLastError());
-    const cudaStream_t side = m->side ? m->side : st;
-    auto after = [&](cudaStream_t waits, cudaStream_t on, cudaEvent_t ev) {   // `waits` goes on after what `on` has so far
-        if (waits == on) return cudaSuccess;
-        const cudaError_t e = cudaEventRecord(ev, on);
-        return e == cudaSuccess ? cudaStreamWaitEvent(waits, ev, 0) : e;
+    const cudaStream_t side = m->overlap ? m->side[0] : st, last = m->overlap ? m->side[1] : st;
+    cudaError_t ce = cudaSuccess;
+    auto after = [&](cudaStream_t waits, cudaStream_t on, int i) {   // `waits` goes on after what `on` has so far
+        if (!m->overlap) return;
+        const cudaError_t r = cudaEventRecord(m->ev[i], on), w = cudaStreamWaitEvent(waits, m->ev[i], 0);
+        if (ce == cudaSuccess) ce = r != cudaSuccess ? r : w;
     };
     auto colsum = [&](const float *g, float *out, uint32_t C, cudaStream_t on) {
         colsum_kernel<<<(C + kSumCols - 1) / kSumCols, 256, 0, on>>>(g, out, n, C);
@@ -1332,26 +1335,28 @@ ann_status train_step(ann_mlp *m, const float *x, const uint32_t *labels, const 
     EpiArgs e{};
     e.err = m->d_error;
     const uint32_t chain = (m->h2 + 63) / 64 * ((n + BM - 1) / BM);   // CTAs of the second layer's gradient
-    const uint32_t spare = side != st && 2 * chain <= (uint32_t)m->num_sms ? chain : 0;
-    cudaError_t ce = after(side, st, m->ev[0]);
+    const uint32_t spare = m->overlap && 2 * chain <= (uint32_t)m->num_sms ? chain : 0;
+    after(side, st, 0);
     if (ce != cudaSuccess) return cuda_fail(ce, "MLP training step");
     e.c = da2; e.ldc = m->h2; e.cb = da2b; e.mask = m->h2b;
     s = gemm<EPI_MASK, false, true>(m->dzb, m->Wb[2], n, m->h2, m->out, e, st);
     e.c = m->gW[2];
     if (s == ANN_OK) s = gemm<EPI_F32, true, true>(m->dzb, m->h2b, m->out, m->h2, n, e, side, spare);
     colsum(m->z, m->gb[2], m->out, side);
-    ce = after(side, st, m->ev[1]);
+    after(side, st, 1);
     e.c = da1; e.ldc = m->h1; e.cb = da1b; e.mask = m->h1b;
     if (s == ANN_OK) s = gemm<EPI_MASK, false, true>(da2b, m->Wb[1], n, m->h1, m->h2, e, st);
     e.c = m->gW[1];
     if (s == ANN_OK) s = gemm<EPI_F32, true, true>(da2b, m->h1b, m->h2, m->h1, n, e, side);
     colsum(da2, m->gb[1], m->h2, side);
+    after(last, st, 2);
     e.c = m->gW[0]; e.ldc = m->d;
     if (s == ANN_OK) s = gemm<EPI_F32, true, true>(da1b, m->xb, m->h1, m->d, n, e, st);
-    colsum(da1, m->gb[0], m->h1, st);
-    const cudaError_t joined = after(st, side, m->ev[2]);
+    colsum(da1, m->gb[0], m->h1, last);
+    after(st, side, 3);
+    after(st, last, 4);
     if (s != ANN_OK) return s;   // joined all the same
-    if (ce != cudaSuccess || joined != cudaSuccess) return cuda_fail(ce != cudaSuccess ? ce : joined, "MLP training step");
+    if (ce != cudaSuccess) return cuda_fail(ce, "MLP training step");
     m->step++;
     const AdamHP h{lr, beta1, beta2, eps, weight_decay, (float)(1.0 - std::pow((double)beta1, (double)m->step)),
                    (float)(1.0 - std::pow((double)beta2, (double)m->step))};
@@ -1379,7 +1384,7 @@ void mlp_free_all(ann_mlp *m)
                  m->epoch_loss, m->mean, m->inv_std};
     for (void *x : q) if (x) cudaFree(x);
     for (cudaEvent_t ev : m->ev) if (ev) cudaEventDestroy(ev);
-    if (m->side) cudaStreamDestroy(m->side);
+    for (cudaStream_t side : m->side) if (side) cudaStreamDestroy(side);
 }
 
 }  // namespace
