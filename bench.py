@@ -42,7 +42,7 @@ METRIC = "QPS at recall@10>=0.95 on 1 GB300: plain FP32 vs FP16/FP8+learned entr
 UNIT = "queries/s"
 RECALL_TARGET = 0.95
 SWEEP = (16, 32, 64, 128, 256)
-KERNEL_SOURCES = ("paper_2507_17094_gb300/csrc/search.cu", "paper_2507_17094_gb300/csrc/ann_internal.cuh")
+KERNEL_SOURCES = tuple("paper_2507_17094_gb300/csrc/" + f for f in ("search.cu", "search_common.cuh", "ann_internal.cuh"))
 
 
 # ------------------------------------------------------------------ helpers
