@@ -63,12 +63,16 @@ __device__ __forceinline__ void write_order(uint32_t *det, const uint32_t (&mine
 // is a table of 4,096 ranks in shared memory under a multiplicative hash chosen
 // per node so that the list's ids fall into different slots (a random multiplier
 // does for 96 ids in one try of three), and a comparison with the id of that
-// rank: no probing, so the lanes of a warp never diverge. Four second-hop lists
-// are gathered at once (K x K x 4 bytes a node, half of them from DRAM at
-// 500,000 x 96). Measured there: a binary search of a sorted copy of the list
-// 16.0 ms, linear probing 9.3 ms (40 instructions a lookup: some lane always
-// probes on), this 5.2 ms.
+// rank: no probing, so the lanes of a warp never diverge. Eight second-hop
+// lists are gathered at once (K x K x 4 bytes a node, half of them from DRAM at
+// 500,000 x 96) by one loop over the ranks: unrolled over the lane's NW words as
+// well, its code left the instruction cache (128 entries: 8.7 ms against 6.0
+// for 300,000 nodes). Measured at 500,000 x 96: a binary search of a sorted copy
+// of the list 16.0 ms, linear probing 9.3 ms (40 instructions a lookup: some
+// lane always probes on), this 3.9 ms (2, 4, 8 lists at once 5.9, 5.6, 5.5 ms for
+// the whole pruning).
 constexpr uint32_t kRankSlots = 4096, kNoRank = 128;
+constexpr uint32_t kLists = 8;          // second-hop lists gathered at once
 constexpr uint32_t kHashTries = 64;   // multipliers tried; a list none of them keeps apart is searched in order
 
 template <uint32_t NW>
@@ -133,31 +137,40 @@ __global__ void __launch_bounds__(256) detour_rank_kernel(const uint32_t *__rest
         __syncwarp();
     }
     __syncwarp();
+    // entry c of the list of the node ranked p
+    auto entry = [&](uint32_t p, uint32_t c) {
+        const uint32_t w = ids[p];
+        return w < n && lane + 32 * c < K ? __ldg(knn + (size_t)w * K + lane + 32 * c) : ANN_INVALID_ID;
+    };
+    // an unused slot's rank is the marker: its id matches only an invalid
+    // entry, counted where nothing reads
+    auto count = [&](uint32_t p, uint32_t c, uint32_t x, uint32_t r) {
+        if (ids[r] == x && max(p, last[c]) < r) atomicAdd(&det[r], 1u);
+    };
+    if (apart) {
+        #pragma unroll 1
+        for (uint32_t p = 0; p < K; p += kLists) {   // past K the ids are invalid
+            uint32_t x[kLists][NW];
 #pragma unroll
-    for (uint32_t i = 0; i < NW; ++i) {
-#pragma unroll 1
-        for (uint32_t l0 = 0; l0 < 32 && 32 * i + l0 < K; l0 += 4) {
-            uint32_t x[4][NW];
+            for (uint32_t j = 0; j < kLists; ++j)
 #pragma unroll
-            for (uint32_t j = 0; j < 4; ++j) {
-                const uint32_t w = __shfl_sync(0xffffffffu, mine[i], l0 + j);   // past K: invalid
+                for (uint32_t c = 0; c < NW; ++c) x[j][c] = entry(p + j, c);
 #pragma unroll
-                for (uint32_t c = 0; c < NW; ++c)
-                    x[j][c] = w < n && lane + 32 * c < K ? __ldg(knn + (size_t)w * K + lane + 32 * c) : ANN_INVALID_ID;
-            }
+            for (uint32_t j = 0; j < kLists; ++j)
 #pragma unroll
-            for (uint32_t j = 0; j < 4; ++j)
-#pragma unroll
-                for (uint32_t c = 0; c < NW; ++c) {
-                    uint32_t r = kNoRank;
-                    if (apart) r = tab[(x[j][c] * mul) >> 20];
-                    else
-                        for (uint32_t k = K; k-- > 0;) r = ids[k] == x[j][c] ? k : r;
-                    // an unused slot's rank is the marker: its id matches only
-                    // an invalid entry, counted where nothing reads
-                    if (ids[r] == x[j][c] && max(32 * i + l0 + j, last[c]) < r) atomicAdd(&det[r], 1u);
-                }
+                for (uint32_t c = 0; c < NW; ++c) count(p + j, c, x[j][c], tab[(x[j][c] * mul) >> 20]);
         }
+    } else {
+        #pragma unroll 1
+        for (uint32_t p = 0; p < K; ++p)
+#pragma unroll
+            for (uint32_t c = 0; c < NW; ++c) {
+                const uint32_t x = entry(p, c);
+                uint32_t r = kNoRank;
+                #pragma unroll 1
+                for (uint32_t k = K; k-- > 0;) r = ids[k] == x ? k : r;
+                count(p, c, x, r);
+            }
     }
     write_order<NW>(det, mine, K, lane, ordered + (size_t)u * K);
 }
@@ -236,9 +249,9 @@ __global__ void __launch_bounds__(256) detour_order_kernel(const uint32_t *__res
 
 cudaError_t launch_detours(const uint32_t *knn, uint32_t n, uint32_t K, uint32_t *ordered, cudaStream_t st)
 {
-    constexpr uint32_t warps = 8;
-    const uint32_t grid = (n + warps - 1) / warps;
-    auto go = [&](auto kernel, size_t per_warp) {
+    // blocks of four warps pack 44 of the rank tables on an SM, of eight 40
+    auto go = [&](auto kernel, size_t per_warp, uint32_t warps) {
+        const uint32_t grid = (n + warps - 1) / warps;
         const size_t smem = warps * per_warp;
         cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
@@ -248,12 +261,12 @@ cudaError_t launch_detours(const uint32_t *knn, uint32_t n, uint32_t K, uint32_t
     constexpr size_t ranks = kRankSlots + 2 * (kNoRank + 4) * 4;
     auto probing = [](uint32_t nw) { return (size_t)1024 * 5 + nw * 32 * 4; };
     switch ((K + 31) / 32) {
-    case 1: return go(detour_rank_kernel<1>, ranks);
-    case 2: return go(detour_rank_kernel<2>, ranks);
-    case 3: return go(detour_rank_kernel<3>, ranks);
-    case 4: return go(detour_rank_kernel<4>, ranks);
-    case 5: case 6: return go(detour_order_kernel<6>, probing(6));
-    default: return go(detour_order_kernel<8>, probing(8));
+    case 1: return go(detour_rank_kernel<1>, ranks, 4);
+    case 2: return go(detour_rank_kernel<2>, ranks, 4);
+    case 3: return go(detour_rank_kernel<3>, ranks, 4);
+    case 4: return go(detour_rank_kernel<4>, ranks, 4);
+    case 5: case 6: return go(detour_order_kernel<6>, probing(6), 8);
+    default: return go(detour_order_kernel<8>, probing(8), 8);
     }
 }
 
