@@ -104,7 +104,7 @@ struct ServeRing {
     const uint32_t *slot_req;        // cap: request-ring index of each slot (host)
     const ServeReq *reqs;            // host
     uint32_t *done;                  // per request record: queries finished (device; zero between requests)
-    unsigned long long *counters;    // device: [0] queries taken, [1] queries made available, [2] their difference
+    unsigned long long *counters;    // device: the counts of serve_take.cuh
     unsigned long long tail;         // queries published before this launch
     const unsigned long long *live;  // queries published so far (host), for a launch that makes later ones available; or NULL
     volatile uint32_t *flags;        // completion flags (host)

@@ -58,6 +58,7 @@
 #include <vector>
 
 #include "search_common.cuh"
+#include "serve_take.cuh"
 
 using namespace ann;
 
@@ -1013,6 +1014,21 @@ __global__ void __launch_bounds__(128, kSearchBlocksPerSm) search_kernel(const A
     }
 }
 
+// The counts as lane 0 of a warp sees them (serve_take.cuh).
+struct ServeCounts {
+    static constexpr uint32_t kLooks = 1u << 18;   // some tenths of a second
+    unsigned long long *c;
+    int *err;
+    __device__ __forceinline__ unsigned long long load(uint32_t i) const
+    {
+        return *reinterpret_cast<volatile unsigned long long *>(c + i);
+    }
+    __device__ __forceinline__ unsigned long long add(uint32_t i, unsigned long long x) { return atomicAdd(c + i, x); }
+    __device__ __forceinline__ unsigned long long max(uint32_t i, unsigned long long x) { return atomicMax(c + i, x); }
+    __device__ __forceinline__ void fence() { __threadfence(); }
+    __device__ __forceinline__ void gave_up() { atomicExch(err, ANN_DEV_TIMEOUT); }
+};
+
 // Continuous batching: warps of every running serve kernel take queries, in
 // arrival order, from one ring (monotonic query counters; slot = counter mod
 // capacity). A launch makes available the queries published before it and, with
@@ -1024,38 +1040,6 @@ __global__ void __launch_bounds__(128, kSearchBlocksPerSm) search_kernel(const A
 // is queued for them. The request's parameters are copied into the warp's shared
 // memory; the warp that finishes a request's last query raises its completion
 // flag after a system-scope fence.
-//
-// Taking a query is two additions: one to the count of available queries, given
-// back if there was none, and one to the count of those taken. (A compare and
-// swap of the latter fails for all but one of the warps that try together: 3,000
-// queries took 2.7 ms, 0.9 of which was searching.) A warp that gave back looks
-// again before it leaves: of several that fail together the last to give back
-// sees what the others hid, so no available query is left behind.
-
-// Make the queries up to `tail` available; lane 0 only.
-__device__ __forceinline__ void serve_publish(const ServeRing &r, unsigned long long tail)
-{
-    if (tail <= *reinterpret_cast<volatile unsigned long long *>(r.counters + 1)) return;
-    __threadfence();   // what `tail` counts, before the counts
-    const unsigned long long was = atomicMax(r.counters + 1, tail);
-    if (was < tail) atomicAdd(r.counters + 2, tail - was);
-}
-
-// Take the next query: true and its counter in *h; lane 0 only.
-__device__ __forceinline__ bool serve_take(const ServeRing &r, unsigned long long *h)
-{
-    for (uint32_t attempt = 0; attempt < (1u << 20); ++attempt) {
-        if ((long long)atomicAdd(r.counters + 2, ~0ull) > 0) {
-            *h = atomicAdd(r.counters, 1ull);
-            __threadfence();
-            return true;
-        }
-        atomicAdd(r.counters + 2, 1ull);
-        if ((long long)*reinterpret_cast<volatile unsigned long long *>(r.counters + 2) <= 0) break;
-    }
-    return false;
-}
-
 template <int ST, int LPR = 2>
 __global__ void __launch_bounds__(128, kSearchBlocksPerSm) serve_kernel(const Args a, const ServeRing r)
 {
@@ -1067,16 +1051,17 @@ __global__ void __launch_bounds__(128, kSearchBlocksPerSm) serve_kernel(const Ar
     if (lane == 0) mbar_init(ws.bar(), 1);
     fence_mbar_init();
     __syncwarp();
+    ServeCounts counts{r.counters, a.err};
     if (lane == 0) {
         unsigned long long tail = r.tail;
         if (r.live)   // acquire: what it counts was written before it
             asm volatile("ld.acquire.sys.global.u64 %0, [%1];" : "=l"(tail) : "l"(r.live) : "memory");
-        serve_publish(r, tail);
+        serve_publish(counts, tail);
     }
     for (uint32_t served = 0; served < r.per_warp; ++served) {
         unsigned long long h = 0;
         uint32_t got = 0;
-        if (lane == 0) got = serve_take(r, &h);
+        if (lane == 0) got = serve_take(counts, &h);
         got = __shfl_sync(0xffffffffu, got, 0);
         if (!got) break;
         h = __shfl_sync(0xffffffffu, h, 0);
