@@ -1053,10 +1053,10 @@ __global__ void __launch_bounds__(128, kSearchBlocksPerSm) serve_kernel(const Ar
     __syncwarp();
     ServeCounts counts{r.counters, a.err};
     if (lane == 0) {
-        unsigned long long tail = r.tail;
+        unsigned long long live = 0;
         if (r.live)   // acquire: what it counts was written before it
-            asm volatile("ld.acquire.sys.global.u64 %0, [%1];" : "=l"(tail) : "l"(r.live) : "memory");
-        serve_publish(counts, tail);
+            asm volatile("ld.acquire.sys.global.u64 %0, [%1];" : "=l"(live) : "l"(r.live) : "memory");
+        serve_publish(counts, serve_tail(r.tail, live));
     }
     for (uint32_t served = 0; served < r.per_warp; ++served) {
         unsigned long long h = 0;

@@ -296,8 +296,10 @@ ann_status ann_server_submit(ann_server *s, uint64_t req_id, const float *querie
             if (busy == cudaErrorNotReady) cudaGetLastError();
             else e = busy;
             if (e == cudaSuccess) {
-                __atomic_store_n(s->host<uint64_t>(s->o_tail), s->tail + nq, __ATOMIC_RELEASE);
                 st = serve_launch(s->plan, r, warps, pending, c, si);
+                // only now: queued launches publish what they read here, and a
+                // request whose launch was refused is not one of the server's
+                if (st == ANN_OK) __atomic_store_n(s->host<uint64_t>(s->o_tail), s->tail + nq, __ATOMIC_RELEASE);
             }
         }
     }

@@ -21,6 +21,13 @@ namespace ann {
 
 enum ServeCount : uint32_t { kServeTaken = 0, kServePublished, kServeFree, kServeCounts };
 
+// The tail that a launch publishes: its own, which covers its request, or what
+// the host has published since (`live`, 0 if the launch takes no later queries).
+ANN_SERVE_FN unsigned long long serve_tail(unsigned long long own, unsigned long long live)
+{
+    return live > own ? live : own;
+}
+
 // Make the queries up to `tail` available.
 template <typename Counts>
 ANN_SERVE_FN void serve_publish(Counts &c, unsigned long long tail)
