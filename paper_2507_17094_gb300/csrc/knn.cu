@@ -29,8 +29,9 @@
 // more each time), so a row sees about K (growth - 1) survivors per range
 // whatever n is. Survivor buffers have a fixed size: a row that overflows one
 // (many equal distances), and every row if the input holds a value the FP16
-// operands cannot bound (infinities, NaN), is done by knn_exact_kernel, the
-// plain computation, which also serves small inputs.
+// operands cannot bound (infinities, NaN, magnitudes near either end of FP32's
+// range), is done by knn_exact_kernel, the plain computation, which also serves
+// small inputs.
 //
 // Bounds. With x' the centred rows, |x' - fp16(x')| <= delta |x'| + eta
 // measured over all rows (eta: FP16 subnormals), the product's error is at
@@ -40,6 +41,12 @@
 // the order of d 2^-24. So |approx - exact| <= c (N_u + N_v) + kappa, and the
 // test of column v against row u needs one number per column and one per row:
 // (1 - c) N_v - 2 dot(u, v) <= T_u.
+//
+// That holds while the exact distance neither overflows nor loses bits among
+// the subnormal numbers. With the largest |x'| below 2^(e + 1), a distance is
+// below d 2^(2 e + 4), and its subnormal roundings add at most d 2^-150, which
+// is d 2^(-122 - 2 e) in the operands' units and has to vanish in kappa. Both
+// hold with room for -50 <= e <= 50 (kExponent) and any d that is taken.
 #include <algorithm>
 #include <cfloat>
 #include <cmath>
@@ -250,6 +257,14 @@ __global__ void knn_centre_kernel(const float *__restrict__ X, size_t total, uin
     if ((threadIdx.x & 31) == 0) atomicMax(&st->max, mx);
 }
 
+// Whether the bounds hold for rows whose largest |x'| has the bits mb.
+constexpr int kExponent = 50;
+__device__ __forceinline__ bool in_range(uint32_t mb)
+{
+    const int e = (int)(mb >> 23) - 127;
+    return mb == 0 || (e >= -kExponent && e <= kExponent);
+}
+
 // The FP16 operand row j (row stride ld >= d elements, zero past d), scaled
 // so that the largest magnitude lies in [2^14, 2^15), its squared norm in
 // those units, and the relative rounding error. One warp per row.
@@ -261,8 +276,8 @@ __global__ void knn_operand_kernel(const float *__restrict__ X, uint32_t n, uint
     for (uint32_t c = threadIdx.x; c < d; c += blockDim.x) mu[c] = centre(sum[c], samples, st->sample_max);
     __syncthreads();
     const uint32_t mb = st->max;
+    if (!in_range(mb)) return;   // knn_bound_kernel leaves every row to the plain kernel
     const int e = (int)(mb >> 23) - 127;
-    if (mb && (e < -60 || e > 60)) return;   // knn_bound_kernel leaves every row to the plain kernel
     const float s = mb ? exp2f((float)(14 - e)) : 1.0f;
     const uint32_t lane = threadIdx.x & 31;
     const float eta = sqrtf((float)d) * 2.98023224e-8f;   // 2^-25 per element: half an FP16 subnormal step
@@ -306,9 +321,7 @@ __global__ void knn_bound_kernel(const float *__restrict__ norm, uint32_t n, uin
                                  float *__restrict__ lower, KnnState *st)
 {
     const float c = bound_c(st, d);
-    const uint32_t mb = st->max;
-    const int e = (int)(mb >> 23) - 127;
-    const bool bad = (mb && (e < -60 || e > 60)) || !(c < 0.25f);
+    const bool bad = !in_range(st->max) || !(c < 0.25f);
     for (uint32_t j = blockIdx.x * blockDim.x + threadIdx.x; j < n_pad; j += gridDim.x * blockDim.x)
         lower[j] = j < n ? (1.0f - c) * norm[j] : INFINITY;
     if (bad && blockIdx.x == 0 && threadIdx.x == 0) st->all = 1;
