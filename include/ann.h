@@ -271,7 +271,8 @@ ann_status ann_shards_search(ann_shards *shards, const float *queries, uint32_t 
  * per row of a chunk of 39,000 rows) and does without if it cannot have it. */
 ann_status ann_knn_exact(const float *X, uint64_t n, uint32_t dim, uint32_t K, uint32_t *ids, void *stream);
 /* Prune kNN lists (device, n x K; each row distinct ids, ANN_INVALID_ID
- * allowed) to a fixed-degree graph (device, n x degree): edge u -> v at rank
+ * allowed, which is no edge and has no detours) to a fixed-degree graph (device,
+ * n x degree): edge u -> v at rank
  * r is detoured via the node at rank a < r of u's list when v sits in that
  * node's list at a rank c < r; u's list is ordered by (number of detours,
  * rank) and its first degree / 2 entries are kept; every kept edge w -> v,

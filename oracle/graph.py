@@ -11,7 +11,8 @@ tooling under workloads/:
    FP64, ordered by (distance, id);
 2. detour count: edge u -> v at rank r of u's list is detoured via the node
    w at rank a < r of u's list when v appears in w's own list at a rank
-   c < r; det(r) counts such (a, c) pairs;
+   c < r; det(r) counts such (a, c) pairs. An INVALID entry is no edge: it
+   has no detours, and is none's;
 3. order u's list by (det, rank) and keep the first half = degree // 2
    edges (the least detoured);
 4. reverse edges: every kept edge w -> v (at position p of w's kept list)
@@ -57,7 +58,7 @@ def detour_counts(knn: np.ndarray) -> np.ndarray:
                 continue
             for c in range(K):
                 x = int(knn[w, c])
-                r = rank.get(x)
+                r = None if x == INVALID else rank.get(x)
                 if r is not None and a < r and c < r:
                     det[u, r] += 1
     return det

@@ -168,7 +168,7 @@ __global__ void __launch_bounds__(256) detour_rank_kernel(const uint32_t *__rest
                 const uint32_t x = entry(p, c);
                 uint32_t r = kNoRank;
                 #pragma unroll 1
-                for (uint32_t k = K; k-- > 0;) r = ids[k] == x ? k : r;
+                for (uint32_t k = K; k-- > 0;) r = ids[k] == x && x != ANN_INVALID_ID ? k : r;   // invalid: no edge
                 count(p, c, x, r);
             }
     }
