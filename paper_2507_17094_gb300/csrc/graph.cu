@@ -253,7 +253,7 @@ cudaError_t launch_detours(const uint32_t *knn, uint32_t n, uint32_t K, uint32_t
     auto go = [&](auto kernel, size_t per_warp, uint32_t warps) {
         const uint32_t grid = (n + warps - 1) / warps;
         const size_t smem = warps * per_warp;
-        cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaError_t e = raise_shared_limit(kernel, smem);   // each kernel's own constant
         if (e != cudaSuccess) return e;
         kernel<<<grid, warps * 32, smem, st>>>(knn, n, K, ordered);
         return cudaGetLastError();
@@ -472,9 +472,10 @@ ann_status ann_graph_prune(const uint32_t *knn, uint64_t n, uint32_t K, uint32_t
     if (e == cudaSuccess) e = cudaMemsetAsync(ws, 0, zeroed, st);
     const uint32_t L = K + (degree - half);
     constexpr int wpb = 8;
-    const size_t asm_smem = wpb * ((kOfferMax + assemble_slots(L)) * 8 + (size_t)L * 4);
+    constexpr auto asm_bytes = [](uint32_t len) { return wpb * ((kOfferMax + assemble_slots(len)) * 8 + (size_t)len * 4); };
+    const size_t asm_smem = asm_bytes(L);
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(assemble_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)asm_smem);
+        e = raise_shared_limit(assemble_kernel, asm_bytes(2 * ANN_MAX_DEGREE + (ANN_MAX_DEGREE + 1) / 2));
     if (e == cudaSuccess) e = launch_detours(knn, nn, K, ordered, st);
     if (e == cudaSuccess) {
         offer_count_kernel<<<grid_for((uint64_t)n * half, 256), 256, 0, st>>>(ordered, nn, K, half, cnt);

@@ -926,11 +926,10 @@ uint32_t gcd(uint32_t a, uint32_t b)
 }
 
 template <int NSUB, bool FIRST>
-cudaError_t launch_filter(const CUtensorMap &map, uint32_t blocks, size_t smem, uint32_t n, uint32_t nkb, uint32_t row0,
-                          uint32_t t0, uint32_t t1, const KnnWork &w, cudaStream_t st)
+cudaError_t launch_filter(const CUtensorMap &map, uint32_t blocks, size_t smem, int optin, uint32_t n, uint32_t nkb,
+                          uint32_t row0, uint32_t t0, uint32_t t1, const KnnWork &w, cudaStream_t st)
 {
-    cudaError_t e =
-        cudaFuncSetAttribute(knn_filter_kernel<NSUB, FIRST>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = raise_shared_limit(knn_filter_kernel<NSUB, FIRST>, optin);
     if (e != cudaSuccess) return e;
     knn_filter_kernel<NSUB, FIRST><<<blocks, kFilterThreads, smem, st>>>(map, n, nkb, row0, t0, t1, w);
     return cudaGetLastError();
@@ -1037,8 +1036,8 @@ ann_status knn_filtered(const float *X, uint32_t n, uint32_t d, uint32_t K, uint
             kRescoreWarps * (2 * 32 * kChunkStride * 4 + kCarry * 8 + (size_t)((d + 3) & ~3u) * 4);
         // rows of whole 16-byte units
         const bool wide = d % 4 == 0 && (reinterpret_cast<uintptr_t>(X) & 15u) == 0;
-        run(cudaFuncSetAttribute(knn_select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sel_smem));
-        run(cudaFuncSetAttribute(knn_rescore_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)res_smem));
+        run(raise_shared_limit(knn_select_kernel, optin));
+        run(raise_shared_limit(knn_rescore_kernel, optin));
         for (uint32_t row0 = 0; row0 < n && e == cudaSuccess; row0 += chunk_rows) {
             const uint32_t rows = std::min(chunk_rows, n - row0);
             const uint32_t blocks = (rows + block_rows - 1) / block_rows;
@@ -1049,7 +1048,7 @@ ann_status knn_filtered(const float *X, uint32_t n, uint32_t d, uint32_t K, uint
                 const uint32_t first = t0 == 0;
                 const auto launch = nsub == 2 ? (first ? launch_filter<2, true> : launch_filter<2, false>)
                                               : (first ? launch_filter<1, true> : launch_filter<1, false>);
-                run(launch(map, blocks * w.S, filter_smem, n, nkb, row0, t0, t1, w, st));
+                run(launch(map, blocks * w.S, filter_smem, optin, n, nkb, row0, t0, t1, w, st));
                 knn_select_kernel<<<grid_for(rows, kSelectWarps), kSelectWarps * 32, sel_smem, st>>>(
                     n, d, K, row0, rows, first, w);
                 t0 = t1;
@@ -1087,7 +1086,7 @@ ann_status ann_knn_exact(const float *X, uint64_t n, uint32_t dim, uint32_t K, u
         set_error("ann_knn_exact: %zu bytes of shared memory needed (dim %u, K %u), %d available", smem, dim, K, optin);
         return ANN_EINVAL;
     }
-    ANN_CUDA(cudaFuncSetAttribute(knn_exact_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    ANN_CUDA(raise_shared_limit(knn_exact_kernel, optin));
     if (n >= kFilterMin && n < (1ull << 31)) {
         const ann_status s = knn_filtered(X, (uint32_t)n, dim, K, ids, smem, dev, optin, (cudaStream_t)stream);
         if (s != ANN_ENOMEM) return s;

@@ -1314,7 +1314,7 @@ ann_status train_step(ann_mlp *m, const float *x, const uint32_t *labels, const 
     constexpr size_t kRowMax = 200 * 1024;
     const size_t row = (size_t)m->out * 4;
     if (row <= kRowMax) {
-        ANN_CUDA(cudaFuncSetAttribute(softmax_ce_block_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)row));
+        ANN_CUDA(raise_shared_limit(softmax_ce_block_kernel, kRowMax));
         softmax_ce_block_kernel<<<n, 256, row, st>>>(m->z, m->dzb, labels, perm, n, m->out, m->loss);
     } else {
         softmax_ce_kernel<<<(n + 7) / 8, 256, 0, st>>>(m->z, m->dzb, labels, perm, n, m->out, m->loss);

@@ -1123,35 +1123,34 @@ Layout make_layout(uint32_t q_floats, uint32_t cap_buf, uint32_t cap_cand, uint3
 }
 
 template <int ST, bool PROF, int LPR>
-cudaError_t launch_lpr(const Args &a, int warps, int blocks, size_t smem, cudaStream_t st)
+cudaError_t launch_lpr(const Args &a, int warps, int blocks, size_t smem, size_t optin, cudaStream_t st)
 {
-    cudaError_t e =
-        cudaFuncSetAttribute(search_kernel<ST, PROF, LPR>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = raise_shared_limit(search_kernel<ST, PROF, LPR>, optin);
     if (e != cudaSuccess) return e;
     search_kernel<ST, PROF, LPR><<<blocks, warps * 32, smem, st>>>(a);
     return cudaGetLastError();
 }
 
 template <int ST, bool PROF = false>
-cudaError_t launch(const Args &a, int warps, int blocks, size_t smem, cudaStream_t st)
+cudaError_t launch(const Args &a, int warps, int blocks, size_t smem, size_t optin, cudaStream_t st)
 {
-    return a.lpr == 4 ? launch_lpr<ST, PROF, 4>(a, warps, blocks, smem, st)
-                      : launch_lpr<ST, PROF, 2>(a, warps, blocks, smem, st);
+    return a.lpr == 4 ? launch_lpr<ST, PROF, 4>(a, warps, blocks, smem, optin, st)
+                      : launch_lpr<ST, PROF, 2>(a, warps, blocks, smem, optin, st);
 }
 
 template <int ST, int LPR>
-int blocks_per_sm_lpr(int warps, size_t smem)
+int blocks_per_sm_lpr(int warps, size_t smem, size_t optin)
 {
     int nb = 0;
-    cudaFuncSetAttribute(search_kernel<ST, false, LPR>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    raise_shared_limit(search_kernel<ST, false, LPR>, optin);
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, search_kernel<ST, false, LPR>, warps * 32, smem);
     return nb;
 }
 
 template <int ST>
-int blocks_per_sm(int warps, size_t smem, uint32_t lpr)
+int blocks_per_sm(int warps, size_t smem, size_t optin, uint32_t lpr)
 {
-    return lpr == 4 ? blocks_per_sm_lpr<ST, 4>(warps, smem) : blocks_per_sm_lpr<ST, 2>(warps, smem);
+    return lpr == 4 ? blocks_per_sm_lpr<ST, 4>(warps, smem, optin) : blocks_per_sm_lpr<ST, 2>(warps, smem, optin);
 }
 
 int env_int(const char *name, int dflt)
@@ -1318,9 +1317,9 @@ ann_status plan_shape(ann_index *ix, Args &a, uint64_t nq, bool serve, int &warp
             sh.smem = (size_t)sh.lay.total * sh.warps;
             if (sh.smem > ix->smem_optin) continue;
             switch (ix->storage) {
-            case ANN_F32: sh.nb = blocks_per_sm<ANN_F32>(sh.warps, sh.smem, lpr); break;
-            case ANN_F16: sh.nb = blocks_per_sm<ANN_F16>(sh.warps, sh.smem, lpr); break;
-            default: sh.nb = blocks_per_sm<ANN_E4M3>(sh.warps, sh.smem, lpr); break;
+            case ANN_F32: sh.nb = blocks_per_sm<ANN_F32>(sh.warps, sh.smem, ix->smem_optin, lpr); break;
+            case ANN_F16: sh.nb = blocks_per_sm<ANN_F16>(sh.warps, sh.smem, ix->smem_optin, lpr); break;
+            default: sh.nb = blocks_per_sm<ANN_E4M3>(sh.warps, sh.smem, ix->smem_optin, lpr); break;
             }
             // A server's warps take and finish queries one by one, and a block
             // holds its shared memory until its last warp is done: single
@@ -1383,7 +1382,7 @@ ann_status plan_shape(ann_index *ix, Args &a, uint64_t nq, bool serve, int &warp
 struct ServePlanImpl {
     Args a;
     int warps, nb, num_sms, storage;
-    size_t smem;
+    size_t smem, smem_optin;
     ann_visited_pool visited;     // the plan's own tables: n_streams launches at once
     uint32_t slots_per_launch;
 };
@@ -1391,8 +1390,7 @@ struct ServePlanImpl {
 template <int ST, int LPR>
 cudaError_t launch_serve_lpr(const ServePlanImpl &pl, const ServeRing &r, int blocks, cudaStream_t st)
 {
-    cudaError_t e =
-        cudaFuncSetAttribute(serve_kernel<ST, LPR>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pl.smem);
+    cudaError_t e = raise_shared_limit(serve_kernel<ST, LPR>, pl.smem_optin);
     if (e != cudaSuccess) return e;
     serve_kernel<ST, LPR><<<blocks, pl.warps * 32, pl.smem, st>>>(pl.a, r);
     return cudaGetLastError();
@@ -1464,15 +1462,15 @@ ann_status search_launch_ex(ann_index *ix, const float *queries, uint32_t nq, co
     cudaError_t e;
     if (prof) {
         switch (ix->storage) {
-        case ANN_F32: e = launch<ANN_F32, true>(a, warps, blocks, smem, stream); break;
-        case ANN_F16: e = launch<ANN_F16, true>(a, warps, blocks, smem, stream); break;
-        default: e = launch<ANN_E4M3, true>(a, warps, blocks, smem, stream); break;
+        case ANN_F32: e = launch<ANN_F32, true>(a, warps, blocks, smem, ix->smem_optin, stream); break;
+        case ANN_F16: e = launch<ANN_F16, true>(a, warps, blocks, smem, ix->smem_optin, stream); break;
+        default: e = launch<ANN_E4M3, true>(a, warps, blocks, smem, ix->smem_optin, stream); break;
         }
     } else {
         switch (ix->storage) {
-        case ANN_F32: e = launch<ANN_F32>(a, warps, blocks, smem, stream); break;
-        case ANN_F16: e = launch<ANN_F16>(a, warps, blocks, smem, stream); break;
-        default: e = launch<ANN_E4M3>(a, warps, blocks, smem, stream); break;
+        case ANN_F32: e = launch<ANN_F32>(a, warps, blocks, smem, ix->smem_optin, stream); break;
+        case ANN_F16: e = launch<ANN_F16>(a, warps, blocks, smem, ix->smem_optin, stream); break;
+        default: e = launch<ANN_E4M3>(a, warps, blocks, smem, ix->smem_optin, stream); break;
         }
     }
     if (e != cudaSuccess) return cuda_fail(e, "search_kernel launch");
@@ -1501,6 +1499,7 @@ ann_status serve_plan(ann_index *ix, const ann_search_params *maxp, uint32_t n_g
     pl->a.counter = ix->d_counter;
     pl->a.err = ix->d_error;
     pl->num_sms = ix->num_sms;
+    pl->smem_optin = ix->smem_optin;
     pl->storage = ix->storage;
     *plan = pl;
     return ANN_OK;

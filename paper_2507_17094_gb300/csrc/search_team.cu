@@ -653,7 +653,7 @@ bool try_teams(const TeamSearch &t, uint32_t least_rows, cudaStream_t stream, cu
         const TeamArgs g = plan(t, std::min(rows, round_up(t.cap_cand, 4)), NT / 2);
         if (g.lay.total > t.smem_optin) continue;
         int nb = 0;
-        *e = cudaFuncSetAttribute(team_kernel<ST, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g.lay.total);
+        *e = raise_shared_limit(team_kernel<ST, NT>, t.smem_optin);
         if (*e == cudaSuccess)
             *e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, team_kernel<ST, NT>, NT, g.lay.total);
         if (*e != cudaSuccess) return true;
