@@ -69,11 +69,12 @@ ann_status cuda_fail(cudaError_t e, const char *what);
 
 inline uint32_t round_up(uint32_t x, uint32_t m) { return (x + m - 1) / m * m; }
 
-// Raise a kernel's limit of dynamic shared memory to `bytes`, always the same
-// ones for a kernel: what a block of the device may have (`smem_optin`), or the
-// most that the kernel ever takes. The limit belongs to the kernel: one set to
-// what this launch needs could be lowered by another host thread before the
-// launch, which would then be refused.
+// Raise a kernel's limit of dynamic shared memory on the current device to
+// `bytes`, always the same ones for a kernel: what a block of the device may have
+// (`smem_optin`), or the most that the kernel ever takes. The limit belongs to
+// the kernel: one set to what this launch needs could be lowered by another host
+// thread before the launch, which would then be refused. It belongs to the
+// device, too, so it is not remembered as done for the process.
 template <typename Kernel>
 inline cudaError_t raise_shared_limit(Kernel *kernel, size_t bytes)
 {

@@ -19,7 +19,6 @@
 #include <cuda_bf16.h>
 
 #include <algorithm>
-#include <atomic>
 #include <cmath>
 #include <cstdio>
 #include <cstdlib>
@@ -1194,30 +1193,23 @@ ann_status gemm(const __nv_bfloat16 *A, const __nv_bfloat16 *B, uint32_t M, uint
         s = BMN ? make_map(&tb, B, K, N, 64) : make_map(&tb, B, N, K, mode == 2 ? BN / 2 : narrow ? 64 : 128);
     if (s != ANN_OK) return s;
     const uint32_t grid = gemm_grid(M, N, (uint32_t)sms - spare, mode);
-    static std::atomic<bool> attr[4];
-    const auto prepare = [&](const void *kernel, int smem, int which) {
-        if (attr[which].load(std::memory_order_relaxed)) return cudaSuccess;
-        const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        if (e == cudaSuccess) attr[which].store(true, std::memory_order_relaxed);
-        return e;
-    };
     if (narrow) {
         if constexpr (EPI != EPI_TOPP) {
             constexpr int smem = ring_smem(EPI, 64);
-            ANN_CUDA(prepare((const void *)gemm_kernel<EPI, 0, AMN, BMN, 64>, smem, 3));
+            ANN_CUDA(raise_shared_limit(gemm_kernel<EPI, 0, AMN, BMN, 64>, smem));
             const uint32_t tiles = (N + 63) / 64 * ((M + BM - 1) / BM);
             gemm_kernel<EPI, 0, AMN, BMN, 64><<<std::min(tiles, (uint32_t)sms - spare), GEMM_THREADS, smem, st>>>(ta, tb, M, N, K, e);
         }
     } else if (mode == 0) {
         constexpr int smem = ring_smem(EPI, BN);
-        ANN_CUDA(prepare((const void *)gemm_kernel<EPI, 0, AMN, BMN>, smem, 0));
+        ANN_CUDA(raise_shared_limit(gemm_kernel<EPI, 0, AMN, BMN>, smem));
         gemm_kernel<EPI, 0, AMN, BMN><<<grid, GEMM_THREADS, smem, st>>>(ta, tb, M, N, K, e);
     } else if constexpr (EPI == EPI_TOPP) {
         if (mode == 1) {
-            ANN_CUDA(prepare((const void *)gemm_kernel<EPI, 1>, RES_SMEM, 1));
+            ANN_CUDA(raise_shared_limit(gemm_kernel<EPI, 1>, RES_SMEM));
             gemm_kernel<EPI, 1><<<grid, GEMM_THREADS, RES_SMEM, st>>>(ta, tb, M, N, K, e);
         } else {
-            ANN_CUDA(prepare((const void *)gemm_kernel<EPI, 2>, RES_SMEM, 2));
+            ANN_CUDA(raise_shared_limit(gemm_kernel<EPI, 2>, RES_SMEM));
             cudaLaunchConfig_t cfg{};
             cfg.gridDim = dim3(grid);
             cfg.blockDim = dim3(GEMM_THREADS);

@@ -87,3 +87,17 @@ def test_one_calls_limit_leaves_the_others_launch_possible(L, make, large, small
         at.value = None
     assert statuses and not any(statuses), L.ann_last_error()
     assert status == 0, L.ann_last_error()
+
+
+@pytest.mark.parametrize("rows", [8, 64])
+def test_a_network_on_a_second_device(L, rows):
+    """The limit belongs to the device, too: networks on two devices of one
+    process, forward, training and prediction, the second after the first."""
+    for device in (0, 1, 0):
+        h, x = network(L, 2000, device), f32(64, 16)
+        logits, y = f32(64, 2000), np.zeros(64, np.uint32)
+        seeds, pmax = np.zeros((64, 8), np.uint32), f32(64)
+        assert L.ann_mlp_forward(h, x.ctypes.data, rows, logits.ctypes.data, None) == 0, L.ann_last_error()
+        assert L.ann_mlp_train_step(h, x.ctypes.data, y.ctypes.data, rows, 1e-3, 0.9, 0.999, 1e-8, 0.0, None, None) == 0
+        assert L.ann_mlp_predict(h, x.ctypes.data, rows, 8, 0.0, seeds.ctypes.data, pmax.ctypes.data, None) == 0
+        assert L.ann_mlp_free(h) == 0
