@@ -68,41 +68,6 @@ struct EpiArgs {
     int *err;
 };
 
-// Cluster helpers (the multicast logits kernel runs in clusters of two CTAs).
-__device__ __forceinline__ uint32_t cluster_rank()
-{
-    uint32_t r;
-    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-    return r;
-}
-
-__device__ __forceinline__ void cluster_sync_all()
-{
-    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-
-// A 2-D TMA load whose data, and the completion of its bytes, land at the
-// same shared-memory offsets in every CTA of `mask` within the cluster.
-__device__ __forceinline__ void tma_load_2d_mc(void *dst, const CUtensorMap *map, int x, int y, uint64_t *bar,
-                                               uint16_t mask)
-{
-    asm volatile(
-        "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes.multicast::cluster [%0], [%1, "
-        "{%2, %3}], [%4], %5;" ::"r"(smem_addr(dst)),
-        "l"(map), "r"(x), "r"(y), "r"(smem_addr(bar)), "h"(mask)
-        : "memory");
-}
-
-// tcgen05.commit arriving on the barrier at the same offset in every CTA of `mask`.
-__device__ __forceinline__ void mma_commit_mc(uint64_t *bar, uint16_t mask)
-{
-    asm volatile(
-        "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(
-            smem_addr(bar)),
-        "h"(mask)
-        : "memory");
-}
-
 // 2^x by the hardware approximation (MUFU): the softmax sum only decides the
 // confidence fallback, relative error ~2^-22 is ample.
 __device__ __forceinline__ float ex2_approx(float x)
@@ -401,19 +366,15 @@ __device__ __forceinline__ void topp_flush(const EpiArgs &e, const TopP &tp, uin
     o[2 * TOPP + 1] = tp.sm;
 }
 
-// MODE 0: the ring of (A, B) tiles; 1: resident A; 2: resident A, and the
-// CTAs run in clusters of two on the two row blocks of a pair, loading half
-// of each B tile each and multicasting it to both (B is read from L2 once
-// per pair instead of once per CTA). AMN / BMN (MODE 0): A is given as K x M, B
-// as K x N, row-major (MN-major operands), so that a product with a transposed
-// matrix reads the matrix itself.
-template <int EPI, int MODE = 0, bool AMN = false, bool BMN = false, int NT = BN>
+// RESA: A is resident, else a ring of (A, B) tiles. AMN / BMN (the ring): A is
+// given as K x M, B as K x N, row-major (MN-major operands), so that a product
+// with a transposed matrix reads the matrix itself.
+template <int EPI, bool RESA = false, bool AMN = false, bool BMN = false, int NT = BN>
 __global__ void __launch_bounds__(GEMM_THREADS, 1)
     gemm_kernel(const __grid_constant__ CUtensorMap tA, const __grid_constant__ CUtensorMap tB, uint32_t M,
                 uint32_t N, uint32_t K, EpiArgs e)
 {
-    constexpr bool RESA = MODE >= 1, MC = MODE == 2;
-    static_assert(NT == BN || (NT == 64 && MODE == 0 && EPI != EPI_TOPP), "narrow tiles: plain ring only");
+    static_assert(NT == BN || (NT == 64 && !RESA && EPI != EPI_TOPP), "narrow tiles: plain ring only");
     constexpr uint32_t TILE_N = NT * BK * 2;   // bytes of a B tile
     extern __shared__ uint8_t smem_raw[];
     const uint32_t pad = (1024u - (smem_addr(smem_raw) & 1023u)) & 1023u;
@@ -435,20 +396,16 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
     const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t nkb = (K + BK - 1) / BK;
     const uint32_t n_tiles = (N + NT - 1) / NT, m_tiles = (M + BM - 1) / BM;
-    // work units: tiles, or with clusters (row-block pair, column tile);
-    // unit t covers row block rb(t) = row unit (t / n_tiles), or with
-    // clusters row block 2 (t / n_tiles) + the CTA's rank in its pair
-    const uint32_t crank = MC ? cluster_rank() : 0u;
-    const uint32_t units = MC ? gridDim.x / 2 : gridDim.x, me = MC ? blockIdx.x / 2 : blockIdx.x;
-    const uint32_t tiles = n_tiles * (MC ? (m_tiles + 1) / 2 : m_tiles);
-    const uint32_t per = (tiles + units - 1) / units;
+    // unit t is column tile t % n_tiles of row block t / n_tiles; a CTA walks
+    // a contiguous range of them
+    const uint32_t tiles = n_tiles * m_tiles, me = blockIdx.x;
+    const uint32_t per = (tiles + gridDim.x - 1) / gridDim.x;
     const uint32_t t_begin = min(tiles, me * per), t_end = min(tiles, t_begin + per);
-    auto rb_of_unit = [&](uint32_t u) { return MC ? 2 * u + crank : u; };
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < NST; ++s) {
             mbar_init(&full[s], 1);
-            mbar_init(&empty[s], MC ? 2 : 1);   // with clusters, both CTAs' MMAs free a stage
+            mbar_init(&empty[s], 1);
         }
         for (int b = 0; b < 2; ++b) {
             mbar_init(&acc_full[b], 1);
@@ -458,8 +415,6 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
         mbar_init(a_empty, 1);
         fence_mbar_init();
     }
-    // both CTAs' barriers exist before either multicasts into the other
-    if (MC) cluster_sync_all();
     if (warp == 1) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_addr(tmem_slot)),
                      "r"((uint32_t)(2 * NT))
@@ -483,7 +438,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
                     if (loads > 0 && !(ok = mbar_wait_bounded(a_empty, (loads - 1) & 1, e.err))) break;
                     mbar_arrive_expect_tx(a_full, nkb * TILE_A);
                     for (uint32_t kb = 0; kb < nkb; ++kb)
-                        tma_load_2d(sA + kb * TILE_A, &tA, (int)(kb * BK), (int)(rb_of_unit(u) * BM), a_full);
+                        tma_load_2d(sA + kb * TILE_A, &tA, (int)(kb * BK), (int)(u * BM), a_full);
                     cur_u = u;
                     ++loads;
                 }
@@ -491,11 +446,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
                     const uint32_t s = it % NST, ph = (it / NST) & 1;
                     if (!(ok = mbar_wait_bounded(&empty[s], ph ^ 1, e.err))) break;
                     mbar_arrive_expect_tx(&full[s], TILE_N);
-                    if (MC)   // this CTA's half of the B tile (64 rows), to both CTAs
-                        tma_load_2d_mc(sB + s * TILE_N + crank * (TILE_N / 2), &tB, (int)(kb * BK),
-                                       (int)(n0 + crank * (NT / 2)), &full[s], (uint16_t)3);
-                    else
-                        tma_load_2d(sB + s * TILE_N, &tB, (int)(kb * BK), (int)n0, &full[s]);
+                    tma_load_2d(sB + s * TILE_N, &tB, (int)(kb * BK), (int)n0, &full[s]);
                 }
             }
         }
@@ -557,8 +508,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
 #pragma unroll
                     for (uint32_t k = 1; k < BK / 16; ++k)
                         mma_f16kind_lo<true>(acc, aa + a_step * k, bb + b_step * k, idesc);
-                    if (MC) mma_commit_mc(&empty[s], (uint16_t)3);   // frees the stage in both CTAs
-                    else mma_commit(&empty[s]);
+                    mma_commit(&empty[s]);
                     if (kb + 1 == nkb) {
                         mma_commit(&acc_full[buf]);
                         // the last tile of this row block: A may be replaced
@@ -583,11 +533,11 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
             if (!ok) break;
             tc_fence_after();
             const uint32_t u = t / n_tiles, n0 = (t % n_tiles) * NT;
-            const uint32_t m = rb_of_unit(u) * BM + q * 32 + lane;
+            const uint32_t m = u * BM + q * 32 + lane;
             if (EPI == EPI_TOPP && u != cur_u) {
                 // a new row block: the previous one's partial is complete
                 if (cur_u != 0xFFFFFFFFu) {
-                    const uint32_t pm = rb_of_unit(cur_u) * BM + q * 32 + lane;
+                    const uint32_t pm = cur_u * BM + q * 32 + lane;
                     if (pm < M) topp_flush(e, tp, pm, (me - (cur_u * n_tiles) / per) * 2 + h);
                 }
                 tp.reset();
@@ -616,15 +566,12 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
             }
         }
         if (EPI == EPI_TOPP && cur_u != 0xFFFFFFFFu) {
-            const uint32_t pm = rb_of_unit(cur_u) * BM + q * 32 + lane;
+            const uint32_t pm = cur_u * BM + q * 32 + lane;
             if (pm < M) topp_flush(e, tp, pm, (me - (cur_u * n_tiles) / per) * 2 + h);
         }
     }
     tc_fence_before();
     __syncthreads();
-    // no CTA leaves while its pair may still multicast into it or arrive on
-    // its barriers
-    if (MC) cluster_sync_all();
     if (warp == 1) {
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"((uint32_t)(2 * NT))
                      : "memory");
@@ -1097,75 +1044,31 @@ ann_status make_map(CUtensorMap *map, const void *ptr, uint32_t rows, uint32_t K
 }
 
 // Which GEMM variant runs: the fused top-P logits with K <= RES_K keep A
-// resident (ANN_GEMM_RESIDENT_A=0 turns that off); ANN_GEMM_MULTICAST=1
-// runs them in clusters of two CTAs that share each B tile by multicast
-// (measured no faster: the L2 reads of B are not what bounds the kernel);
-// everything else streams both operands.
-int gemm_mode(int epi, uint32_t K)
+// resident (ANN_GEMM_RESIDENT_A=0 turns that off); everything else streams both
+// operands.
+bool resident_a(int epi, uint32_t K)
 {
     static const bool res_on = env_flag("ANN_GEMM_RESIDENT_A", true);
-    static const bool mc_on = env_flag("ANN_GEMM_MULTICAST", false);
-    if (epi != EPI_TOPP || K > (uint32_t)RES_K || !res_on) return 0;
-    return mc_on ? 2 : 1;
+    return epi == EPI_TOPP && K <= (uint32_t)RES_K && res_on;
 }
 
-// Work units of a launch (tiles, or with clusters row-block pairs x column
-// tiles) and the persistent grid: one CTA per SM (pairs of CTAs with
-// clusters), fewer if there is less work.
-uint32_t gemm_units(uint32_t M, uint32_t N, int mode)
-{
-    const uint32_t n_tiles = (N + BN - 1) / BN, m_tiles = (M + BM - 1) / BM;
-    return n_tiles * (mode == 2 ? (m_tiles + 1) / 2 : m_tiles);
-}
+// Tiles of a launch and the persistent grid: one CTA per SM, fewer if there
+// are fewer tiles.
+uint32_t gemm_tiles(uint32_t M, uint32_t N) { return (N + BN - 1) / BN * ((M + BM - 1) / BM); }
 
-// Clusters of two that can be resident at once (SMs pair up within a GPC,
-// so this can be below half the SM count); queried once.
-uint32_t pair_slots(uint32_t sms);
-
-uint32_t gemm_grid(uint32_t M, uint32_t N, uint32_t sms, int mode = 0)
-{
-    const uint32_t units = gemm_units(M, N, mode);
-    return mode == 2 ? 2 * std::max(1u, std::min(units, pair_slots(sms))) : std::max(1u, std::min(units, sms));
-}
+uint32_t gemm_grid(uint32_t M, uint32_t N, uint32_t sms) { return std::max(1u, std::min(gemm_tiles(M, N), sms)); }
 
 // Top-P partial slots per row: two column halves times the largest number
-// of CTAs (pairs, with clusters) whose contiguous unit ranges meet one row
-// unit.
-uint32_t topp_slots(uint32_t M, uint32_t N, uint32_t sms, int mode)
+// of CTAs whose contiguous tile ranges meet one row block.
+uint32_t topp_slots(uint32_t M, uint32_t N, uint32_t sms)
 {
     const uint32_t n_tiles = (N + BN - 1) / BN;
-    const uint32_t units = gemm_units(M, N, mode), row_units = units / n_tiles;
-    const uint32_t ctas = mode == 2 ? gemm_grid(M, N, sms, mode) / 2 : gemm_grid(M, N, sms, mode);
-    const uint32_t per = (units + ctas - 1) / ctas;
+    const uint32_t tiles = gemm_tiles(M, N), ctas = gemm_grid(M, N, sms);
+    const uint32_t per = (tiles + ctas - 1) / ctas;
     uint32_t smax = 1;
-    for (uint32_t u = 0; u < row_units; ++u)
+    for (uint32_t u = 0; u < tiles / n_tiles; ++u)
         smax = std::max(smax, ((u + 1) * n_tiles - 1) / per - (u * n_tiles) / per + 1);
     return 2 * smax;
-}
-
-uint32_t pair_slots(uint32_t sms)
-{
-    static uint32_t cached = 0;
-    if (!cached) {
-        cudaFuncSetAttribute(gemm_kernel<EPI_TOPP, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, RES_SMEM);
-        cudaLaunchConfig_t cfg{};
-        cfg.gridDim = dim3(sms);
-        cfg.blockDim = dim3(GEMM_THREADS);
-        cfg.dynamicSmemBytes = RES_SMEM;
-        cudaLaunchAttribute at[1];
-        at[0].id = cudaLaunchAttributeClusterDimension;
-        at[0].val.clusterDim.x = 2;
-        at[0].val.clusterDim.y = 1;
-        at[0].val.clusterDim.z = 1;
-        cfg.attrs = at;
-        cfg.numAttrs = 1;
-        int n = 0;
-        if (cudaOccupancyMaxActiveClusters(&n, gemm_kernel<EPI_TOPP, 2>, &cfg) != cudaSuccess || n <= 0)
-            n = (int)(sms / 2);
-        cudaGetLastError();
-        cached = (uint32_t)std::min<int>(n, (int)(sms / 2));
-    }
-    return cached;
 }
 
 // C = A * B^T; AMN / BMN: A is given as K x M, B as K x N. `spare` SMs are left
@@ -1179,7 +1082,6 @@ ann_status gemm(const __nv_bfloat16 *A, const __nv_bfloat16 *B, uint32_t M, uint
         set_error("gemm: K = %u must be a multiple of 8", K);
         return ANN_EINVAL;
     }
-    const int mode = gemm_mode(EPI, K);
     CUtensorMap ta, tb;
     ann_status s = AMN ? make_map(&ta, A, K, M, 64) : make_map(&ta, A, M, K);
     // Tiles of 64 columns where tiles of 128 would leave more than half of the
@@ -1188,42 +1090,27 @@ ann_status gemm(const __nv_bfloat16 *A, const __nv_bfloat16 *B, uint32_t M, uint
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const bool narrow = EPI != EPI_TOPP && 2 * gemm_units(M, N, 0) <= (uint32_t)sms;
+    const bool narrow = EPI != EPI_TOPP && 2 * gemm_tiles(M, N) <= (uint32_t)sms;
     if (s == ANN_OK)
-        s = BMN ? make_map(&tb, B, K, N, 64) : make_map(&tb, B, N, K, mode == 2 ? BN / 2 : narrow ? 64 : 128);
+        s = BMN ? make_map(&tb, B, K, N, 64) : make_map(&tb, B, N, K, narrow ? 64 : 128);
     if (s != ANN_OK) return s;
-    const uint32_t grid = gemm_grid(M, N, (uint32_t)sms - spare, mode);
+    const uint32_t grid = gemm_grid(M, N, (uint32_t)sms - spare);
     if (narrow) {
         if constexpr (EPI != EPI_TOPP) {
             constexpr int smem = ring_smem(EPI, 64);
-            ANN_CUDA(raise_shared_limit(gemm_kernel<EPI, 0, AMN, BMN, 64>, smem));
+            ANN_CUDA(raise_shared_limit(gemm_kernel<EPI, false, AMN, BMN, 64>, smem));
             const uint32_t tiles = (N + 63) / 64 * ((M + BM - 1) / BM);
-            gemm_kernel<EPI, 0, AMN, BMN, 64><<<std::min(tiles, (uint32_t)sms - spare), GEMM_THREADS, smem, st>>>(ta, tb, M, N, K, e);
+            gemm_kernel<EPI, false, AMN, BMN, 64><<<std::min(tiles, (uint32_t)sms - spare), GEMM_THREADS, smem, st>>>(ta, tb, M, N, K, e);
         }
-    } else if (mode == 0) {
+    } else if (resident_a(EPI, K)) {
+        if constexpr (EPI == EPI_TOPP) {
+            ANN_CUDA(raise_shared_limit(gemm_kernel<EPI, true>, RES_SMEM));
+            gemm_kernel<EPI, true><<<grid, GEMM_THREADS, RES_SMEM, st>>>(ta, tb, M, N, K, e);
+        }
+    } else {
         constexpr int smem = ring_smem(EPI, BN);
-        ANN_CUDA(raise_shared_limit(gemm_kernel<EPI, 0, AMN, BMN>, smem));
-        gemm_kernel<EPI, 0, AMN, BMN><<<grid, GEMM_THREADS, smem, st>>>(ta, tb, M, N, K, e);
-    } else if constexpr (EPI == EPI_TOPP) {
-        if (mode == 1) {
-            ANN_CUDA(raise_shared_limit(gemm_kernel<EPI, 1>, RES_SMEM));
-            gemm_kernel<EPI, 1><<<grid, GEMM_THREADS, RES_SMEM, st>>>(ta, tb, M, N, K, e);
-        } else {
-            ANN_CUDA(raise_shared_limit(gemm_kernel<EPI, 2>, RES_SMEM));
-            cudaLaunchConfig_t cfg{};
-            cfg.gridDim = dim3(grid);
-            cfg.blockDim = dim3(GEMM_THREADS);
-            cfg.dynamicSmemBytes = RES_SMEM;
-            cfg.stream = st;
-            cudaLaunchAttribute at[1];
-            at[0].id = cudaLaunchAttributeClusterDimension;
-            at[0].val.clusterDim.x = 2;
-            at[0].val.clusterDim.y = 1;
-            at[0].val.clusterDim.z = 1;
-            cfg.attrs = at;
-            cfg.numAttrs = 1;
-            ANN_CUDA(cudaLaunchKernelEx(&cfg, gemm_kernel<EPI, 2>, ta, tb, M, N, K, e));
-        }
+        ANN_CUDA(raise_shared_limit(gemm_kernel<EPI, false, AMN, BMN>, smem));
+        gemm_kernel<EPI, false, AMN, BMN><<<grid, GEMM_THREADS, smem, st>>>(ta, tb, M, N, K, e);
     }
     ANN_CUDA(cudaGetLastError());
     return ANN_OK;
@@ -1680,7 +1567,7 @@ ann_status ann_mlp_predict(ann_mlp *m, const float *x, uint32_t n, uint32_t P, f
     ann_status s = ANN_OK;
     for (uint32_t r0 = 0; r0 < n && s == ANN_OK; r0 += m->maxb) {
         const uint32_t rows = std::min(m->maxb, n - r0);
-        const uint32_t ntiles = topp_slots(rows, m->out, (uint32_t)m->num_sms, gemm_mode(EPI_TOPP, m->h2));
+        const uint32_t ntiles = topp_slots(rows, m->out, (uint32_t)m->num_sms);
         const size_t need = (size_t)rows * ntiles * (2 * TOPP + 2) * 4;
         if (need > m->part_cap) {
             if (m->part) cudaFree(m->part);
