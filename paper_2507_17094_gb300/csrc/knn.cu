@@ -443,6 +443,8 @@ __global__ void __launch_bounds__(kFilterThreads, 1)
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
     int *err = &w.st->err;
+    bool ok = true;                         // false: a wait of this thread ran out
+    uint32_t it = 0, tc = 0, issued = 0;    // stages and lower[] slots it has loaded, stages it issued MMAs on
 
     if (warp == 0) {
         if (lane == 0) {
@@ -451,8 +453,7 @@ __global__ void __launch_bounds__(kFilterThreads, 1)
                 for (uint32_t kb = 0; kb < nkb; ++kb)
                     tma_load_2d(sA + (sub * nkb + kb) * kTileBytes, &map, (int)(kb * kBK),
                                 (int)(arow + sub * kTileRows), a_full);
-            uint32_t it = 0, tc = 0, s = 0, ph = 0;
-            bool ok = true;
+            uint32_t s = 0, ph = 0;
             for (uint32_t t = b0; t < b1 && ok; ++t, ++tc) {
                 const uint32_t ls = tc & low_mask;
                 if (!(ok = mbar_wait_bounded(&low_empty[ls], ((tc >> low_shift) & 1) ^ 1, err))) break;
@@ -465,16 +466,8 @@ __global__ void __launch_bounds__(kFilterThreads, 1)
                     ++it;
                     if (++s == w.stages) { s = 0; ph ^= 1; }
                 }
-                if (!ok) ++tc;
             }
-            // the loads in flight land before the CTA ends, whatever the others do
-            if (!ok) {
-                for (uint32_t i = it > w.stages ? it - w.stages : 0; i < it; ++i)
-                    mbar_wait_bounded(&full[i % w.stages], (i / w.stages) & 1, err);
-                for (uint32_t i = tc > w.low_slots ? tc - w.low_slots : 0; i < tc; ++i)
-                    mbar_wait_bounded(&low_full[i & low_mask], (i >> low_shift) & 1, err);
-            }
-            if (b0 == b1 || !ok) mbar_wait_bounded(a_full, 0, err);
+            if (b0 == b1) ok = mbar_wait_bounded(a_full, 0, err);
         }
     } else if (warp == 1) {
         constexpr uint32_t idesc = idesc_fp16(kTileRows, kTileRows);
@@ -482,13 +475,16 @@ __global__ void __launch_bounds__(kFilterThreads, 1)
         auto wait = [&](uint64_t *bar, uint32_t parity) {
             return __all_sync(0xffffffffu, mbar_wait_bounded(bar, parity, err));
         };
-        uint32_t tc = 0, s = 0, ph = 0;
-        bool ok = b0 == b1 || wait(a_full, 0);
+        uint32_t s = 0, ph = 0;
+        ok = b0 == b1 || wait(a_full, 0);
         for (uint32_t t = b0; t < b1 && ok; ++t, ++tc) {
             const uint32_t buf = tc & 1, use = tc >> 1;
             if (!(ok = wait(&acc_empty[buf], (use & 1) ^ 1))) break;
             for (uint32_t kb = 0; kb < nkb; ++kb) {
-                if (!(ok = wait(&full[s], ph))) break;
+                if (!(ok = wait(&full[s], ph))) {
+                    issued = kb;
+                    break;
+                }
                 tc_fence_after();
                 const uint32_t bb = b_lo + s * (kTileBytes >> 4);
                 if (elect_one()) {
@@ -508,7 +504,9 @@ __global__ void __launch_bounds__(kFilterThreads, 1)
                 __syncwarp();
                 if (++s == w.stages) { s = 0; ph ^= 1; }
             }
+            if (!ok) break;
         }
+        issued += tc * nkb;
     } else {
         // warp's rows: 32 (warp % 4) .. + 31 of each row tile; its part: one
         // half of the columns of every second tile. The two groups of eight
@@ -525,10 +523,10 @@ __global__ void __launch_bounds__(kFilterThreads, 1)
             list[sub] = next[sub] = w.kept + ((size_t)lr * lists + seg * kParts + h) * cap;
         }
         for (uint32_t t = b0 + buf; t < b1; t += 2) {
-            const uint32_t tc = t - b0, ls = tc & low_mask;
-            if (!__all_sync(0xffffffffu, mbar_wait_bounded(&low_full[ls], (tc >> low_shift) & 1, err) &&
-                                             mbar_wait_bounded(&acc_full[buf], (tc >> 1) & 1, err)))
-                break;
+            const uint32_t at = t - b0, ls = at & low_mask;
+            ok = __all_sync(0xffffffffu, mbar_wait_bounded(&low_full[ls], (at >> low_shift) & 1, err) &&
+                                             mbar_wait_bounded(&acc_full[buf], (at >> 1) & 1, err));
+            if (!ok) break;
             tc_fence_after();
             // a list without room for the whole part is marked overfull
 #pragma unroll
@@ -603,7 +601,17 @@ __global__ void __launch_bounds__(kFilterThreads, 1)
         }
     }
     tc_fence_before();
-    __syncthreads();
+    if (__syncthreads_or(!ok)) {
+        // a role gave up: what the others have in flight ends before the CTA does
+        auto wait = [&](uint64_t *bar, uint32_t parity) { mbar_wait_bounded(bar, parity, err); };
+        if (warp == 0) {
+            wait_last_uses(it, w.stages, [&](uint32_t i, uint32_t parity) { wait(&full[i], parity); });
+            wait_last_uses(tc, w.low_slots, [&](uint32_t i, uint32_t parity) { wait(&low_full[i], parity); });
+            wait(a_full, 0);
+        }
+        if (warp == 1) wait_last_use(issued, w.stages, [&](uint32_t i, uint32_t parity) { wait(&empty[i], parity); });
+        __syncthreads();
+    }
     if (warp == 1)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kCols) : "memory");
 }

@@ -425,13 +425,14 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
+    bool ok = true;                          // false: a wait of this thread ran out
+    uint32_t it = 0, loads = 0, issued = 0;  // stages and row blocks this thread has loaded, stages it issued MMAs on
 
     if (warp == 0 && RESA) {
         if (lane == 0) {
             // A once per row block (after the MMAs on the previous one are
             // done), then the B tiles of each of the block's column tiles
-            uint32_t it = 0, loads = 0, cur_u = 0xFFFFFFFFu;
-            bool ok = true;
+            uint32_t cur_u = 0xFFFFFFFFu;
             for (uint32_t t = t_begin; t < t_end && ok; ++t) {
                 const uint32_t u = t / n_tiles, n0 = (t % n_tiles) * NT;
                 if (u != cur_u) {
@@ -452,11 +453,13 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
         }
     } else if (warp == 0) {
         uint32_t s = 0, ph = 0;
-        bool ok = true;
         for (uint32_t t = t_begin; t < t_end && ok; ++t) {
             const uint32_t m0 = (t / n_tiles) * BM, n0 = (t % n_tiles) * NT;
             for (uint32_t kb = 0; kb < nkb; ++kb) {
-                if (!(ok = __all_sync(0xffffffffu, mbar_wait_bounded(&empty[s], ph ^ 1, e.err)))) break;
+                if (!(ok = __all_sync(0xffffffffu, mbar_wait_bounded(&empty[s], ph ^ 1, e.err)))) {
+                    it = kb;
+                    break;
+                }
                 if (elect_one()) {
                     uint8_t *a = sA + s * TILE_A, *b = sB + s * TILE_N;
                     mbar_arrive_expect_tx(&full[s], TILE_A + TILE_N);
@@ -476,7 +479,12 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
                 __syncwarp();
                 if (++s == NST) { s = 0; ph ^= 1; }
             }
+            if (!ok) {
+                it += (t - t_begin) * nkb;
+                break;
+            }
         }
+        if (ok) it = (t_end - t_begin) * nkb;
     } else if (warp == 1) {
         // all lanes run the loop, one issues (elect_one says why)
         constexpr uint32_t idesc = idesc_bf16(BM, NT) | (AMN ? kIdescAMN : 0u) | (BMN ? kIdescBMN : 0u);
@@ -486,20 +494,22 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
         auto wait = [&](uint64_t *bar, uint32_t parity) {
             return __all_sync(0xffffffffu, mbar_wait_bounded(bar, parity, e.err));
         };
-        uint32_t s = 0, ph = 0, tc = 0, loads = 0, cur_u = 0xFFFFFFFFu;
-        bool ok = true;
+        uint32_t s = 0, ph = 0, tc = 0, row_blocks = 0, cur_u = 0xFFFFFFFFu;
         for (uint32_t t = t_begin; t < t_end && ok; ++t, ++tc) {
             const uint32_t u = t / n_tiles;
             if (RESA && u != cur_u) {
-                if (!(ok = wait(a_full, loads & 1))) break;
+                if (!(ok = wait(a_full, row_blocks & 1))) break;
                 cur_u = u;
-                ++loads;
+                ++row_blocks;
             }
             const uint32_t buf = tc & 1, use = tc >> 1;
             if (!(ok = wait(&acc_empty[buf], (use & 1) ^ 1))) break;
             const uint32_t acc = tmem + buf * NT;
             for (uint32_t kb = 0; kb < nkb; ++kb) {
-                if (!(ok = wait(&full[s], ph))) break;
+                if (!(ok = wait(&full[s], ph))) {
+                    issued = kb;
+                    break;
+                }
                 tc_fence_after();
                 const uint32_t aa = a_lo + (RESA ? kb : s) * (TILE_A >> 4), bb = b_lo + s * (TILE_N >> 4);
                 if (elect_one()) {
@@ -519,7 +529,9 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
                 __syncwarp();
                 if (++s == NST) { s = 0; ph ^= 1; }
             }
+            if (!ok) break;
         }
+        issued += tc * nkb;
     } else {
         // epilogue warps 2..9: warp w reads accumulator lanes 32 * (w % 4) ..
         // + 31 (its quarter) and columns 64 * h .. + 63 of each tile
@@ -529,8 +541,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
         tp.reset();
         for (uint32_t t = t_begin; t < t_end; ++t, ++tc) {
             const uint32_t buf = tc & 1, use = tc >> 1;
-            const bool ok = __all_sync(0xffffffffu, mbar_wait_bounded(&acc_full[buf], use & 1, e.err));
-            if (!ok) break;
+            if (!(ok = __all_sync(0xffffffffu, mbar_wait_bounded(&acc_full[buf], use & 1, e.err)))) break;
             tc_fence_after();
             const uint32_t u = t / n_tiles, n0 = (t % n_tiles) * NT;
             const uint32_t m = u * BM + q * 32 + lane;
@@ -571,7 +582,14 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
         }
     }
     tc_fence_before();
-    __syncthreads();
+    if (__syncthreads_or(!ok)) {
+        // a role gave up: what the others have in flight ends before the CTA does
+        auto wait = [&](uint64_t *bar, uint32_t parity) { mbar_wait_bounded(bar, parity, e.err); };
+        if (warp == 0) wait_last_uses(it, NST, [&](uint32_t i, uint32_t parity) { wait(&full[i], parity); });
+        if (warp == 0) wait_last_use(loads, 1, [&](uint32_t, uint32_t parity) { wait(a_full, parity); });
+        if (warp == 1) wait_last_use(issued, NST, [&](uint32_t i, uint32_t parity) { wait(&empty[i], parity); });
+        __syncthreads();
+    }
     if (warp == 1) {
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"((uint32_t)(2 * NT))
                      : "memory");

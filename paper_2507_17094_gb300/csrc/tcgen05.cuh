@@ -8,6 +8,7 @@
 #include <atomic>
 
 #include "ann_internal.cuh"
+#include "ring_wait.cuh"
 
 // ------------------------------------------------------------------ PTX
 __device__ __forceinline__ void tma_load_2d(void *dst, const CUtensorMap *map, int x, int y, uint64_t *bar)
