@@ -18,6 +18,11 @@ buffers, so host<->device copies are inside its timed region.
 cores) on a bounded sample of the same workload and prints the same line.
 Under torchrun with N > 1 every rank searches its own replica and the value
 is the whole job's queries over the slowest rank's time.
+
+The last line of the output is the result, one JSON object of at most 2,500
+characters, so that it survives readers that keep only the end of the output.
+Every form's sweep, the per-phase profile, the serving run and the other
+workloads' legs are a line before it, "details " and a JSON object.
 """
 
 from __future__ import annotations
@@ -942,6 +947,23 @@ def run_leg_child(w: str, args, device: int, verbose: bool) -> dict:
     return json.loads(lines[-1])
 
 
+DETAIL_KEYS = ("forms", "serving", "phase_profile", "workloads")
+
+
+def result_lines(line: dict):
+    """The lines rank 0 prints: the details, then the result, which alone is a
+    JSON line: the record without them, and each form's itopk, recall and
+    rate."""
+    details = {k: line[k] for k in DETAIL_KEYS if k in line}
+    result = {k: v for k, v in line.items() if k not in details}
+    result["forms"] = {}
+    for name, f in details.get("forms", {}).items():
+        for s in f.get("sweep", ()):
+            if s["itopk"] == f["itopk"]:
+                result["forms"][name] = [s["itopk"], round(s["recall"], 3), round(s["qps"])]
+    return "details " + json.dumps(details), json.dumps(result)
+
+
 def run_leg(args):
     """Child side of run_leg_child: one leg on one GPU, its result as one
     JSON line on stdout."""
@@ -1279,7 +1301,7 @@ def run_ours(args):
     for ix_ in indexes.values():
         ix_.close()
     if rank == 0:
-        print(json.dumps(line), flush=True)
+        print("\n".join(result_lines(line)), flush=True)
     if dist is not None:
         dist.barrier()
         dist.destroy_process_group()

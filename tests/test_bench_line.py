@@ -1,0 +1,56 @@
+"""The benchmark's last line stays short enough for readers that keep only the
+last 3,000 characters of the output, however much its legs report."""
+import json
+
+
+def record():
+    sweep = [{"itopk": L, "recall": 0.9619999999999999, "ms": 1.000383973121643, "qps": 9996161.742571257}
+             for L in (16, 32, 64, 128, 256)]
+    forms = {name: {"storage": "f16", "entry": "learned", "dgs_discard": 0.75, "dgs_min_match": 0.0, "rerank": True,
+                    "itopk": 32, "sweep": sweep, "ms_per_launch": [1.000383973121643] * 9}
+             for name in ("paper_fp32", "fp16_rerank", "e4m3_rerank", "learned_fp16_rerank", "learned_e4m3_rerank",
+                          "random_fp32", "random_fp16_rerank", "ghost_nodgs_fp32", "simdgs_fp32")}
+    forms["_learned_entry"] = {1: {"epoch_loss": [3.14159265358979] * 8}}
+    x = 34528.26678105673
+    return {
+        "metric": "QPS at recall@10>=0.95 on 1 GB300: plain FP32 vs FP16/FP8+learned entry", "value": x * 300,
+        "unit": "queries/s", "n_gpus": 8, "steps": 20000, "warmup": 5000, "ms_per_step": x, "higher_is_better": True,
+        "scaling": "weak", "vs_baseline": None, "dtype": "f32",
+        "data": "synthetic (seeded Gaussian mixture; no dataset files)",
+        "config": {"workload": "scale-1M-96d", "n": 10 ** 9, "dim": 4096, "degree": 128, "nq": 10 ** 6,
+                   "form": "learned_e4m3_rerank", "k": 10, "itopk": 512, "search_width": 16, "max_iters": 10 ** 4,
+                   "entry": "learned", "ghost_n": 10 ** 6, "ghost_max_iters": 1000, "ghost_search_width": 16,
+                   "dgs_discard": 0.123456789012345, "dgs_cooldown": 0.30000000000000004, "storage": "e4m3",
+                   "recall_at_10": 0.9624999999999999, "recall_target": 0.95,
+                   "l2": "flushed between steps (256 MB write outside the timed events)", "parallelism": "replicas x8"},
+        "forms": forms,
+        "roofline": {"bound": "hbm", "achieved": x, "peak": x, "unit": "GB/s", "frac": 0.5339999999999999,
+                     "peak_source": "measured", "traffic": 1712549888, "algorithmic_bytes_per_launch": x * 1e5,
+                     "kernel": "search_kernel<E4M3>"},
+        "clocks": {"sm_mhz": 2070.0, "sm_max_mhz": 2070.0, "power_w_max": 1401.23,
+                   "reasons": ["hw_slowdown", "hw_thermal_slowdown", "sw_thermal_slowdown", "sw_power_cap"],
+                   "samples": 10000},
+        "e2e": {"value": x * 300, "unit": "queries/s", "h2d_bytes_per_step": 10 ** 10, "d2h_bytes_per_step": 10 ** 9,
+                "steps": 20000,
+                "api": "LearnedEntry.seeds + Index.search (ann_mlp_predict + ann_search), pinned host copies"},
+        "gpu_launches": 20000,
+        "cpu_baseline": {"value": x, "unit": "queries/s", "cores": 144, "kind": "oracle",
+                         "sample": "the first 10000 of the 1000000 queries x 50 passes, same search parameters (itopk "
+                                   "512), plain-C oracle on all host cores, 100.00 s wall", "ids_match_gpu": x},
+        "serving": {"rows": [x] * 500}, "phase_profile": {"share": {str(i): x for i in range(21)}},
+        "workloads": {str(w): {"rows": [x] * 1000} for w in range(6)}, "wall_s": x, "budget_s": 1020.0}
+
+
+def test_the_result_is_one_short_json_line():
+    import bench
+    rec = record()
+    details, result = bench.result_lines(rec)
+    assert "\n" not in details + result and not details.startswith("{")
+    assert len(result) <= 2500, len(result)
+    got = json.loads(result)
+    for k, v in rec.items():
+        if k not in bench.DETAIL_KEYS:
+            assert got[k] == v, k
+    assert got["forms"]["paper_fp32"] == [32, 0.962, 9996162] and len(got["forms"]) == 9
+    kept = json.loads(details[len("details "):])
+    assert kept["workloads"] == rec["workloads"] and set(kept) == set(bench.DETAIL_KEYS)
