@@ -23,19 +23,6 @@ __device__ __forceinline__ void tma_load_2d(void *dst, const CUtensorMap *map, i
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
-// Shared-memory matrix descriptor, K-major operand in the 128-byte swizzle
-// layout TMA writes: rows of 128 bytes, 8-row groups 1024 bytes apart.
-__device__ __forceinline__ uint64_t desc_sw128(uint32_t saddr)
-{
-    uint64_t d = 0;
-    d |= (uint64_t)((saddr & 0x3FFFFu) >> 4);        // start address
-    d |= (uint64_t)1 << 16;                           // leading byte offset (unused in this layout)
-    d |= (uint64_t)(1024 >> 4) << 32;                 // stride byte offset: next 8-row group
-    d |= (uint64_t)1 << 46;                           // descriptor version of this architecture
-    d |= (uint64_t)2 << 61;                           // swizzle: 128 bytes
-    return d;
-}
-
 // Instruction descriptor: BF16 x BF16 -> FP32, both K-major, M m, N n.
 __host__ __device__ constexpr uint32_t idesc_bf16(uint32_t m, uint32_t n)
 {
@@ -48,17 +35,9 @@ __host__ __device__ constexpr uint32_t idesc_fp16(uint32_t m, uint32_t n)
     return (1u << 4) | ((n >> 3) << 17) | ((m >> 4) << 24);
 }
 
-// One tcgen05.mma of kind::f16 (K 16; both operands FP16 or both BF16, as idesc says).
-__device__ __forceinline__ void mma_f16kind(uint32_t tmem_d, uint64_t da, uint64_t db, uint32_t idesc, uint32_t acc)
-{
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem_d),
-        "l"(da), "l"(db), "r"(idesc), "r"(acc)
-        : "memory");
-}
-
-// desc_sw128's high word (both majors: 1,024 bytes between 8-row groups)
+// High word of a shared-memory matrix descriptor in the 128-byte swizzle layout
+// TMA writes, both majors: 1,024 bytes between 8-row groups (the stride offset),
+// the descriptor version of this architecture, the swizzle.
 constexpr uint32_t kDescHi = (1024u >> 4) | (1u << 14) | (2u << 29);
 
 // MN-major operands (the K index is the row of a row-major matrix): TMA boxes of
@@ -84,12 +63,15 @@ __device__ __forceinline__ bool elect_one()
     return p != 0;
 }
 
-// The same with the descriptors' low words (desc_lo) and compile-time ACC:
-// one thread issues all MMAs of a CTA, so each instruction it spends on an
-// operand's descriptor delays the tensor cores. Stepping K by 16 elements adds
-// 2 to a low word, the next 128 x 64 tile adds 1024.
+// Low word of a K-major operand's descriptor (rows of 128 bytes): the start
+// address; the leading offset is unused in this layout. Stepping K by 16
+// elements adds 2, the next 128 x 64 tile adds 1024.
 __device__ __forceinline__ uint32_t desc_lo(uint32_t saddr) { return ((saddr & 0x3FFFFu) >> 4) | (1u << 16); }
 
+// One tcgen05.mma of kind::f16 (K 16; both operands FP16 or both BF16, as idesc
+// says) from the descriptors' low words and with compile-time ACC: one thread
+// issues all MMAs of a CTA, so each instruction it spends on an operand's
+// descriptor delays the tensor cores.
 template <bool ACC>
 __device__ __forceinline__ void mma_f16kind_lo(uint32_t tmem_d, uint32_t da, uint32_t db, uint32_t idesc)
 {
