@@ -159,9 +159,11 @@ ann_status ann_index_export(const ann_index *index, int which, void *host_dst, u
  *   stream       cudaStream_t (NULL = legacy default stream)
  * Asynchronous on `stream`; returns after the launch. The launch shape is
  * chosen per call from the parameters and nq (rows gathered per round: 16, or 8
- * or 4 where the resident warps that this admits take the batch in fewer fillings); the
- * environment variable ANN_STAGE_ROWS fixes the rows per round instead (for
- * experiments). Results do not depend on the shape. */
+ * or 4 where the resident warps that this admits take the batch in fewer fillings;
+ * a batch whose every query gets a thread block at once runs on a block per query
+ * instead of a warp); the environment variable ANN_STAGE_ROWS fixes the rows per
+ * round instead, on a warp per query whatever the batch (for experiments). Results
+ * and counters do not depend on the shape. */
 ann_status ann_search(ann_index *index, const float *queries, uint32_t nq, const ann_search_params *params,
                       const uint32_t *given_seeds, uint32_t n_given, uint32_t *ids, float *dists,
                       ann_query_stats *stats, void *stream);
@@ -194,13 +196,15 @@ ann_status ann_search_host_noalloc(ann_index *index, const float *queries, uint3
 /* Per-phase time of the search (the measurement of Section 5.5, Fig. 11:
  * SM clock readings around the parts of the kernel). The same search and
  * results as ann_search (ids, dists device nq x k; no stats), run by a build
- * of the kernel that reads the clock at every phase boundary and adds each
- * warp's elapsed cycles to cycles[stage * ANN_PROFILE_PHASES + phase] (host,
- * ANN_PROFILE_STAGES x ANN_PROFILE_PHASES uint64, summed over all warps;
- * zeroed first). Stages: 0 ghost stage, 1 base graph, 2 rerank and output.
- * Phases: 0 parent selection and the adjacency / direction / parent-row
- * fetch, 1 DGS selection, 2 visited-set test-and-insert (and seeding),
- * 3 waiting for gathered rows, 4 distances, 5 merge, 6 the rest (query load,
+ * of its kernel with a warp per query (whatever the batch: ann_search gives the
+ * queries of a small batch a block each) that reads the clock at every phase
+ * boundary and adds each warp's elapsed cycles to cycles[stage *
+ * ANN_PROFILE_PHASES + phase] (host, ANN_PROFILE_STAGES x ANN_PROFILE_PHASES
+ * uint64, summed over all warps; zeroed first). Stages: 0 ghost stage, 1 base
+ * graph, 2 rerank and output. Phases: 0 parent selection, 1 DGS selection with
+ * its loads of lists, direction words and parent rows (of several parents, also
+ * the visited test of all but the last), 2 visited-set test-and-insert (and
+ * seeding, and the lists' loads without DGS), 3 waiting for gathered rows, 4 distances, 5 merge, 6 the rest (query load,
  * set clears, stage switch, output). Cycles are per-warp wall time, so they
  * include time a warp waits while others issue. Allocates a temporary of
  * 192 bytes per warp slot; synchronous on `stream`. */
@@ -406,8 +410,8 @@ ann_status ann_mlp_load(const char *path, int device, uint32_t max_batch, ann_ml
  * Continuous-batching server (not in the paper). Requests (batches of any
  * size, each with its own ann_search_params up to the server's max_params)
  * are admitted while others run and share the GPU query by query: one ring
- * of query slots (page-locked host memory the device reads and writes), a FIFO
- * that the warps of every running search kernel take queries from, per-warp
+ * of query slots (page-locked host memory the device reads and writes: capacity
+ * x (4 dim + 8 k + 4) bytes, locked once at creation), a FIFO that the warps of every running search kernel take queries from, per-warp
  * queue and visited state resident in shared memory while a query runs.
  * Admission is by buffer memory: submit returns ANN_EBUSY when the ring or the
  * request records are full (poll, then retry).

@@ -2,9 +2,9 @@
 // staging (Section 3.2.2) and direction-guided selection (Section 3.3.2).
 //
 // Design (GB300-first, not the paper's 32-thread-block CAGRA kernel):
-//   - persistent CTAs of 4 warps; each warp owns one query at a time and pulls
-//     the next query index from a device counter, so long and short searches
-//     balance across the 152 SMs;
+//   - persistent CTAs of 4, 2 or 1 warps; each warp owns one query at a time
+//     and pulls the next query index from a device counter, so long and short
+//     searches balance across the 152 SMs;
 //   - per warp, a small shared-memory region (about 8 KB for itopk 32 on
 //     96-d FP32) holds the query, the priority queue, the candidate list and
 //     16 staged rows, so 24 warps share an SM and hide each other's memory
@@ -1032,9 +1032,11 @@ struct ServeCounts {
 // Continuous batching: warps of every running serve kernel take queries, in
 // arrival order, from one ring (monotonic query counters; slot = counter mod
 // capacity). A launch makes available the queries published before it and, with
-// `live`, those published until its warps start; each request brings a launch,
-// so all are taken, and a warp serves at most `per_warp` queries and then
-// leaves, so SMs free up for other kernels. Queries, records and results are
+// `live`, those published until its warps start; each request brings a launch
+// with room for all that were in flight, whose warps leave early only when
+// everything published has been taken, so all are taken (serve_take.cuh). A warp
+// serves at most `per_warp` queries and then leaves, so SMs free up for other
+// kernels. Queries, records and results are
 // host memory, read and written over the chip-to-chip link: a query's few
 // hundred bytes are small against the row bytes its search gathers, and no copy
 // is queued for them. The request's parameters are copied into the warp's shared
@@ -1435,8 +1437,8 @@ ann_status search_launch_ex(ann_index *ix, const float *queries, uint32_t nq, co
     // counter) are shared, so a launch on another stream waits for the last
     if (ix->busy_set && ix->busy_stream != stream) ANN_CUDA(cudaStreamWaitEvent(stream, ix->busy, 0));
     // a batch small enough that each query can have a block of its own goes to
-    // the teams (search_team.cu); the profile and a fixed ANN_STAGE_ROWS are
-    // the warp kernel's
+    // the teams (search_team.cu), which have neither the profile's clocks nor a
+    // fixed ANN_STAGE_ROWS: those are the warp kernel's
     if (!prof && env_int("ANN_STAGE_ROWS", 0) <= 0) {
         const TeamSearch t{a.view[1], a.view[0], a.ghost_ids, a.x32, a.row32_bytes, a.d, a.w, a.cap_buf, a.cap_cand,
                            a.gbm_words, q.n_keep < ix->degree || q.min_match > 0, q, queries, nq, given,

@@ -15,11 +15,13 @@
 // visible, so no copy, event or second stream is needed. Only the learned
 // entry's prediction needs the queries on the device: a copy and the prediction
 // on an ingest stream, which the launches then wait for. Kernels of successive
-// requests overlap and take queries from the same FIFO; each launch has a warp
-// for every query in flight, its own request's included, so every published
-// query is served. Measured: 200 requests of 1-64 queries at once 19.5 -> 4.5 ms
-// (2.7 of which the host spends submitting them), one request of 6,548 queries
-// 5.1 -> 2.1, of 608 3.5 -> 0.76.
+// requests overlap and take queries from the same FIFO; each launch has room for
+// every query in flight, its own request's included, and its warps leave early
+// only when all that is published has been taken (serve_take.cuh), so every
+// published query is served. A request counts as published once its launch was
+// accepted. Measured: 200 requests of 1-64 queries at once 19.5 -> 4.5 ms (2.7 of
+// which the host spends submitting them), one request of 6,548 queries 5.1 ->
+// 2.1, of 608 3.5 -> 0.76.
 //
 // poll(): a request is done when its flag is set (by the warp that finished its
 // last query, after a system-scope fence); its results are copied out of the
