@@ -958,9 +958,8 @@ def result_lines(line: dict):
     result = {k: v for k, v in line.items() if k not in details}
     result["forms"] = {}
     for name, f in details.get("forms", {}).items():
-        for s in f.get("sweep", ()):
-            if s["itopk"] == f["itopk"]:
-                result["forms"][name] = [s["itopk"], round(s["recall"], 3), round(s["qps"])]
+        if "qps" in f:
+            result["forms"][name] = [f["itopk"], round(f["recall"], 3), round(f["qps"])]
     return "details " + json.dumps(details), json.dumps(result)
 
 

@@ -4,10 +4,9 @@ import json
 
 
 def record():
-    sweep = [{"itopk": L, "recall": 0.9619999999999999, "ms": 1.000383973121643, "qps": 9996161.742571257}
-             for L in (16, 32, 64, 128, 256)]
     forms = {name: {"storage": "f16", "entry": "learned", "dgs_discard": 0.75, "dgs_min_match": 0.0, "rerank": True,
-                    "itopk": 32, "sweep": sweep, "ms_per_launch": [1.000383973121643] * 9}
+                    "itopk": 32, "qps": 9996161.742571257, "ms_per_step": 1.000383973121643,
+                    "recall": 0.9619999999999999, "gbs": 3565.2419644437787, "hash_resets": 0}
              for name in ("paper_fp32", "fp16_rerank", "e4m3_rerank", "learned_fp16_rerank", "learned_e4m3_rerank",
                           "random_fp32", "random_fp16_rerank", "ghost_nodgs_fp32", "simdgs_fp32")}
     forms["_learned_entry"] = {1: {"epoch_loss": [3.14159265358979] * 8}}
