@@ -272,7 +272,9 @@ ann_status ann_shards_search(ann_shards *shards, const float *queries, uint32_t 
  * and (96 rows x (dim + 1) + 32 K x 2) x 4 bytes of shared memory must fit a
  * block (ANN_EINVAL otherwise). Asynchronous on `stream`; from 1,024 nodes on
  * it takes a temporary in stream order (2 n dim bytes and at most about 20 KB
- * per row of a chunk of 39,000 rows) and does without if it cannot have it. */
+ * per row of a chunk of 39,000 rows) and does without if it cannot have it. Up
+ * to 64 MB of it stay reserved on the device for the next call, until an
+ * allocation of the library is refused. */
 ann_status ann_knn_exact(const float *X, uint64_t n, uint32_t dim, uint32_t K, uint32_t *ids, void *stream);
 /* Prune kNN lists (device, n x K; each row distinct ids, ANN_INVALID_ID
  * allowed, which is no edge and has no detours) to a fixed-degree graph (device,

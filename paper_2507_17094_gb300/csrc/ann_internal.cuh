@@ -81,6 +81,14 @@ inline cudaError_t raise_shared_limit(Kernel *kernel, size_t bytes)
     return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
 }
 
+// A temporary of `bytes` on the current device in the order of `st` (free it
+// with cudaFreeAsync), from a pool of the library's own that keeps up to
+// kTemporaryKeep freed bytes mapped. The default pool gives everything back at
+// each synchronisation, and mapping it again costs a call some 190 us. What is
+// kept goes back to the device when an allocation of the library is refused.
+constexpr uint64_t kTemporaryKeep = 64ull << 20;
+cudaError_t temporary_alloc(void **p, size_t bytes, cudaStream_t st);
+
 // Make `dev` current for an entry point, remembering the caller's device in
 // *prev (-1 if it could not be read). Returns ANN_EDEVICE, with the message
 // set, when the switch fails: the entry point must then return without

@@ -11,6 +11,7 @@
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
+#include <mutex>
 #include <vector>
 
 #include "ann_internal.cuh"
@@ -52,10 +53,55 @@ void set_error(const char *fmt, ...)
     va_end(ap);
 }
 
+// The pools of temporaries, by device, made on first use.
+constexpr int kMaxDevices = 64;
+static std::mutex g_temporary_mu;
+static cudaMemPool_t g_temporary[kMaxDevices] = {};
+
+// The current device's pool, NULL if it cannot be had.
+static cudaMemPool_t temporary_pool()
+{
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return nullptr;
+    std::lock_guard<std::mutex> lk(g_temporary_mu);
+    if (!g_temporary[dev]) {
+        // another stream of this thread may be under capture
+        cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+        cudaThreadExchangeStreamCaptureMode(&mode);
+        cudaMemPoolProps props{};
+        props.allocType = cudaMemAllocationTypePinned;
+        props.location.type = cudaMemLocationTypeDevice;
+        props.location.id = dev;
+        cudaMemPool_t pool = nullptr;
+        uint64_t keep = kTemporaryKeep;
+        cudaError_t e = cudaMemPoolCreate(&pool, &props);
+        if (e == cudaSuccess) e = cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
+        if (e == cudaSuccess) g_temporary[dev] = pool;
+        else cudaGetLastError();
+        cudaThreadExchangeStreamCaptureMode(&mode);
+    }
+    return g_temporary[dev];
+}
+
+cudaError_t temporary_alloc(void **p, size_t bytes, cudaStream_t st)
+{
+    // under capture the allocation becomes a node of the graph, with its memory
+    cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
+    const cudaError_t known = cudaStreamIsCapturing(st, &capturing);
+    if (known != cudaSuccess) cudaGetLastError();
+    const cudaMemPool_t pool =
+        known == cudaSuccess && capturing == cudaStreamCaptureStatusNone ? temporary_pool() : nullptr;
+    return pool ? cudaMallocFromPoolAsync(p, bytes, pool, st) : cudaMallocAsync(p, bytes, st);
+}
+
 ann_status cuda_fail(cudaError_t e, const char *what)
 {
     set_error("%s: %s", what, cudaGetErrorString(e));
-    return e == cudaErrorMemoryAllocation ? ANN_ENOMEM : ANN_ECUDA;
+    if (e != cudaErrorMemoryAllocation) return ANN_ECUDA;
+    std::lock_guard<std::mutex> lk(g_temporary_mu);
+    for (cudaMemPool_t pool : g_temporary)
+        if (pool) cudaMemPoolTrimTo(pool, 0);
+    return ANN_ENOMEM;
 }
 
 ann_status enter_device(int dev, int *prev, const char *who)

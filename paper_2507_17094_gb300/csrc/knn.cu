@@ -933,9 +933,10 @@ __global__ void __launch_bounds__(kRescoreWarps * 32)
 // ------------------------------------------------------------ host
 // Rows from which the filter runs. Measured plain / filtered, us a call: 1,024
 // rows 194 / 85 (32 dimensions, K 16), 357 / 96 (96, 32), 1,274 / 142 (64,
-// 256); 4,096 rows 425 / 129, 877 / 151, 2,301 / 300. Below this the filter
-// still is the faster one back to back, but mapping its workspace after a
-// synchronisation costs about what it saves.
+// 256); 4,096 rows 425 / 129, 877 / 151, 2,301 / 300. After a synchronisation,
+// with the workspace kept (temporary_alloc), 1,024 x 8, K 8: 134 / 86; 2,000 x 32,
+// K 16: 293 / 95; 10,000 x 96, K 32: 2,550 / 275 (280, 360 and 700 with a workspace
+// mapped anew).
 constexpr uint64_t kFilterMin = 1024;
 
 uint32_t gcd(uint32_t a, uint32_t b)
@@ -1021,7 +1022,7 @@ ann_status knn_filtered(const float *X, uint32_t n, uint32_t d, uint32_t K, uint
     const size_t o_kept = take(std::max(kept_bytes(chunk_rows), kept_bytes(last_rows)));
     const size_t o_nk = take((size_t)chunk_rows * kParts * kMaxS * 4);
     uint8_t *ws = nullptr;
-    if (cudaMallocAsync((void **)&ws, bytes, st) != cudaSuccess) {
+    if (temporary_alloc((void **)&ws, bytes, st) != cudaSuccess) {
         cudaGetLastError();
         set_error("ann_knn_exact: no room for a workspace of %zu bytes", bytes);
         return ANN_ENOMEM;

@@ -75,7 +75,10 @@ extern "C" {
 
 int fake_busy = 0;                       // cudaStreamQuery's answer
 int fake_fail_launches = 0;              // launches to refuse
-unsigned long long fake_launches = 0;
+unsigned long long fake_launches = 0, fake_pools = 0, fake_temporaries = 0, fake_trims = 0, fake_pool_keep = 0;
+int fake_no_temporaries = 0;             // refuse allocations from a pool
+int fake_no_memory = 0;                  // refuse cudaMalloc
+int fake_capturing = 0;                  // cudaStreamIsCapturing's answer
 void (*fake_after_limit)(void) = nullptr;   // called after each cudaFuncSetAttribute outside the hook itself
 
 void fake_run_serve()
@@ -199,10 +202,42 @@ cudaError_t cudaGetLastError() { return std::exchange(last, cudaSuccess); }
 const char *cudaGetErrorString(cudaError_t) { return "an error of the stand-in runtime"; }
 cudaError_t cudaMalloc(void **p, size_t n)
 {
-    *p = std::calloc(1, n + 256);
+    *p = fake_no_memory ? nullptr : std::calloc(1, n + 256);
     return *p ? cudaSuccess : result(cudaErrorMemoryAllocation);
 }
 cudaError_t cudaMallocAsync(void **p, size_t n, cudaStream_t) { return cudaMalloc(p, n); }
+struct CUmemPoolHandle_st {
+    int device;
+    unsigned long long keep;
+};
+cudaError_t cudaMemPoolCreate(cudaMemPool_t *pool, const cudaMemPoolProps *props)
+{
+    ++fake_pools;
+    *pool = new CUmemPoolHandle_st{props->location.id, 0};
+    return cudaSuccess;
+}
+cudaError_t cudaMemPoolSetAttribute(cudaMemPool_t pool, cudaMemPoolAttr a, void *value)
+{
+    if (a == cudaMemPoolAttrReleaseThreshold) pool->keep = fake_pool_keep = *(unsigned long long *)value;
+    return cudaSuccess;
+}
+cudaError_t cudaMallocFromPoolAsync(void **p, size_t n, cudaMemPool_t pool, cudaStream_t)
+{
+    if (fake_no_temporaries || pool->device != device) return result(cudaErrorMemoryAllocation);
+    ++fake_temporaries;
+    return cudaMalloc(p, n);
+}
+cudaError_t cudaMemPoolTrimTo(cudaMemPool_t, size_t)
+{
+    ++fake_trims;
+    return cudaSuccess;
+}
+cudaError_t cudaStreamIsCapturing(cudaStream_t, cudaStreamCaptureStatus *s)
+{
+    *s = fake_capturing ? cudaStreamCaptureStatusActive : cudaStreamCaptureStatusNone;
+    return cudaSuccess;
+}
+cudaError_t cudaThreadExchangeStreamCaptureMode(cudaStreamCaptureMode *) { return cudaSuccess; }
 cudaError_t cudaHostAlloc(void **p, size_t n, unsigned) { return cudaMalloc(p, n); }
 cudaError_t cudaHostGetDevicePointer(void **d, void *h, unsigned)
 {
