@@ -81,6 +81,8 @@ int fake_no_memory = 0;                  // refuse cudaMalloc
 int fake_capturing = 0;                  // cudaStreamIsCapturing's answer
 void (*fake_after_limit)(void) = nullptr;   // called after each cudaFuncSetAttribute outside the hook itself
 
+void fake_set_device(int d) { device = d; }
+
 void fake_run_serve()
 {
     for (const Serve &s : queued) {

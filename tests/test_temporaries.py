@@ -26,9 +26,9 @@ def test_one_bounded_pool_per_device_that_is_given_back(L):
     assert knn() == 0 and knn() == 0
     assert word("pools").value == 1 and word("temporaries").value == 2
     assert 0 < word("pool_keep").value <= 64 << 20
-    L.cudaSetDevice(1)
+    L.fake_set_device(1)
     assert knn() == 0 and word("pools").value == 2 and word("temporaries").value == 3
-    L.cudaSetDevice(0)
+    L.fake_set_device(0)
     word("no_temporaries", C.c_int).value = 1
     launches = word("launches").value
     assert knn() == 0 and word("launches").value == launches + 1   # the plain kernel alone
