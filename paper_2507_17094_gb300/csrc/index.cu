@@ -100,7 +100,7 @@ ann_status cuda_fail(cudaError_t e, const char *what)
     if (e != cudaErrorMemoryAllocation) return ANN_ECUDA;
     std::lock_guard<std::mutex> lk(g_temporary_mu);
     for (cudaMemPool_t pool : g_temporary)
-        if (pool) cudaMemPoolTrimTo(pool, 0);
+        if (pool && cudaMemPoolTrimTo(pool, 0) != cudaSuccess) cudaGetLastError();
     return ANN_ENOMEM;
 }
 
